@@ -133,9 +133,10 @@ bool range_ok(const hg_cache* c, int32_t begin, int32_t count) {
   return c && count >= 1 && begin >= 0 && (int64_t)begin + count <= c->d.L;
 }
 
-// Decode work plan.  Chunk sizes are chosen so that a launch has at most one
-// wave of work items (the CTAs that are resident at once: four per SM for up
-// to 8 queries per KV head, two above) of similar cost.  Chunk sizes are
+// Decode work plan.  Chunk sizes are chosen so that a launch has one wave of
+// work items (the CTAs that are resident at once: four per SM for up to 8
+// queries per KV head, two above) of similar cost, or, where that leaves them
+// uneven, two to three waves of smaller ones (plan_decode).  Chunk sizes are
 // multiples of 64 tokens and depend only on the layer range and the device,
 // so the workspace bound holds for every appended count.
 int sm_count() {
@@ -187,54 +188,6 @@ SegBytes seg_bytes(const Dims& d) {
   return b;
 }
 
-int max_items_of(const Dims& d, const DecodePlan& p);
-ChunkCounts counts_of(const Dims& d, int appended, const DecodePlan& p);
-
-DecodePlan plan_decode(const hg_cache* c, int begin, int count) {
-  const Dims& d = c->d;
-  const SegBytes sb = seg_bytes(d);
-  double total = 0.0;
-  for (int l = begin; l < begin + count; ++l) {
-    for (int h = 0; h < d.H; ++h) {
-      const int cls = head_class(d, c->layer_mask[l], h);
-      if (cls == kProtected) {
-        total += d.T * sb.bf16;
-      } else {
-        const int nc = ncoded(d);
-        total += (d.T - nc) * sb.bf16 + nc * (cls == kKeysOnly ? sb.coded_k : sb.coded_u);
-      }
-    }
-  }
-  total *= d.B;
-  const int wave = (d.G <= 8 ? 4 : 2) * sm_count();
-  double item = total / wave;
-  if (item < 16384.0) item = 16384.0;
-  // Grow the item size until the items (at the largest appended count) fit
-  // one wave, or every segment is a single chunk.
-  DecodePlan p;
-  for (int iter = 0; iter < 64; ++iter, item *= 1.05) {
-    p.cbU = chunk_tokens(d.T - ncoded(d) + d.S_new, sb.bf16, item, 64);
-    p.cqU = chunk_tokens(ncoded(d), sb.coded_u, item, 64);
-    p.cqK = chunk_tokens(ncoded(d), sb.coded_k, item, 64);
-    p.cbP = chunk_tokens(d.T + d.S_new, sb.bf16, item, 64);
-    long long items = 0;
-    for (int l = begin; l < begin + count; ++l)
-      items += (long long)d.B * row_chunks(d, c->layer_mask[l], counts_of(d, d.S_new, p));
-    if (items <= wave) break;
-    if (p.cbU >= d.T - ncoded(d) + d.S_new && p.cqU >= ncoded(d) && p.cqK >= ncoded(d) &&
-        p.cbP >= d.T + d.S_new)
-      break;
-  }
-  // The merging CTA stages every split's partial of a head in its stage buffer.
-  while (max_items_of(d, p) > decode_max_splits(d.G)) {
-    p.cbU *= 2;
-    p.cqU *= 2;
-    p.cqK *= 2;
-    p.cbP *= 2;
-  }
-  return p;
-}
-
 ChunkCounts counts_of(const Dims& d, int appended, const DecodePlan& p) {
   return chunk_counts(d, appended, p.cbU, p.cqU, p.cqK, p.cbP);
 }
@@ -247,9 +200,119 @@ int max_items_of(const Dims& d, const DecodePlan& p) {
   return m > prot ? m : prot;
 }
 
+// Unprotected and protected (layer, KV head) pairs of a layer range.
+struct HeadCounts {
+  int unprot, prot;
+};
+
+HeadCounts head_counts(const hg_cache* c, int begin, int count) {
+  HeadCounts n = {0, 0};
+  for (int l = begin; l < begin + count; ++l) n.prot += popc64(c->layer_mask[l]);
+  n.unprot = count * c->d.H - n.prot;
+  return n;
+}
+
+// Chunk sizes for items of about `item` byte-equivalents.
+DecodePlan plan_for(const Dims& d, const SegBytes& sb, double item) {
+  DecodePlan p;
+  p.cbU = chunk_tokens(d.T - ncoded(d) + d.S_new, sb.bf16, item, 64);
+  p.cqU = chunk_tokens(ncoded(d), sb.coded_u, item, 64);
+  p.cqK = chunk_tokens(ncoded(d), sb.coded_k, item, 64);
+  p.cbP = chunk_tokens(d.T + d.S_new, sb.bf16, item, 64);
+  return p;
+}
+
+// The merging CTA stages every split's partial of a head in its stage buffer.
+void limit_splits(const Dims& d, DecodePlan* p) {
+  while (max_items_of(d, *p) > decode_max_splits(d.G)) {
+    p->cbU *= 2;
+    p->cqU *= 2;
+    p->cqK *= 2;
+    p->cbP *= 2;
+  }
+}
+
+size_t plan_ws_bytes(const Dims& d, int count, const DecodePlan& p) {
+  return (size_t)ws_bytes(d, count, max_items_of(d, p));
+}
+
+// The work plan of a launch over layers [begin, +count): *one_wave has at most
+// one wave of items (its workspace is the least a launch accepts); the
+// returned plan is the one to run when its workspace is at hand.
+DecodePlan plan_decode(const hg_cache* c, int begin, int count, DecodePlan* one_wave) {
+  const Dims& d = c->d;
+  const SegBytes sb = seg_bytes(d);
+  const HeadCounts hc = head_counts(c, begin, count);
+  const double nc = ncoded(d);
+  const double head_u = (d.T - nc) * sb.bf16 + nc * sb.coded_u;
+  const double head_p = d.keys_only ? (d.T - nc) * sb.bf16 + nc * sb.coded_k : d.T * sb.bf16;
+  const double total = d.B * (hc.unprot * head_u + hc.prot * head_p);
+  const int wave = (d.G <= 8 ? 4 : 2) * sm_count();
+  const double mean = total / wave;
+  double item = std::max(mean, 16384.0);
+  // Grow the item size until the items (at the largest appended count) fit
+  // one wave, or every segment is a single chunk.
+  DecodePlan p;
+  for (int iter = 0; iter < 64; ++iter, item *= 1.05) {
+    p = plan_for(d, sb, item);
+    const ChunkCounts cc = counts_of(d, d.S_new, p);
+    int nb;
+    const long long items = (long long)d.B * ((long long)hc.unprot * head_chunks(kQuantized, cc, &nb) +
+                                              (long long)hc.prot * head_chunks(d.keys_only ? kKeysOnly : kProtected, cc, &nb));
+    if (items <= wave) break;
+    if (p.cbU >= d.T - ncoded(d) + d.S_new && p.cqU >= ncoded(d) && p.cqK >= ncoded(d) &&
+        p.cbP >= d.T + d.S_new)
+      break;
+  }
+  limit_splits(d, &p);
+  if (one_wave) *one_wave = p;
+  // One wave balances only when the heads cut into pieces of about the mean
+  // cost per resident CTA.  When whole segments are as large as that (a layer
+  // of a large batch: 256 heads over 608 CTAs), the rounding leaves chunks of
+  // up to twice the mean, and the launch lasts as long as they do.  Then
+  // pieces of half the mean run as two to three waves instead, costliest
+  // first: one layer of 32 rows, 8 KV heads and 8,576 tokens, 150 -> 90 us (96
+  // and 91 us at 2/3 and 1/3 of the mean); 3,520 tokens of 4-bit rotated keys,
+  // 84 -> 53 us (53, 58).  Chunks under 256 KB keep one wave: a
+  // CTA's start and merge (about 8 us) outweigh the balance there (28 layers
+  // of 4 heads: 15.3 us a step in one wave, 18.1 with pieces of 2/3).
+  double worst = 0;
+  if (hc.unprot || d.keys_only) worst = std::min(p.cbU, d.T - ncoded(d)) * sb.bf16;
+  if (hc.unprot) worst = std::max(worst, std::min(p.cqU, ncoded(d)) * sb.coded_u);
+  if (hc.prot)
+    worst = std::max(worst, d.keys_only ? std::min(p.cqK, ncoded(d)) * sb.coded_k : std::min(p.cbP, d.T) * sb.bf16);
+  if (mean > 262144.0 && worst > 1.15 * mean) {
+    p = plan_for(d, sb, mean / 2);
+    limit_splits(d, &p);
+  }
+  return p;
+}
+
+// Least workspace a launch accepts / workspace of the plan it then runs with.
+size_t ws_least_for(const hg_cache* c, int begin, int count) {
+  DecodePlan one;
+  plan_decode(c, begin, count, &one);
+  return plan_ws_bytes(c->d, count, one);
+}
+
 size_t ws_size_for(const hg_cache* c, int begin, int count) {
-  const DecodePlan p = plan_decode(c, begin, count);
-  return (size_t)ws_bytes(c->d, count, max_items_of(c->d, p));
+  DecodePlan one;
+  const DecodePlan p = plan_decode(c, begin, count, &one);
+  return std::max(plan_ws_bytes(c->d, count, one), plan_ws_bytes(c->d, count, p));
+}
+
+// A launch over more than kMaxLayersPerLaunch layers reuses the workspace for
+// each group of layers; the bound is the largest over every placement.
+template <class F>
+hg_status workspace_bound(const hg_cache* c, int32_t layer_count, size_t* bytes, F size_for) {
+  if (!c || !bytes || layer_count < 1 || layer_count > c->d.L) return HG_ERR_INVALID_ARG;
+  size_t need = 0;
+  for (int b = 0; b < c->d.L; ++b) {
+    const int n = std::min<int>(std::min<int>(layer_count, kMaxLayersPerLaunch), c->d.L - b);
+    need = std::max(need, size_for(c, b, n));
+  }
+  *bytes = need;
+  return HG_OK;
 }
 
 hg_status cuda_status(cudaError_t e) { return e == cudaSuccess ? HG_OK : HG_ERR_CUDA; }
@@ -486,16 +549,7 @@ hg_status hg_append_kv(hg_cache* c, int32_t layer_begin, int32_t layer_count, co
 }
 
 hg_status hg_decode_workspace_size(const hg_cache* c, int32_t layer_count, size_t* bytes) {
-  if (!c || !bytes || layer_count < 1 || layer_count > c->d.L) return HG_ERR_INVALID_ARG;
-  // A launch over more than kMaxLayersPerLaunch layers reuses the workspace for
-  // each group of layers; the bound is the largest over every placement.
-  size_t need = 0;
-  for (int b = 0; b < c->d.L; ++b) {
-    const int n = std::min<int>(std::min<int>(layer_count, kMaxLayersPerLaunch), c->d.L - b);
-    need = std::max(need, ws_size_for(c, b, n));
-  }
-  *bytes = need;
-  return HG_OK;
+  return workspace_bound(c, layer_count, bytes, ws_size_for);
 }
 
 hg_status hg_workspace_clear(void* ws, size_t bytes, hg_stream_t stream) {
@@ -541,56 +595,32 @@ hg_status hg_workspace_status(const void* ws, uint32_t* status, hg_stream_t stre
 
 namespace {
 
-// CTA order of the work items.  Consecutive CTAs land on different SMs and
-// CTA b and b + (number of SMs) mostly on the same one, so the items are
-// sorted by estimated cost (largest first) and dealt out in rounds of one per
-// SM, every other round reversed: each SM gets a mix of large and small items
-// instead of whatever the (layer, row, head) enumeration puts together.
-// Returns the number of ordered CTAs (0: natural order).
-int order_items(const hg_cache* c, int begin, int count, const DecodeParams& p, int total,
-                uint32_t* order) {
-  if (total > kMaxOrderedItems || total < 2) return 0;
-  const Dims& d = c->d;
-  if (d.B > kOrderMaxRow || p.max_items > kOrderMaxChunk) return 0;
+// The launch's runs of items, costliest full chunk first; returns the items.
+// Consecutive CTAs land on different SMs and CTA b and b + (number of SMs)
+// mostly on the same one, so the kernel takes the items in rounds of one per
+// SM, every other round reversed: each SM gets a mix of large and small items.
+int fill_runs(const Dims& d, const HeadCounts& hc, DecodeParams* p) {
   const SegBytes sb = seg_bytes(d);
-  std::vector<std::pair<double, int>> cost;
-  std::vector<uint32_t> rec;
-  cost.reserve(total);
-  rec.reserve(total);
-  int item = 0;
-  for (int i = 0; i < count; ++i) {
-    const DecodeLayer& L = p.layer[i];
-    const ChunkCounts cc = {L.nbU, L.nqU, L.nqK, L.nbP};
-    for (int b = 0; b < d.B; ++b) {
-      for (int h = 0; h < d.H; ++h) {
-        const int cls = head_class(d, c->layer_mask[begin + i], h);
-        int nb;
-        const int ni = head_chunks(cls, cc, &nb);
-        const int blen = (cls == kProtected ? d.T : d.T - d.nq + d.ns) + L.appended;
-        const int clen = ncoded(d);
-        const int bc = (cls == kProtected) ? p.plan.cbP : p.plan.cbU;
-        const int qc = (cls == kKeysOnly) ? p.plan.cqK : p.plan.cqU;
-        const double qb = (cls == kKeysOnly) ? sb.coded_k : sb.coded_u;
-        for (int r = 0; r < ni; ++r) {
-          double w;
-          if (r < nb) w = std::min(bc, blen - r * bc) * sb.bf16;
-          else w = std::min(qc, clen - (r - nb) * qc) * qb;
-          cost.emplace_back(w, item++);
-          rec.push_back(order_record(i, b, h, r));
-        }
-      }
-    }
+  struct Run {
+    double cost;
+    int kind, heads, chunks;
+  };
+  const DecodePlan& pl = p->plan;
+  Run runs[kWorkRuns] = {
+      {std::min(pl.cqU, ncoded(d)) * sb.coded_u, kWorkCoded, hc.unprot, p->counts.nqU},
+      {std::min(pl.cqK, ncoded(d)) * sb.coded_k, kWorkKeysOnly, d.keys_only ? hc.prot : 0, p->counts.nqK},
+      {std::min(pl.cbP, d.T) * sb.bf16, kWorkProtected, d.keys_only ? 0 : hc.prot, p->counts.nbP},
+      {std::min(pl.cbU, d.T - ncoded(d)) * sb.bf16, kWorkBf16, hc.unprot + (d.keys_only ? hc.prot : 0), p->counts.nbU}};
+  std::stable_sort(runs, runs + kWorkRuns, [](const Run& a, const Run& b) { return a.cost > b.cost; });
+  int total = 0, n = 0;
+  for (const Run& r : runs) {
+    const int items = r.heads * d.B * r.chunks;
+    if (items == 0) continue;
+    total += items;
+    p->run[n++] = {r.kind, total, r.heads};
   }
-  if (item != total) return 0;
-  std::stable_sort(cost.begin(), cost.end(),
-                   [](const std::pair<double, int>& a, const std::pair<double, int>& b) { return a.first > b.first; });
-  const int S = sm_count();
-  for (int j = 0; j < total; ++j) {
-    const int r = j / S, s = j % S;
-    const bool full_round = (r + 1) * S <= total;
-    const int blk = r * S + ((r & 1) && full_round ? S - 1 - s : s);
-    order[blk] = rec[cost[j].second];
-  }
+  for (; n < kWorkRuns; ++n) p->run[n] = {kWorkBf16, total, 1};
+  p->deal = sm_count();
   return total;
 }
 
@@ -613,7 +643,9 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     p.d = d;
     p.arena = c->arena;
     p.n_layers = n;
-    p.plan = plan_decode(c, layer_begin + done, n);
+    DecodePlan one_wave;
+    p.plan = plan_decode(c, layer_begin + done, n, &one_wave);
+    if (plan_ws_bytes(d, n, p.plan) > ws_bytes_given) p.plan = one_wave;
     p.max_items = max_items_of(d, p.plan);
     p.scale_log2 = scale * 1.4426950408889634f;
     p.q = static_cast<const uint16_t*>(q) + (size_t)done * layer_elems;
@@ -628,22 +660,19 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     p.counters = reinterpret_cast<uint32_t*>(wsb + kWsHeaderBytes);
     p.partials = reinterpret_cast<float*>(wsb + kWsHeaderBytes + ws_counter_bytes(d, n));
     fill_table(c, layer_begin + done, n, &p.lt);
-    int total = 0;
+    int most = 0, unprot = 0;
     for (int i = 0; i < n; ++i) {
       const int l = layer_begin + done + i;
-      const ChunkCounts cc = counts_of(d, c->appended[l], p.plan);
-      DecodeLayer& dl = p.layer[i];
-      dl.appended = c->appended[l];
-      dl.nbU = cc.nbU;
-      dl.nqU = cc.nqU;
-      dl.nqK = cc.nqK;
-      dl.nbP = cc.nbP;
-      dl.items_per_row = row_chunks(d, c->layer_mask[l], cc);
-      dl.item_base = total;
-      total += dl.items_per_row * d.B;
+      p.appended[i] = c->appended[l];
+      most = std::max(most, c->appended[l]);
+      p.unprot_before[i] = unprot;
+      unprot += d.H - popc64(c->layer_mask[l]);
     }
-    p.total_items = total;
-    p.n_order = order_items(c, layer_begin + done, n, p, total, p.order);
+    // chunk counts at the largest appended count of the launch: a layer with
+    // fewer tokens may get an empty last chunk, which merges as nothing
+    p.counts = counts_of(d, most, p.plan);
+    p.total_items = fill_runs(d, {unprot, n * d.H - unprot}, &p);
+    const int total = p.total_items;
     const hg_status st = cuda_status(launch_decode(p, total, reinterpret_cast<cudaStream_t>(stream)));
     if (st != HG_OK) return st;
   }
@@ -657,7 +686,7 @@ hg_status decode_checks(const hg_cache* c, int32_t layer_begin, int32_t layer_co
   if (!(softmax_scale == softmax_scale)) return HG_ERR_INVALID_ARG;  // NaN
   for (int done = 0; done < layer_count; done += kMaxLayersPerLaunch) {
     const int n = std::min(kMaxLayersPerLaunch, layer_count - done);
-    if (ws_bytes_given < ws_size_for(c, layer_begin + done, n)) return HG_ERR_WORKSPACE_TOO_SMALL;
+    if (ws_bytes_given < ws_least_for(c, layer_begin + done, n)) return HG_ERR_WORKSPACE_TOO_SMALL;
   }
   return HG_OK;
 }
@@ -695,6 +724,10 @@ hg_status hg_decode_step(hg_cache* c, int32_t layer_begin, int32_t layer_count, 
 }  // extern "C"
 
 namespace hg {
+
+hg_status decode_least_workspace(const hg_cache* c, int32_t layer_count, size_t* bytes) {
+  return workspace_bound(c, layer_count, bytes, ws_least_for);
+}
 
 hg_status decode_attention_on_scratch(const hg_cache* c, int32_t layer_begin, int32_t layer_count,
                                       const void* q, void* out, float softmax_scale, void* scratch,

@@ -1199,6 +1199,40 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
   }
 }
 
+// (layer in the launch, batch row, KV head, chunk of the head) of CTA x's item.
+// Runs of items and, in a run, chunks, heads and rows are found by arithmetic
+// on the launch parameters, the layer by a warp-wide comparison with the
+// per-layer counts, the head by its rank among the layer's mask bits, so the
+// order of items -- costliest first, dealt out over the SMs -- needs no table
+// and holds for any number of items.
+__device__ __forceinline__ void locate_item(const DecodeParams& p, int x, int& li, int& b, int& h, int& r) {
+  const Dims& d = p.d;
+  const int round = x / p.deal;
+  int item = x;
+  if ((round & 1) && (round + 1) * p.deal <= p.total_items) item = (2 * round + 1) * p.deal - 1 - x;
+  int k = 0, start = 0;
+  while (k + 1 < kWorkRuns && item >= p.run[k].end) start = p.run[k++].end;
+  const int kind = p.run[k].kind;
+  const int rows = p.run[k].heads * d.B;
+  const int in_run = item - start;
+  const int chunk = in_run / rows, in_chunk = in_run - chunk * rows;
+  const int rank = in_chunk / d.B;  // of the (layer, head) among the run's
+  b = in_chunk - rank * d.B;
+  r = (kind == kWorkBf16 || kind == kWorkProtected) ? chunk : p.counts.nbU + chunk;
+  // heads of this kind in the layers before layer l
+  const bool all = kind == kWorkBf16 && d.keys_only, prot = kind == kWorkKeysOnly || kind == kWorkProtected;
+  auto before = [&](int l) { return all ? l * d.H : (prot ? l * d.H - p.unprot_before[l] : p.unprot_before[l]); };
+  li = 0;
+  if (p.n_layers > 1) {
+    const int l0 = threadIdx.x & 31, l1 = l0 + 32;
+    const bool in0 = l0 < p.n_layers && before(l0) <= rank, in1 = l1 < p.n_layers && before(l1) <= rank;
+    li = __popc(__ballot_sync(kFull, in0)) + __popc(__ballot_sync(kFull, in1)) - 1;
+  }
+  const int n = rank - before(li);
+  const uint64_t mask = p.lt.mask[li];
+  h = all ? n : nth_bit(prot ? mask : ~mask, n);
+}
+
 template <int BITS, int NT, int BASE, int MB>
 __global__ void __launch_bounds__(kThreads, NT == 1 ? 4 : 2)
 decode_kernel(const __grid_constant__ DecodeParams p) {
@@ -1219,37 +1253,13 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
     *reinterpret_cast<volatile int*>(smem + SmemLayout<NT>::bar + 8 * kMaxStages) = 0;  // abort flag
     prefetch_tensormap(&p.arena_map);
   }
-  // (layer, batch row, KV head, chunk) of this CTA's item: a packed record
-  // for host-ordered CTAs, else a search of the layer and head tables
-  int li = 0, b, h, r;
-  if ((int)blockIdx.x < p.n_order) {
-    const uint32_t e = p.order[blockIdx.x];
-    li = (int)(e & 63u);
-    h = (int)((e >> 6) & 63u);
-    r = (int)((e >> 12) & 31u);
-    b = (int)(e >> 17);
-  } else {
-    const int item = (int)blockIdx.x;
-    while (li + 1 < p.n_layers && p.layer[li + 1].item_base <= item) ++li;
-    const DecodeLayer& L0 = p.layer[li];
-    const int in_layer = item - L0.item_base;
-    b = in_layer / L0.items_per_row;
-    r = in_layer - b * L0.items_per_row;
-    const ChunkCounts c0 = {L0.nbU, L0.nqU, L0.nqK, L0.nbP};
-    for (h = 0; h < d.H; ++h) {
-      int nb0;
-      const int n0 = head_chunks(head_class(d, p.lt.mask[li], h), c0, &nb0);
-      if (r < n0) break;
-      r -= n0;
-    }
-  }
+  int li, b, h, r;
+  locate_item(p, (int)blockIdx.x, li, b, h, r);
   const int G = d.G;
-  const DecodeLayer& L = p.layer[li];
   const uint64_t mask = p.lt.mask[li];
-  const ChunkCounts cc = {L.nbU, L.nqU, L.nqK, L.nbP};
   const int cls = head_class(d, mask, h);
   int nb;
-  const int ni = head_chunks(cls, cc, &nb);
+  const int ni = head_chunks(cls, p.counts, &nb);
   const LayerGeom lg = layer_geom(d, mask);
   const HeadGeom hd = head_geom(d, lg, h);
   const char* Lb = p.arena + p.lt.base[li];
@@ -1271,7 +1281,7 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
   if (!coded) {
     const int c = (cls == kProtected) ? p.plan.cbP : p.plan.cbU;
     tb = r * c;
-    te = min(tb + c, hd.bf16_prefill + L.appended);
+    te = min(tb + c, hd.bf16_prefill + p.appended[li]);
   } else {
     const int c = (cls == kKeysOnly) ? p.plan.cqK : p.plan.cqU;
     tb = (r - nb) * c;
@@ -1292,7 +1302,7 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
     sg.v = Lb + hd.vb + b * hd.kb_bs;
     sg.k_row0 = (int)((p.lt.base[li] + hd.kb + b * hd.kb_bs) >> 8);
     sg.v_row0 = (int)((p.lt.base[li] + hd.vb + b * hd.kb_bs) >> 8);
-    const int pos = hd.bf16_prefill + L.appended - 1;  // the step's new token
+    const int pos = hd.bf16_prefill + p.appended[li] - 1;  // the step's new token
     if (p.k_new && pos >= tb && pos < te) {
       const size_t row = (((size_t)li * d.B + b) * d.H + h) * kD;
       sg.new_pos = pos;

@@ -54,26 +54,21 @@ struct AppendParams {
 //   cqU  coded tokens of quantized heads               (codes for K and V)
 //   cqK  coded tokens of keys-only heads               (BF16 K, coded V)
 //   cbP  BF16 tokens of protected K+V heads
-// Per layer, the host passes the resulting chunk counts of each kind.
 struct DecodePlan {
   int cbU, cqU, cqK, cbP;
 };
 
-struct DecodeLayer {
-  int appended;
-  int nbU, nqU, nqK, nbP;  // chunks per head of each kind
-  int items_per_row;       // chunks of all heads of one batch row
-  int item_base;           // first work item of this layer in the launch
+// A run of work items of one kind: every chunk of that kind in the launch.
+// Items of a run are numbered chunk-major (all heads' first chunks, then all
+// second ones ..., so the short last chunks come last), then by (layer, KV
+// head) of the kind's heads in order, then by batch row.
+enum WorkKind : int { kWorkBf16 = 0, kWorkCoded = 1, kWorkKeysOnly = 2, kWorkProtected = 3 };
+struct WorkRun {
+  int kind;   // WorkKind
+  int end;    // items of this run and of the runs before it
+  int heads;  // (layer, KV head) pairs of the launch that have this kind
 };
-
-// Largest launch whose CTAs get a host-chosen item order.
-constexpr int kMaxOrderedItems = 1024;
-// Packed work item: layer in the launch (6 bits), KV head (6), chunk of the
-// head (5), batch row (15).
-HG_HD uint32_t order_record(int li, int b, int h, int r) {
-  return (uint32_t)li | ((uint32_t)h << 6) | ((uint32_t)r << 12) | ((uint32_t)b << 17);
-}
-constexpr int kOrderMaxRow = 1 << 15, kOrderMaxChunk = 1 << 5;
+constexpr int kWorkRuns = 4;
 
 struct DecodeParams {
   // The arena as a two-dimensional BF16 tensor [arena_bytes / 256][128]: every
@@ -84,6 +79,7 @@ struct DecodeParams {
   const char* arena;
   int n_layers;
   DecodePlan plan;
+  ChunkCounts counts;  // chunks per head of each kind, at the launch's largest appended count
   int max_items;       // split slots per (layer, row, head) in the workspace
   float scale_log2;    // softmax_scale * log2(e)
   const uint16_t* q;   // [n_layers][B][Hq][128]
@@ -94,16 +90,16 @@ struct DecodeParams {
   const uint16_t* k_new;
   const uint16_t* v_new;
   int total_items;
+  // Runs of items, costliest chunks first; CTA x takes item x, with every
+  // second full round of `deal` CTAs (one per SM) in reverse order.
+  WorkRun run[kWorkRuns];
+  int deal;
   uint32_t* status;    // workspace status word (kStatus* bits; zero while healthy)
   uint32_t* counters;  // [n_layers][B][H]
   float* partials;     // [n_layers][B][H][max_items][G][132]
   LayerTable lt;
-  DecodeLayer layer[kMaxLayersPerLaunch];
-  // Work item of each CTA below n_order, as a packed record (order_record):
-  // the kernel reads its item's coordinates instead of searching the layer
-  // and head tables.  CTAs from n_order on take item blockIdx.x.
-  int n_order;
-  uint32_t order[kMaxOrderedItems];
+  int appended[kMaxLayersPerLaunch];
+  int unprot_before[kMaxLayersPerLaunch];  // unprotected (layer, KV head) pairs in the layers before
 };
 
 // BF16 rows per TMA box of the arena tensor map.
@@ -134,6 +130,9 @@ int decode_max_splits(int G);
 hg_status decode_attention_on_scratch(const hg_cache* cache, int32_t layer_begin, int32_t layer_count,
                                       const void* q, void* out, float softmax_scale, void* scratch,
                                       size_t scratch_bytes, hg_stream_t stream);
+// Least workspace that every launch over layer_count layers accepts (the
+// one-wave work plan's; hg_decode_workspace_size may ask for more).
+hg_status decode_least_workspace(const hg_cache* cache, int32_t layer_count, size_t* bytes);
 // Device address of the allocation-free entry point's scratch array on the
 // current device (its first 512 bytes are a workspace header with the status
 // word at byte 0).

@@ -188,8 +188,8 @@ HG_HD int bf16_pos(const Dims& d, int cls, int t) {
 // chunks: BF16 segments of quantized / keys-only heads into chunks of cbU
 // tokens, coded segments into chunks of cqU (quantized heads) or cqK
 // (keys-only heads) tokens, BF16 segments of protected K+V heads into chunks
-// of cbP tokens.  A work item is one chunk.  Items of one (layer, row) are
-// numbered head by head, BF16 chunks before coded chunks.
+// of cbP tokens.  A work item is one chunk; a head's chunks are numbered BF16
+// chunks first, then coded chunks.
 // ---------------------------------------------------------------------------
 HG_HD int cdiv(int a, int b) { return (a + b - 1) / b; }
 
@@ -216,10 +216,19 @@ HG_HD int head_chunks(int cls, const ChunkCounts& c, int* n_bf16) {
   return c.nbU + (cls == kKeysOnly ? c.nqK : c.nqU);
 }
 
-HG_HD int row_chunks(const Dims& d, uint64_t mask, const ChunkCounts& c) {
-  int tot = 0, nb;
-  for (int h = 0; h < d.H; ++h) tot += head_chunks(head_class(d, mask, h), c, &nb);
-  return tot;
+// Position of the n-th set bit of m (n from 0; m has more than n set bits).
+HG_HD int nth_bit(uint64_t m, int n) {
+  int pos = 0;
+#pragma unroll
+  for (int w = 32; w >= 1; w >>= 1) {
+    const int c = popc64(m & ((1ull << w) - 1ull));
+    if (n >= c) {
+      n -= c;
+      pos += w;
+      m >>= w;
+    }
+  }
+  return pos;
 }
 
 // Decode workspace: a 512-byte header (status word at byte 0), a counter per

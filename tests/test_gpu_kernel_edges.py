@@ -1,0 +1,78 @@
+"""Kernels and dispatch rules at the sizes where they can go wrong, against the CPU oracle."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2609_35800_gb300 as hg
+from paper_2609_35800_gb300 import workloads as wl
+from paper_2609_35800_gb300.runner import CacheRunner
+
+from parity import assert_close, attention_reference, bits16, n_salient
+
+pytestmark = pytest.mark.gpu
+
+SIGMA = float(np.float32(1.0 / np.sqrt(128.0)))
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_35800_gb300 import build
+    build.build()
+
+
+def _row_reference(runner, layer, row, k, v, q, news):
+    """fp64 attention of one batch row: the oracle on that row's prefill plus the appended tokens."""
+    w = runner.w
+    o = oracle.quantize_layer(bits16(k[row:row + 1]), bits16(v[row:row + 1]), w.img_start, w.image, w.base, w.bits,
+                              runner.mask[layer], int(w.keys_only), w.kivi_group_tokens, w.kivi_group_channels,
+                              w.kivi_residual, meta16=w.meta_bits == 32, n_salient=n_salient(w))
+    ak = [bits16(kn[layer, row:row + 1]) for kn, _ in news]
+    av = [bits16(vn[layer, row:row + 1]) for _, vn in news]
+    return attention_reference(runner, o, bits16(q[layer, row:row + 1]), ak, av, SIGMA)
+
+
+@pytest.mark.parametrize("name,layers", [("internvl25_8b", 1), ("qwen25vl72b", 1), ("internvl25_8b", 3)])
+def test_decode_in_several_waves(name, layers):
+    """One layer of a large batch: heads too large to balance in one wave run as two to three waves of
+    smaller chunks (more than 1,024 of them over three layers)."""
+    w = dataclasses.replace(wl.WORKLOADS[name], layers=layers, decode_steps=2)
+    runner = CacheRunner(w)
+    kept = runner.quantize_all(keep=True)
+    news = []
+    for step in range(2):
+        k_new, v_new = wl.step_new_kv(w, step, "cuda")
+        q = wl.step_query(w, step, "cuda")
+        out = runner.decode_step(step, q=q, k_new=k_new, v_new=v_new)
+        news.append((k_new, v_new))
+    for layer in {0, layers - 1}:
+        for row in (0, w.batch - 1):
+            ref = _row_reference(runner, layer, row, *kept[layer], q, news)
+            assert_close(bits16(out[layer, row:row + 1]), ref, "%s layer %d row %d" % (name, layer, row))
+
+
+@pytest.mark.parametrize("base,keys_only,prefix", [(wl.BASE_MINMAX, 0, 0), (wl.BASE_MINMAX, 1, 64),
+                                                   (wl.BASE_AKVQ, 0, 64), (wl.BASE_KIVI, 1, 32)])
+def test_decode_layers_with_different_appended_counts(base, keys_only, prefix):
+    """Layers of one launch that hold 0, 1 and 70 appended tokens: the launch's chunk counts are the
+    largest layer's, so the others have an empty last BF16 chunk (with no text at all, an empty only one)."""
+    w = wl.custom("uneven", 3, 2, 8, 4, prefix, 320, 0, base, 2, keys_only, decode_steps=70, seed=5,
+                  protected=[(0, 1), (1, 0), (2, 3)], residual=0)
+    runner = CacheRunner(w)
+    kept = runner.quantize_all(keep=True)
+    counts = (0, 1, 70)
+    news = [wl.step_new_kv(w, s, "cuda") for s in range(70)]
+    for layer, n in enumerate(counts):
+        for k_new, v_new in news[:n]:
+            hg.hg_append_kv(runner.cache, layer, 1, k_new[layer], v_new[layer])
+    q = wl.step_query(w, 0, "cuda")
+    out = torch.full_like(q, float("nan"))
+    hg.hg_decode_attention(runner.cache, 0, 3, q, out, SIGMA, runner.ws, runner.ws_bytes)
+    for layer, n in enumerate(counts):
+        for row in range(w.batch):
+            ref = _row_reference(runner, layer, row, *kept[layer], q, news[:n])
+            assert_close(bits16(out[layer, row:row + 1]), ref, "layer %d row %d" % (layer, row))
