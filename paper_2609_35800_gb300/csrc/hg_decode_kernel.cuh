@@ -7,12 +7,13 @@
 // keys with coded values.  The only branch on the mask or the image span is
 // therefore taken once per CTA.
 //
-// Tiles of the chunk stream through a TMA pipeline in a 64 KB shared buffer
-// (two to four stages depending on the tile size, one mbarrier each): BF16
-// rows arrive as tensor-map boxes with the 128-byte swizzle, packed codes and
-// metadata as one bulk copy per array, all issued by one thread.  Each warp
-// owns 16-token slices and computes, with mma.sync
-// m16n8k16 (BF16 in, fp32 accumulate):
+// Each of the CTA's four warps takes a quarter of the chunk's tokens and
+// streams it through a TMA pipeline of its own (12 KB, two to four slots with
+// an mbarrier each, copies issued by its lane 0): BF16 rows arrive as
+// tensor-map boxes with the 128-byte swizzle, packed codes and metadata as
+// one bulk copy per array.  The warps meet only before their first tile and
+// after their last one.  A warp works on 16-token slices and computes, with
+// mma.sync m16n8k16 (BF16 in, fp32 accumulate):
 //   S^T[token][query] = K . q     A = keys (BF16 via ldmatrix, or codes
 //                                 expanded exactly to BF16 in registers),
 //                                 B = the G queries of the KV head (padded to 8)
@@ -53,9 +54,8 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kWarps = 4;
-constexpr int kBufBytes = 49152;   // pipeline buffer (stages of one tile each)
-constexpr int kBf16Tile = 48;      // tokens per tile of BF16 rows (K 12 KB + V 12 KB)
-constexpr int kMixTile = 48;       // tokens per tile of BF16 keys + coded values
+constexpr int kBufBytes = 49152;   // pipeline buffers of the four warps
+constexpr int kWarpBuf = kBufBytes / kWarps;
 constexpr int kPartialStride = kD + 4;  // m, l, 2 pad, o[128]: rows of 528 bytes (16-byte multiple)
 // Shared memory, from a 1024-byte aligned base (swizzled TMA boxes need it).
 constexpr int kStageOff = 0;                    // pipeline buffer
@@ -70,10 +70,10 @@ __device__ __forceinline__ int qidx(int r, int c) { return r * kQRow + c; }
 template <int NT>
 struct SmemLayout {
   static constexpr int q = kStageOff + kBufBytes;  // float q[NT * 8][kQRow] (qidx)
-  static constexpr int bar = q + NT * 8 * kQRow * 4;  // mbarrier per stage (4), abort flag
-  static constexpr int bytes = bar + 64 + 1024;    // + alignment slack
+  static constexpr int bar = q + NT * 8 * kQRow * 4;  // mbarrier per warp and slot (4 x 4), abort flag
+  static constexpr int bytes = bar + 192 + 1024;   // + alignment slack
 };
-constexpr int kMaxStages = 4;
+constexpr int kMaxSlots = 4;  // per warp
 constexpr unsigned kFull = 0xffffffffu;
 // A wait for a tile is declared stuck after kWaitRounds suspensions of up to
 // kWaitSleepNs each (about a second); a healthy wait ends within microseconds.
@@ -87,10 +87,6 @@ template <int VM>
 struct NZOf {
   static constexpr int value = VM == V_TOKEN ? 1 : (VM == V_KIVI ? 4 : 1);
 };
-
-// Tokens per tile of coded K + coded V: per-token groups 256 (2-bit) / 128
-// (4-bit); KIVI-style (32 bytes of key metadata per token) 128.
-__host__ __device__ constexpr int coded_tile(int bits, int km) { return (bits == 2 && km != 2) ? 256 : 128; }
 
 struct Seg {
   const char* k;   // BF16 key rows (K_BF16)
@@ -216,68 +212,89 @@ __device__ __forceinline__ void meta_quad(const char* base, int i, float2 (&m)[4
   }
 }
 
+// One warp's pipeline.  A tile is the tokens between two refills.  SPLIT (BF16
+// rows for K and V): a 16-token tile's K and V rows land in slots of their
+// own, so a K slot is refilled while the tile's values are still at work --
+// three 4 KB slots where two 8 KB ones would not fit.  Else a slot holds a
+// whole tile, as large as fits twice, since a wait and a refill cost a warp
+// as much as a third of a slice: 64 tokens of per-token 2-bit codes (5 KB; 32
+// and 48 measured 4% and 1.5% slower on one layer of 32 rows, 8 KV heads and
+// 8,576 tokens), 32 at 3 and 4 bits (16: 3% slower with rotated 4-bit keys; the
+// value offsets are folded once per tile, and over 48 or 64 tokens of wider
+// codes the fp32 accumulators lose bits that the output shows), a KIVI-style
+// group of 32, 16 tokens of BF16 keys and coded values.
+//
+// Before, one thread filled a ring of tiles for all four warps, with a CTA
+// barrier per tile: a warp had one or two 16-token slices between barriers.
+// Separate pipelines, with every address known to be the same in the warp's
+// lanes (the refill runs on the uniform path), measured, one layer per launch:
+// that layer 90 -> 84 us, 3,520 tokens of 4-bit rotated keys 53 -> 50 us,
+// 32 KV heads of KIVI-style codes in 16 rows 123 -> 109 us, one row of 4 KV
+// heads and 1,460 tokens 9.4 -> 8.1 us.
 template <int BITS, int KM, int VM, int MB>
 struct Tile {
-  static constexpr int tokens = (KM == K_BF16 && VM == V_BF16) ? kBf16Tile
-                                : (KM == K_BF16 ? kMixTile : coded_tile(BITS, KM));
+  static constexpr bool SPLIT = KM == K_BF16 && VM == V_BF16;
+  static constexpr int tokens = (KM == K_BF16) ? 16 : (KM == K_KIVI ? kKiviGroup : (BITS == 2 ? 64 : 32));
   static constexpr int kc_bytes = (KM == K_BF16) ? tokens * 256 : tokens * 16 * BITS;
   static constexpr int km_bytes = (KM == K_TOKEN) ? tokens * MB : (KM == K_KIVI ? tokens * 4 * MB : 0);
   static constexpr int vc_bytes = (VM == V_BF16) ? tokens * 256 : tokens * 16 * BITS;
   static constexpr int vm_bytes = (VM == V_TOKEN) ? tokens * MB : (VM == V_KIVI ? tokens * 4 * MB : 0);
-  static constexpr int kc_off = 0;
-  static constexpr int km_off = kc_off + kc_bytes;
-  static constexpr int vc_off = km_off + km_bytes;
+  static constexpr int km_off = kc_bytes;  // from the tile's K base
+  static constexpr int vc_off = SPLIT ? 0 : km_off + km_bytes;  // from its V base (not SPLIT: the slot)
   static constexpr int vm_off = vc_off + vc_bytes;
-  // stages start on 1024-byte boundaries (swizzled BF16 boxes)
-  static constexpr int stage_bytes = ((vm_off + vm_bytes + 1023) / 1024) * 1024;
-  static constexpr int stages = (kBufBytes / stage_bytes) > kMaxStages ? kMaxStages : (kBufBytes / stage_bytes);
-  static_assert(stages >= 2, "a tile must fit twice in the pipeline buffer");
-  static_assert(tokens % kArenaBoxRows == 0, "BF16 tiles are whole TMA boxes");
-  static_assert(VM != V_BF16 || vc_off % 1024 == 0, "swizzled value boxes start on 1024-byte boundaries");
+  // slots that hold BF16 rows start on 1024-byte boundaries (swizzled boxes)
+  static constexpr int align = (KM == K_BF16) ? 1024 : 128;
+  static constexpr int slot_bytes = ((SPLIT ? kc_bytes : vm_off + vm_bytes) + align - 1) / align * align;
+  static constexpr int slots = (kWarpBuf / slot_bytes) > kMaxSlots ? kMaxSlots : (kWarpBuf / slot_bytes);
+  static_assert(slots >= 2, "a tile must fit twice in a warp's buffer");
+  static_assert(KM != K_BF16 || tokens == kArenaBoxRows, "a BF16 tile is one TMA box high");
+  static_assert(kWarpBuf % 1024 == 0, "the warps' buffers keep the slots' alignment");
 };
 
-// One tile into a stage, issued by a single thread: the expected byte count
-// on the stage's mbarrier, then the copies.  A BF16 operand of R rows lands
-// as two column halves of R x 128 bytes (channels 0-63, 64-127), each written
-// by TMA boxes of kArenaBoxRows rows with the 128-byte swizzle (16-byte chunk
-// c of row r at chunk c ^ (r % 8)); rows past the chunk end are loaded too and
-// ignored or zeroed by the consumers.  Packed codes and metadata arrive as one
-// bulk copy per array (metadata rounded up to 16 bytes: the arena pads every
-// metadata row to 16 bytes); bytes past nvalid tokens are left stale.
-template <int BITS, int KM, int VM, int MB>
-__device__ __forceinline__ void issue_tile(uint32_t st, uint32_t bar, const Seg& sg, int t0, int nvalid,
-                                           const CUtensorMap* map) {
-  using TL = Tile<BITS, KM, VM, MB>;
-  constexpr int kmb = (KM == K_TOKEN) ? MB : 4 * MB;  // metadata bytes per token
-  constexpr int vmb = (VM == V_TOKEN) ? MB : 4 * MB;
-  constexpr int kBox = kArenaBoxRows * 128;  // bytes of one box
-  const int boxes = (nvalid + kArenaBoxRows - 1) / kArenaBoxRows;
-  const uint32_t kc_bytes = (KM == K_BF16) ? boxes * 2 * kBox : nvalid * 16 * BITS;
-  const uint32_t km_bytes = (KM == K_BF16) ? 0u : (uint32_t)((nvalid * kmb + 15) & ~15);
-  const uint32_t vc_bytes = (VM == V_BF16) ? boxes * 2 * kBox : nvalid * 16 * BITS;
-  const uint32_t vm_bytes = (VM == V_BF16) ? 0u : (uint32_t)((nvalid * vmb + 15) & ~15);
-  mbar_arrive_expect_tx(bar, kc_bytes + km_bytes + vc_bytes + vm_bytes);
-  if (KM == K_BF16) {
-    for (int bx = 0; bx < boxes; ++bx)
-      for (int hf = 0; hf < 2; ++hf)
-        tma_load_2d(st + TL::kc_off + hf * (TL::tokens * 128) + bx * kBox, map, hf * 64,
-                    sg.k_row0 + t0 + bx * kArenaBoxRows, bar);
-  } else {
-    bulk_g2s(st + TL::kc_off, sg.kc + (size_t)t0 * 16 * BITS, kc_bytes, bar);
-    bulk_g2s(st + TL::km_off, sg.km + (size_t)t0 * kmb, km_bytes, bar);
-  }
-  if (VM == V_BF16) {
-    for (int bx = 0; bx < boxes; ++bx)
-      for (int hf = 0; hf < 2; ++hf)
-        tma_load_2d(st + TL::vc_off + hf * (TL::tokens * 128) + bx * kBox, map, hf * 64,
-                    sg.v_row0 + t0 + bx * kArenaBoxRows, bar);
-  } else {
-    bulk_g2s(st + TL::vc_off, sg.vc + (size_t)t0 * 16 * BITS, vc_bytes, bar);
-    bulk_g2s(st + TL::vm_off, sg.vm + (size_t)t0 * vmb, vm_bytes, bar);
-  }
+// BF16 rows [row0, +16) of the arena into shared memory at dst: two column
+// halves of 16 x 128 bytes (channels 0-63, 64-127), each a TMA box with the
+// 128-byte swizzle (16-byte chunk c of row r at chunk c ^ (r % 8)).  Rows past
+// the segment's end are loaded too and ignored or zeroed by the consumer.
+__device__ __forceinline__ void issue_rows(uint32_t dst, const CUtensorMap* map, int row0, uint32_t bar) {
+  tma_load_2d(dst, map, 0, row0, bar);
+  tma_load_2d(dst + kArenaBoxRows * 128, map, 64, row0, bar);
 }
 
-// Bounded wait for a phase of a stage's mbarrier.  On timeout, or once another
+// Fill i of a warp's pipeline into its slot, issued by a single thread: the
+// expected byte count on the slot's mbarrier, then the copies.  SPLIT: fill 2t
+// is the K rows of the warp's tile t, fill 2t + 1 its V rows; else fill t is
+// tile t.  Packed codes and metadata arrive as one bulk copy per array
+// (metadata rounded up to 16 bytes: the arena pads every metadata row to 16
+// bytes); bytes past the range [wb, we) are left stale.
+template <int BITS, int KM, int VM, int MB>
+__device__ __forceinline__ void issue_fill(uint32_t slot, uint32_t bar, const Seg& sg, int i, int wb, int we,
+                                           const CUtensorMap* map) {
+  using TL = Tile<BITS, KM, VM, MB>;
+  const int t0 = wb + (TL::SPLIT ? i >> 1 : i) * TL::tokens;
+  if (TL::SPLIT) {
+    mbar_arrive_expect_tx(bar, TL::kc_bytes);
+    issue_rows(slot, map, ((i & 1) ? sg.v_row0 : sg.k_row0) + t0, bar);
+    return;
+  }
+  constexpr int kmb = (KM == K_TOKEN) ? MB : 4 * MB;  // metadata bytes per token
+  constexpr int vmb = (VM == V_TOKEN) ? MB : 4 * MB;
+  const int n = min(TL::tokens, we - t0);
+  const uint32_t kc_bytes = (KM == K_BF16) ? TL::kc_bytes : n * 16 * BITS;
+  const uint32_t km_bytes = (KM == K_BF16) ? 0u : (uint32_t)((n * kmb + 15) & ~15);
+  const uint32_t vc_bytes = n * 16 * BITS;
+  const uint32_t vm_bytes = (uint32_t)((n * vmb + 15) & ~15);
+  mbar_arrive_expect_tx(bar, kc_bytes + km_bytes + vc_bytes + vm_bytes);
+  if (KM == K_BF16) {
+    issue_rows(slot, map, sg.k_row0 + t0, bar);
+  } else {
+    bulk_g2s(slot, sg.kc + (size_t)t0 * 16 * BITS, kc_bytes, bar);
+    bulk_g2s(slot + TL::km_off, sg.km + (size_t)t0 * kmb, km_bytes, bar);
+  }
+  bulk_g2s(slot + TL::vc_off, sg.vc + (size_t)t0 * 16 * BITS, vc_bytes, bar);
+  bulk_g2s(slot + TL::vm_off, sg.vm + (size_t)t0 * vmb, vm_bytes, bar);
+}
+
+// Bounded wait for a phase of a slot's mbarrier.  On timeout, or once another
 // warp gave up, marks the CTA aborted, records the failure in the workspace
 // status word and returns false (the caller skips the tile's work).
 __device__ __forceinline__ bool wait_tile(uint32_t bar, uint32_t parity, volatile int* abort, uint32_t* status,
@@ -480,28 +497,31 @@ __device__ __forceinline__ void vscale_update(WarpState<NT, NZ>& ws, float smax)
 }
 
 // ---------------------------------------------------------------------------
-// One tile: every warp processes its 16-token slices
+// One tile of a warp: kst / vst its K and V in shared memory.  between() runs
+// after the last read of kst by a SPLIT tile (one slice) and returns false
+// when the values did not arrive; the tile's probabilities are then dropped.
 // ---------------------------------------------------------------------------
-template <int BITS, int NT, int KM, int VM, bool ROT, int MB>
-__device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws, const char* st,
+template <int BITS, int NT, int KM, int VM, bool ROT, int MB, class F>
+__device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws, const char* kst, const char* vst,
                                              int nvalid, const uint32_t (&qb)[NT][8][2],
                                              const uint32_t (&ql)[NT][8][2], const float* q_s,
                                              const float (&s1)[NT][2], const float (&s0)[NT][2],
-                                             float scale_log2, int warp, int lane) {
+                                             float scale_log2, int lane, F&& between) {
   using TL = Tile<BITS, KM, VM, MB>;
   constexpr int NZ = NZOf<VM>::value;
   const int g = lane >> 2, tq = lane & 3;
-  const uint32_t st_u32 = smem_u32(st);
-  const uint32_t* kc32 = reinterpret_cast<const uint32_t*>(st + TL::kc_off);
-  const char* kmp = st + TL::km_off;
-  const uint32_t* vc32 = reinterpret_cast<const uint32_t*>(st + TL::vc_off);
-  const char* vmp = st + TL::vm_off;
+  const uint32_t k_u32 = smem_u32(kst), v_u32 = smem_u32(vst) + TL::vc_off;
+  const uint32_t* kc32 = reinterpret_cast<const uint32_t*>(kst);
+  const char* kmp = kst + TL::km_off;
+  const uint32_t* vc32 = reinterpret_cast<const uint32_t*>(vst + TL::vc_off);
+  const char* vmp = vst + TL::vm_off;
 
   // KIVI-style keys: a warp takes whole 32-token groups (two slices) so the
   // group's scaled query fragments are built once.
   constexpr int SPU = (KM == K_KIVI) ? 2 : 1;  // slices per unit
   constexpr int UNITS = TL::tokens / (16 * SPU);
-  for (int u = warp; u < UNITS; u += kWarps) {
+#pragma unroll 1
+  for (int u = 0; u < UNITS; ++u) {
     if (u * 16 * SPU >= nvalid) break;
     float acc[SPU][NT][4];
 #pragma unroll
@@ -519,7 +539,7 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
     if (KM == K_BF16) {
       const int tok0 = u * 16;
       const int row = tok0 + (lane & 7) + 8 * ((lane >> 3) & 1);
-      const uint32_t rbase = st_u32 + TL::kc_off + row * 128;
+      const uint32_t rbase = k_u32 + row * 128;
       const int rsw = lane & 7, ch = lane >> 4;  // row % 8; second 8 channels of the k-step
       float acc2[NT][4];
 #pragma unroll
@@ -538,6 +558,7 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
       for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[0][nt][i] += acc2[nt][i];
+      if (TL::SPLIT && !between()) return;
     } else if (KM == K_TOKEN) {
       const int tok0 = u * 16;
       float acc2[NT][4];
@@ -751,14 +772,14 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
           // that 0 * (non-finite) cannot reach the accumulators
           for (int i = lane; i < (tok0 + 16 - nvalid) * 16; i += 32) {
             const int rr = nvalid + (i >> 4), c = i & 15;
-            *reinterpret_cast<uint4*>(const_cast<char*>(st) + TL::vc_off + (c >> 3) * (TL::tokens * 128) +
+            *reinterpret_cast<uint4*>(const_cast<char*>(vst) + TL::vc_off + (c >> 3) * (TL::tokens * 128) +
                                       rr * 128 + (c & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
           }
-          fence_proxy_async_shared();  // the stage is refilled by TMA later
+          fence_proxy_async_shared();  // the slot is refilled by TMA later
           __syncwarp();
         }
         const int row = tok0 + (lane & 7) + 8 * (lane >> 4);
-        const uint32_t rbase = st_u32 + TL::vc_off + row * 128;
+        const uint32_t rbase = v_u32 + row * 128;
         const int rsw = lane & 7, ch = (lane >> 3) & 1;
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) {
@@ -1039,28 +1060,36 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
                                          const uint4 (&qv)[QPieces<NT>::n], int G, float* parts) {
   using TL = Tile<BITS, KM, VM, MB>;
   constexpr int NZ = NZOf<VM>::value;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  // the same in every lane, and known to be: the pipeline's addresses and
+  // branches below are uniform
+  const int warp = __shfl_sync(kFull, tid >> 5, 0);
   const int g = lane >> 2, tq = lane & 3;
   float* q_s = reinterpret_cast<float*>(smem + SmemLayout<NT>::q);
-  char* stages = smem + kStageOff;
-
-  // Every tile that fits the buffer goes in flight before anything else;
-  // later tiles, if any, reuse stages as the ring advances.  Tile i uses stage
-  // i % STAGES and phase i / STAGES of that stage's mbarrier.
-  constexpr int STAGES = TL::stages;
   const float scale_log2 = p.scale_log2;
-  const int n_tiles = (te - tb + TL::tokens - 1) / TL::tokens;
-  const uint32_t st0 = smem_u32(stages);
-  const uint32_t bars = smem_u32(smem + SmemLayout<NT>::bar);
-  volatile int* abort = reinterpret_cast<volatile int*>(smem + SmemLayout<NT>::bar + 8 * kMaxStages);
   constexpr int QV = QPieces<NT>::n;
+
+  // This warp's quarter of the chunk (whole 16-token slices, KIVI-style key
+  // groups) and its pipeline: fill i uses slot i % SLOTS and phase i / SLOTS
+  // of that slot's mbarrier.
+  constexpr int SLOTS = TL::slots, FPT = TL::SPLIT ? 2 : 1;  // fills per tile
+  constexpr int GRAN = (KM == K_KIVI) ? kKiviGroup : 16;
+  const int span = (max(te - tb, 0) + kWarps * GRAN - 1) / (kWarps * GRAN) * GRAN;
+  const int wb = min(tb + warp * span, te), we = min(wb + span, te);
+  const int n_tiles = (max(we - wb, 0) + TL::tokens - 1) / TL::tokens;
+  const int n_fills = n_tiles * FPT;
+  char* buf = smem + kStageOff + warp * kWarpBuf;
+  const uint32_t buf0 = smem_u32(buf);
+  const uint32_t bars = smem_u32(smem + SmemLayout<NT>::bar) + warp * (8 * kMaxSlots);
+  volatile int* abort = reinterpret_cast<volatile int*>(smem + SmemLayout<NT>::bar + 8 * kMaxSlots * kWarps);
   // Only the first tile goes in flight now: with every CTA of the launch
   // starting at once, first tiles alone make a burst the memory system serves
-  // quickly, so compute starts early; the other stages are filled once the
+  // quickly, so compute starts early; the other slots are filled once the
   // first tile has landed.
-  int issued = n_tiles > 0 ? 1 : 0;  // meaningful in thread 0
-  if (tid == 0 && issued)
-    issue_tile<BITS, KM, VM, MB>(st0, bars, sg, tb, min(TL::tokens, te - tb), &p.arena_map);
+  int issued = min(n_fills, FPT);
+  if (elect_one())
+    for (int i = 0; i < issued; ++i)
+      issue_fill<BITS, KM, VM, MB>(buf0 + i * TL::slot_bytes, bars + 8 * i, sg, i, wb, we, &p.arena_map);
 
   // Queries of this KV head's group (fp32, rows >= G zero), rotated for
   // AKVQ-style coded keys.
@@ -1121,35 +1150,62 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
   }
   ws.vb = __uint_as_float(0x00800000u);  // 2^-126: no value scale seen yet
 
-  for (int it = 0; it < n_tiles; ++it) {
-    const int st = it % STAGES;
-    const bool ok = __all_sync(kFull, !*abort && wait_tile(bars + 8 * st, (it / STAGES) & 1, abort, p.status));
-    __syncthreads();
-    if (tid == 0 && !*abort) {
-      // tile 0 landed: fill the other stages; later, refill the stage of tile it - 1
-      const int upto = (it == 0) ? min(n_tiles, STAGES) : min(n_tiles, it + STAGES);
-      if (it > 0 && issued < upto) fence_proxy_async_shared();
-      for (; issued < upto; ++issued)
-        issue_tile<BITS, KM, VM, MB>(st0 + (issued % STAGES) * TL::stage_bytes, bars + 8 * (issued % STAGES), sg,
-                                     tb + issued * TL::tokens, min(TL::tokens, te - tb - issued * TL::tokens),
-                                     &p.arena_map);
+  // Wait for fill f (in slot fs, phase parity fp), then move on to the next.
+  int fs = 0, fp = 0;
+  auto landed = [&]() {
+    if (__all_sync(kFull, mbar_try_wait(bars + 8 * fs, fp))) return true;
+    return (bool)__all_sync(kFull, wait_tile(bars + 8 * fs, fp, abort, p.status));
+  };
+  auto next = [&]() {
+    if (++fs == SLOTS) {
+      fs = 0;
+      fp ^= 1;
     }
-    if (ok)
-      compute_tile<BITS, NT, KM, VM, ROT, MB>(ws, stages + st * TL::stage_bytes,
-                                              min(TL::tokens, te - tb - it * TL::tokens), qb, ql, q_s, s1, s0,
-                                              scale_log2, warp, lane);
+  };
+  // Refill the slot just consumed (every lane has read it).
+  auto refill = [&]() {
+    __syncwarp();
+    if (issued < n_fills) {
+      if (elect_one()) {
+        fence_proxy_async_shared();
+        issue_fill<BITS, KM, VM, MB>(buf0 + fs * TL::slot_bytes, bars + 8 * fs, sg, issued, wb, we, &p.arena_map);
+      }
+      ++issued;
+    }
+    next();
+  };
+#pragma unroll 1
+  for (int it = 0; it < n_tiles; ++it) {
+    if (!landed()) break;
+    if (it == 0) {  // tile 0 landed: fill the other slots
+      const int upto = min(n_fills, SLOTS);
+      if (elect_one())
+        for (int i = issued; i < upto; ++i)
+          issue_fill<BITS, KM, VM, MB>(buf0 + i * TL::slot_bytes, bars + 8 * i, sg, i, wb, we, &p.arena_map);
+      issued = upto;
+    }
+    const char* kst = buf + fs * TL::slot_bytes;
+    const char* vst = TL::SPLIT ? buf + (fs + 1 == SLOTS ? 0 : fs + 1) * TL::slot_bytes : kst;
+    bool ok = true;
+    compute_tile<BITS, NT, KM, VM, ROT, MB>(ws, kst, vst, min(TL::tokens, we - wb - it * TL::tokens), qb, ql, q_s, s1,
+                                            s0, scale_log2, lane, [&]() {
+                                              refill();
+                                              return ok = landed();
+                                            });
+    if (TL::SPLIT && !ok) break;
+    refill();
   }
-  if (tid == 0 && *abort) {
-    // A stage is refilled only after its previous tile landed, so only the
-    // last STAGES tiles can still be in flight: let them land (bounded)
-    // before the buffer is reused or the CTA exits.
-    for (int t = (issued > STAGES ? issued - STAGES : 0); t < issued; ++t)
-      for (uint32_t i = 0; i < kWaitRounds && !mbar_try_wait_sleep(bars + 8 * (t % STAGES), (t / STAGES) & 1,
+  if (*abort && lane == 0) {
+    // A slot is refilled only after its previous fill landed, so only the
+    // last SLOTS fills can still be in flight: let them land (bounded) before
+    // the buffer is reused or the CTA exits.
+    for (int t = (issued > SLOTS ? issued - SLOTS : 0); t < issued; ++t)
+      for (uint32_t i = 0; i < kWaitRounds && !mbar_try_wait_sleep(bars + 8 * (t % SLOTS), (t / SLOTS) & 1,
                                                                     kWaitSleepNs);
            ++i) {
       }
   }
-  __syncthreads();  // stage buffers are reused for the reduction below
+  __syncthreads();  // the warps' buffers are reused for the reduction below
 
   // ---- per-warp results: reduce l and the value-zero terms over the 8 rows g ----
 #pragma unroll
@@ -1248,9 +1304,9 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
   if ((int)blockIdx.x >= p.total_items) return;
   if (threadIdx.x == 0) {
     const uint32_t bars = smem_u32(smem + SmemLayout<NT>::bar);
-    for (int s = 0; s < kMaxStages; ++s) mbar_init(bars + 8 * s, 1);
+    for (int s = 0; s < kMaxSlots * kWarps; ++s) mbar_init(bars + 8 * s, 1);
     mbar_init_fence();
-    *reinterpret_cast<volatile int*>(smem + SmemLayout<NT>::bar + 8 * kMaxStages) = 0;  // abort flag
+    *reinterpret_cast<volatile int*>(smem + SmemLayout<NT>::bar + 8 * kMaxSlots * kWarps) = 0;  // abort flag
     prefetch_tensormap(&p.arena_map);
   }
   int li, b, h, r;

@@ -68,6 +68,14 @@ __device__ __forceinline__ void grid_launch_dependents() {
 }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
+// True in one lane of a converged warp, chosen by the hardware: code under it
+// is known to run once per warp, so its addresses can stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+  return ok != 0;
+}
+
 // Transpose of an 8x8 16-bit matrix held one row-pair per lane.
 __device__ __forceinline__ uint32_t movtrans(uint32_t x) {
   uint32_t y;
