@@ -154,6 +154,9 @@ int sm_count() {
 
 int round_up_to(int x, int g) { return ((x + g - 1) / g) * g; }
 
+// Below this mean cost per resident CTA a launch is latency-bound (seg_bytes).
+constexpr double kLatencyCost = 131072.0;
+
 // Split a segment of len tokens of bpt bytes each into pieces of about
 // item_bytes; returns the chunk size in tokens (a multiple of granule).
 int chunk_tokens(int len, double bpt, double item_bytes, int granule) {
@@ -165,26 +168,39 @@ int chunk_tokens(int len, double bpt, double item_bytes, int granule) {
 }
 
 // Cost per token of each segment kind, in byte-equivalents: the bytes a chunk
-// streams plus a compute term calibrated on measured per-CTA timelines of the
-// decode kernel (a 2-bit coded token costs about 0.6 of a BF16 token's time
-// although it moves 0.16 of its bytes).  Balancing cost rather than bytes
-// keeps compute-heavy coded chunks short.
+// streams plus a compute term.  Balancing cost rather than bytes keeps
+// compute-heavy coded chunks short.
 struct SegBytes {
   double bf16, coded_u, coded_k;
 };
 
-SegBytes seg_bytes(const Dims& d) {
+// latency: a launch whose CTAs hold little more than a tile per warp each.  A
+// chunk then takes as long as its chain of tiles, whatever their bytes, and a
+// coded token costs more than half a BF16 one (calibrated on per-CTA
+// timelines).  Else the warp instructions of the decode kernel per token, at
+// about 8 bytes each: a 16-token slice measured 245 of BF16 rows, 220 of
+// per-token 2-bit codes (255 at 4 bits, rotated), 278 of KIVI-style 2-bit codes
+// with one query per KV head and 770 with more than two.
+SegBytes seg_bytes(const Dims& d, bool latency) {
   SegBytes b;
   const double codes = 16.0 * d.bits;  // 128 codes
   const double pair = (double)meta_pair_bytes(d);
   const double kmeta = d.base == kKivi ? 4.0 * pair : pair;
   const double vmeta = pair * vgroups(d);
-  // compute term per coded token (3-bit: the 2-bit expansion plus its bit-2 plane)
-  const double instr_u = d.base == kKivi ? (d.bits == 2 ? 66.0 : (d.bits == 3 ? 76.0 : 78.0))
-                                         : (d.bits == 2 ? 30.0 : (d.bits == 3 ? 38.0 : 40.0));
-  b.bf16 = 512.0 + 8.0 * 5.0;
-  b.coded_u = 2.0 * codes + kmeta + vmeta + 8.0 * instr_u;
-  b.coded_k = 256.0 + codes + vmeta + 8.0 * 16.0;
+  double instr, bf16, mixed;  // per coded token, BF16 token, BF16 key + coded value
+  if (latency) {
+    instr = d.base == kKivi ? (d.bits == 2 ? 66.0 : (d.bits == 3 ? 76.0 : 78.0))
+                            : (d.bits == 2 ? 30.0 : (d.bits == 3 ? 38.0 : 40.0));
+    bf16 = 5.0;
+    mixed = 16.0;
+  } else {
+    if (d.base == kKivi) instr = d.G <= 2 ? (d.bits == 2 ? 17.0 : 20.0) : (d.bits == 2 ? 48.0 : 55.0);
+    else instr = d.bits == 2 ? 13.5 : 16.0;
+    bf16 = mixed = 15.0;
+  }
+  b.bf16 = 512.0 + 8.0 * bf16;
+  b.coded_u = 2.0 * codes + kmeta + vmeta + 8.0 * instr;
+  b.coded_k = 256.0 + codes + vmeta + 8.0 * mixed;
   return b;
 }
 
@@ -232,73 +248,96 @@ void limit_splits(const Dims& d, DecodePlan* p) {
   }
 }
 
+// The same, growing only the chunks of the heads that have too many.
+void limit_splits_by_kind(const Dims& d, DecodePlan* p) {
+  const int most = decode_max_splits(d.G), nc = ncoded(d);
+  const auto at_most = [](int len, int n) { return round_up_to(cdiv(std::max(len, 1), std::max(n, 1)), 64); };
+  const int text = d.T - nc + d.S_new;
+  p->cbU = std::max(p->cbU, at_most(text, most / 2));
+  const int left = most - cdiv(text, p->cbU);
+  p->cqU = std::max(p->cqU, at_most(nc, left));
+  p->cqK = std::max(p->cqK, at_most(nc, left));
+  p->cbP = std::max(p->cbP, at_most(d.T + d.S_new, most));
+}
+
 size_t plan_ws_bytes(const Dims& d, int count, const DecodePlan& p) {
   return (size_t)ws_bytes(d, count, max_items_of(d, p));
 }
 
-// The work plan of a launch over layers [begin, +count): *one_wave has at most
-// one wave of items (its workspace is the least a launch accepts); the
-// returned plan is the one to run when its workspace is at hand.
-DecodePlan plan_decode(const hg_cache* c, int begin, int count, DecodePlan* one_wave) {
-  const Dims& d = c->d;
-  const SegBytes sb = seg_bytes(d);
-  const HeadCounts hc = head_counts(c, begin, count);
+// Cost of a layer range per CTA of a full wave.
+double mean_cost(const Dims& d, const SegBytes& sb, const HeadCounts& hc, int wave) {
   const double nc = ncoded(d);
   const double head_u = (d.T - nc) * sb.bf16 + nc * sb.coded_u;
   const double head_p = d.keys_only ? (d.T - nc) * sb.bf16 + nc * sb.coded_k : d.T * sb.bf16;
-  const double total = d.B * (hc.unprot * head_u + hc.prot * head_p);
-  const int wave = (d.G <= 8 ? 4 : 2) * sm_count();
-  const double mean = total / wave;
-  double item = std::max(mean, 16384.0);
-  // Grow the item size until the items (at the largest appended count) fit
-  // one wave, or every segment is a single chunk.
+  return d.B * (hc.unprot * head_u + hc.prot * head_p) / wave;
+}
+
+// Chunks of at least `item` cost, grown until the items (at the largest
+// appended count) fit one wave or every segment is a single chunk.
+DecodePlan one_wave_plan(const Dims& d, const SegBytes& sb, const HeadCounts& hc, int wave, double item) {
   DecodePlan p;
   for (int iter = 0; iter < 64; ++iter, item *= 1.05) {
     p = plan_for(d, sb, item);
     const ChunkCounts cc = counts_of(d, d.S_new, p);
     int nb;
-    const long long items = (long long)d.B * ((long long)hc.unprot * head_chunks(kQuantized, cc, &nb) +
-                                              (long long)hc.prot * head_chunks(d.keys_only ? kKeysOnly : kProtected, cc, &nb));
-    if (items <= wave) break;
+    const long long per_row = (long long)hc.unprot * head_chunks(kQuantized, cc, &nb) +
+                              (long long)hc.prot * head_chunks(d.keys_only ? kKeysOnly : kProtected, cc, &nb);
+    if (d.B * per_row <= wave) break;
     if (p.cbU >= d.T - ncoded(d) + d.S_new && p.cqU >= ncoded(d) && p.cqK >= ncoded(d) &&
         p.cbP >= d.T + d.S_new)
       break;
   }
-  limit_splits(d, &p);
-  if (one_wave) *one_wave = p;
+  return p;
+}
+
+// The work plan of a launch over layers [begin, +count), and in *least the
+// plan with the least workspace a launch accepts, which runs when the caller's
+// holds no more.
+DecodePlan plan_decode(const hg_cache* c, int begin, int count, DecodePlan* least) {
+  const Dims& d = c->d;
+  const HeadCounts hc = head_counts(c, begin, count);
+  const int wave = (d.G <= 8 ? 4 : 2) * sm_count();
+  const SegBytes lat = seg_bytes(d, true), thr = seg_bytes(d, false);
+  DecodePlan p = one_wave_plan(d, lat, hc, wave, std::max(mean_cost(d, lat, hc, wave), 16384.0));
+  *least = p;
+  limit_splits(d, least);
+  const double mean = mean_cost(d, thr, hc, wave);
+  if (mean < kLatencyCost) {
+    limit_splits_by_kind(d, &p);
+    return p;
+  }
+  p = one_wave_plan(d, thr, hc, wave, mean);
   // One wave balances only when the heads cut into pieces of about the mean
   // cost per resident CTA.  When whole segments are as large as that (a layer
   // of a large batch: 256 heads over 608 CTAs), the rounding leaves chunks of
   // up to twice the mean, and the launch lasts as long as they do.  Then
   // pieces of half the mean run as two to three waves instead, costliest
-  // first: one layer of 32 rows, 8 KV heads and 8,576 tokens, 150 -> 90 us (96
-  // and 91 us at 2/3 and 1/3 of the mean); 3,520 tokens of 4-bit rotated keys,
-  // 84 -> 53 us (53, 58).  Chunks under 256 KB keep one wave: a
-  // CTA's start and merge (about 8 us) outweigh the balance there (28 layers
-  // of 4 heads: 15.3 us a step in one wave, 18.1 with pieces of 2/3).
+  // first: one layer of 32 rows, 8 KV heads and 8,576 tokens 150 -> 90 us (96
+  // and 91 us at 2/3 and 1/3 of the mean); 3,520 tokens of 4-bit rotated keys
+  // 84 -> 53 us (53, 58).  Chunks under 256 KB keep one wave: a CTA's start
+  // and merge (about 8 us) outweigh the balance there (28 layers of 4 heads:
+  // 15.3 us a step in one wave, 18.1 with pieces of 2/3).
   double worst = 0;
-  if (hc.unprot || d.keys_only) worst = std::min(p.cbU, d.T - ncoded(d)) * sb.bf16;
-  if (hc.unprot) worst = std::max(worst, std::min(p.cqU, ncoded(d)) * sb.coded_u);
+  if (hc.unprot || d.keys_only) worst = std::min(p.cbU, d.T - ncoded(d)) * thr.bf16;
+  if (hc.unprot) worst = std::max(worst, std::min(p.cqU, ncoded(d)) * thr.coded_u);
   if (hc.prot)
-    worst = std::max(worst, d.keys_only ? std::min(p.cqK, ncoded(d)) * sb.coded_k : std::min(p.cbP, d.T) * sb.bf16);
-  if (mean > 262144.0 && worst > 1.15 * mean) {
-    p = plan_for(d, sb, mean / 2);
-    limit_splits(d, &p);
-  }
+    worst = std::max(worst, d.keys_only ? std::min(p.cqK, ncoded(d)) * thr.coded_k : std::min(p.cbP, d.T) * thr.bf16);
+  if (mean > 262144.0 && worst > 1.15 * mean) p = plan_for(d, thr, mean / 2);
+  limit_splits_by_kind(d, &p);
   return p;
 }
 
 // Least workspace a launch accepts / workspace of the plan it then runs with.
 size_t ws_least_for(const hg_cache* c, int begin, int count) {
-  DecodePlan one;
-  plan_decode(c, begin, count, &one);
-  return plan_ws_bytes(c->d, count, one);
+  DecodePlan least;
+  plan_decode(c, begin, count, &least);
+  return plan_ws_bytes(c->d, count, least);
 }
 
 size_t ws_size_for(const hg_cache* c, int begin, int count) {
-  DecodePlan one;
-  const DecodePlan p = plan_decode(c, begin, count, &one);
-  return std::max(plan_ws_bytes(c->d, count, one), plan_ws_bytes(c->d, count, p));
+  DecodePlan least;
+  const DecodePlan p = plan_decode(c, begin, count, &least);
+  return std::max(plan_ws_bytes(c->d, count, least), plan_ws_bytes(c->d, count, p));
 }
 
 // A launch over more than kMaxLayersPerLaunch layers reuses the workspace for
@@ -600,7 +639,7 @@ namespace {
 // mostly on the same one, so the kernel takes the items in rounds of one per
 // SM, every other round reversed: each SM gets a mix of large and small items.
 int fill_runs(const Dims& d, const HeadCounts& hc, DecodeParams* p) {
-  const SegBytes sb = seg_bytes(d);
+  const SegBytes sb = seg_bytes(d, mean_cost(d, seg_bytes(d, false), hc, (d.G <= 8 ? 4 : 2) * sm_count()) < kLatencyCost);
   struct Run {
     double cost;
     int kind, heads, chunks;
@@ -643,9 +682,9 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     p.d = d;
     p.arena = c->arena;
     p.n_layers = n;
-    DecodePlan one_wave;
-    p.plan = plan_decode(c, layer_begin + done, n, &one_wave);
-    if (plan_ws_bytes(d, n, p.plan) > ws_bytes_given) p.plan = one_wave;
+    DecodePlan least;
+    p.plan = plan_decode(c, layer_begin + done, n, &least);
+    if (plan_ws_bytes(d, n, p.plan) > ws_bytes_given) p.plan = least;
     p.max_items = max_items_of(d, p.plan);
     p.scale_log2 = scale * 1.4426950408889634f;
     p.q = static_cast<const uint16_t*>(q) + (size_t)done * layer_elems;

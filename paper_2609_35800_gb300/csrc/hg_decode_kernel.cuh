@@ -14,21 +14,29 @@
 // one bulk copy per array.  The warps meet only before their first tile and
 // after their last one.  A warp works on 16-token slices and computes, with
 // mma.sync m16n8k16 (BF16 in, fp32 accumulate):
-//   S^T[token][query] = K . q     A = keys (BF16 via ldmatrix, or codes
-//                                 expanded exactly to BF16 in registers),
+//   S^T[token][query] = K . q     A = keys (BF16 via ldmatrix, or codes masked
+//                                 in registers),
 //                                 B = the G queries of the KV head (padded to 8)
 //   O^T[chan][query] += V^T . P^T A = values (ldmatrix.trans, or codes),
 //                                 B = P^T, transposed from the score fragment
 //                                 with movmatrix.
+// Codes enter the MMAs as FP16 bit patterns: an integer i < 2^11 in the low
+// bits is exactly i 2^-24 (a subnormal, or the binade above them, which
+// continues the same steps), so a masked word is an operand as it is -- no
+// offset to add and remove again, no subtraction -- and a code may sit at any of
+// the low bit positions, where it counts 2^position times.  The position's
+// factor is taken out of the other operand or of the result; 2^24 of the result.
 // Coded keys are contracted in the code domain: with per-token groups
-// k^_d = s c_d + z, so q.k^ = s (q.c) + z sum(q); the key codes enter the MMA
-// as the exact BF16 values 128 + c (no subtraction), and the 128 sum(q) offset
-// is removed in the fp32 epilogue; KIVI-style per-channel
-// groups fold the channel scale into the query (q~_d = q_d s_d, split into a
-// BF16 hi + lo pair) and add sum_d q_d z_d.  Values fold the token scale into
-// P (p s) and add sum_t p_t z_t.  AKVQ-style keys are coded in the rotated
-// domain; since the normalised Hadamard matrix is symmetric and orthonormal,
-// <q, H k'> = <H q, k'>, so the query is rotated once per CTA (hi + lo split).
+// k^_d = s c_d + z, so q.k^ = s (q.c) + z sum(q), with the query row scaled by
+// a power of two into FP16's range (exact).  KIVI-style per-channel groups fold
+// the channel scale into the query (q~_d = q_d s_d, split into a hi + lo pair)
+// and add sum_d q_d z_d.  Values fold the token scale into P (p s) and add
+// sum_t p_t z_t.  (KIVI-style codes with more than two queries per KV head are
+// converted to BF16 keys and FP16 values instead: their pairs sit at bit
+// positions that differ between lanes.)  AKVQ-style keys are coded in the
+// rotated domain; since the normalised Hadamard matrix is symmetric and
+// orthonormal, <q, H k'> = <H q, k'>, so the query is rotated once per CTA (hi +
+// lo split).
 //
 // The online softmax rescales its accumulators only when a running maximum
 // grows by more than 2^8 (probabilities stay <= 256 before normalisation).
@@ -71,7 +79,8 @@ template <int NT>
 struct SmemLayout {
   static constexpr int q = kStageOff + kBufBytes;  // float q[NT * 8][kQRow] (qidx)
   static constexpr int bar = q + NT * 8 * kQRow * 4;  // mbarrier per warp and slot (4 x 4), abort flag
-  static constexpr int bytes = bar + 192 + 1024;   // + alignment slack
+  static constexpr int qn = bar + 192;              // float qn[NT * 8]: scale of each staged query row
+  static constexpr int bytes = qn + 64 + 1024;     // + alignment slack
 };
 constexpr int kMaxSlots = 4;  // per warp
 constexpr unsigned kFull = 0xffffffffu;
@@ -108,26 +117,28 @@ struct Seg {
 template <int BITS>
 __host__ __device__ constexpr uint32_t pair_mask() { return ((1u << BITS) - 1u) * 0x00010001u; }
 
-template <int BITS>
-__device__ __forceinline__ uint32_t pair2(uint32_t x) {  // codes at bits [0,b) and [16,16+b)
-  return codes_bf16x2(x & pair_mask<BITS>());
-}
+// Result of an MMA over codes, in units of 2^-24 (see the file comment).
+constexpr float kCodeUnit = 16777216.f;
 
-// The same pair as the BF16 values (128 + code): exact, without the subtraction.
+// A word (half) of packed codes holds pairs (j, j + half a word) 16 bits apart.
+// Pair j as an MMA operand register: masked at bit code_pos(j) and 16 above,
+// after one of three shifts (2-bit codes, and the 2-bit part of 3-bit codes) or
+// two (4 bits).  The values are 2^code_pos(j) times the codes.  The positions
+// are the high ones of the 11 bits: the tensor cores line an operand's products
+// up by its exponent field, so a code in the lowest bits would lose as many
+// bits of the sum as it has leading zeros (with positions 0..8 in one shift per
+// five pairs, KIVI-style values moved 1% away from the 64-bit result).
 template <int BITS>
-__device__ __forceinline__ uint32_t pair2_off(uint32_t x) {
-  return (x & pair_mask<BITS>()) | 0x43004300u;
-}
-
-// FP16 forms for value codes: exact codes, and 1024 + code.
-template <int BITS>
-__device__ __forceinline__ uint32_t pair2_h(uint32_t x) {
-  return codes_f16x2(x & pair_mask<BITS>());
+__host__ __device__ constexpr int code_pos(int j) {
+  return BITS == 4 ? 4 * (j % 2) : (j < 2 ? 2 * j + 6 : (j < 5 ? 2 * j : 2 * j - 6));
 }
 template <int BITS>
-__device__ __forceinline__ uint32_t pair2_off_h(uint32_t x) {
-  return (x & pair_mask<BITS>()) | 0x64006400u;
+__device__ __forceinline__ uint32_t code_pair(uint32_t w, int j) {
+  const uint32_t x = BITS == 4 ? w >> (8 * (j / 2)) : (j < 2 ? w << 6 : (j < 5 ? w : w >> 6));
+  return x & (pair_mask<BITS == 4 ? 4 : 2>() << code_pos<BITS>(j));
 }
+template <int BITS>
+__host__ __device__ constexpr float code_unit(int j) { return 1.0f / (float)(1 << code_pos<BITS>(j)); }
 
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
@@ -138,28 +149,11 @@ __device__ __forceinline__ float fast_exp2(float x) {
 template <int NT, int NZ>
 struct WarpState {
   float o[NT][8][4];
-  float corr[NT][4];  // 1024 * sum_t P'^T[t][q] for value codes carried as 1024 + c
   float vb;           // coded values: power-of-two bound of the value scales seen so far
   float m[NT][2];
   float l[NT][2];
   float z[NT][2][NZ];
 };
-
-// 2-bit codes of one word sit in pairs (j, j + 8) at bits (2j, 2j + 16).  Pair j
-// is taken from (w >> 6 * (j / 3)) masked at bit 2 * (j % 3): that yields
-// 4^(j % 3) * code, which stays inside the 7-bit BF16 mantissa of 128 + x, and
-// costs one shift per three pairs.  The factor is removed where it is exact
-// (a power of two on the other MMA operand or on the accumulator).
-__device__ __forceinline__ int pos3(int j) { return 2 * (j % 3); }
-__device__ __forceinline__ uint32_t pair2_scaled(uint32_t w, uint32_t w6, uint32_t w12, int j) {
-  const uint32_t src = j < 3 ? w : (j < 6 ? w6 : w12);
-  return (src & (0x00030003u << pos3(j))) | 0x43004300u;
-}
-// The same pair as the FP16 values 1024 + 4^(j % 3) * code (value codes).
-__device__ __forceinline__ uint32_t pair2_scaled_h(uint32_t w, uint32_t w6, uint32_t w12, int j) {
-  const uint32_t src = j < 3 ? w : (j < 6 ? w6 : w12);
-  return (src & (0x00030003u << pos3(j))) | 0x64006400u;
-}
 
 // 1 / x for a power of two x in [2^-126, 2^126], exactly (exponent arithmetic).
 __device__ __forceinline__ float pow2_inv(float x) { return __uint_as_float(0x7F000000u - __float_as_uint(x)); }
@@ -180,6 +174,10 @@ __device__ __forceinline__ uint32_t plane_pair(uint32_t pl, int i, int p) {
 __device__ __forceinline__ uint32_t plane_sel(int bs) {
   return (uint32_t)(bs | (bs << 4) | ((4 + bs) << 8) | ((4 + bs) << 12));
 }
+
+// Bounds of the power-of-two scales: their products and inverses stay finite.
+constexpr float kScaleLow = 7.8886090522101181e-31f;  // 2^-100
+constexpr float kScaleTop = 8.5070591730234616e37f;   // 2^126
 
 // Smallest power of two >= m (m > 0, finite).
 __device__ __forceinline__ float pow2_ceil(float m) {
@@ -231,10 +229,14 @@ __device__ __forceinline__ void meta_quad(const char* base, int i, float2 (&m)[4
 // that layer 90 -> 84 us, 3,520 tokens of 4-bit rotated keys 53 -> 50 us,
 // 32 KV heads of KIVI-style codes in 16 rows 123 -> 109 us, one row of 4 KV
 // heads and 1,460 tokens 9.4 -> 8.1 us.
-template <int BITS, int KM, int VM, int MB>
+//
+// COLS (run_item_cols): SPLIT as well, two KIVI-style groups per tile (K and V
+// 4 KB each at 2 bits), or 16 tokens of BF16 keys and KIVI-style values.
+template <int BITS, int KM, int VM, int MB, bool COLS = false>
 struct Tile {
-  static constexpr bool SPLIT = KM == K_BF16 && VM == V_BF16;
-  static constexpr int tokens = (KM == K_BF16) ? 16 : (KM == K_KIVI ? kKiviGroup : (BITS == 2 ? 64 : 32));
+  static constexpr bool SPLIT = COLS || (KM == K_BF16 && VM == V_BF16);
+  static constexpr int tokens = (KM == K_BF16) ? 16
+                                : (KM == K_KIVI ? (COLS ? 2 : 1) * kKiviGroup : (BITS == 2 ? 64 : 32));
   static constexpr int kc_bytes = (KM == K_BF16) ? tokens * 256 : tokens * 16 * BITS;
   static constexpr int km_bytes = (KM == K_TOKEN) ? tokens * MB : (KM == K_KIVI ? tokens * 4 * MB : 0);
   static constexpr int vc_bytes = (VM == V_BF16) ? tokens * 256 : tokens * 16 * BITS;
@@ -244,7 +246,8 @@ struct Tile {
   static constexpr int vm_off = vc_off + vc_bytes;
   // slots that hold BF16 rows start on 1024-byte boundaries (swizzled boxes)
   static constexpr int align = (KM == K_BF16) ? 1024 : 128;
-  static constexpr int slot_bytes = ((SPLIT ? kc_bytes : vm_off + vm_bytes) + align - 1) / align * align;
+  static constexpr int k_end = kc_bytes + km_bytes, v_end = vm_off + vm_bytes;
+  static constexpr int slot_bytes = ((k_end > v_end ? k_end : v_end) + align - 1) / align * align;
   static constexpr int slots = (kWarpBuf / slot_bytes) > kMaxSlots ? kMaxSlots : (kWarpBuf / slot_bytes);
   static_assert(slots >= 2, "a tile must fit twice in a warp's buffer");
   static_assert(KM != K_BF16 || tokens == kArenaBoxRows, "a BF16 tile is one TMA box high");
@@ -266,16 +269,17 @@ __device__ __forceinline__ void issue_rows(uint32_t dst, const CUtensorMap* map,
 // tile t.  Packed codes and metadata arrive as one bulk copy per array
 // (metadata rounded up to 16 bytes: the arena pads every metadata row to 16
 // bytes); bytes past the range [wb, we) are left stale.
-template <int BITS, int KM, int VM, int MB>
+template <int BITS, int KM, int VM, int MB, bool COLS>
 __device__ __forceinline__ void issue_fill(uint32_t slot, uint32_t bar, const Seg& sg, int i, int wb, int we,
                                            const CUtensorMap* map) {
-  using TL = Tile<BITS, KM, VM, MB>;
+  using TL = Tile<BITS, KM, VM, MB, COLS>;
   const int t0 = wb + (TL::SPLIT ? i >> 1 : i) * TL::tokens;
-  if (TL::SPLIT) {
+  if (KM == K_BF16 && VM == V_BF16) {
     mbar_arrive_expect_tx(bar, TL::kc_bytes);
     issue_rows(slot, map, ((i & 1) ? sg.v_row0 : sg.k_row0) + t0, bar);
     return;
   }
+  const bool do_k = !TL::SPLIT || !(i & 1), do_v = !TL::SPLIT || (i & 1);
   constexpr int kmb = (KM == K_TOKEN) ? MB : 4 * MB;  // metadata bytes per token
   constexpr int vmb = (VM == V_TOKEN) ? MB : 4 * MB;
   const int n = min(TL::tokens, we - t0);
@@ -283,15 +287,19 @@ __device__ __forceinline__ void issue_fill(uint32_t slot, uint32_t bar, const Se
   const uint32_t km_bytes = (KM == K_BF16) ? 0u : (uint32_t)((n * kmb + 15) & ~15);
   const uint32_t vc_bytes = n * 16 * BITS;
   const uint32_t vm_bytes = (uint32_t)((n * vmb + 15) & ~15);
-  mbar_arrive_expect_tx(bar, kc_bytes + km_bytes + vc_bytes + vm_bytes);
-  if (KM == K_BF16) {
-    issue_rows(slot, map, sg.k_row0 + t0, bar);
-  } else {
-    bulk_g2s(slot, sg.kc + (size_t)t0 * 16 * BITS, kc_bytes, bar);
-    bulk_g2s(slot + TL::km_off, sg.km + (size_t)t0 * kmb, km_bytes, bar);
+  mbar_arrive_expect_tx(bar, (do_k ? kc_bytes + km_bytes : 0u) + (do_v ? vc_bytes + vm_bytes : 0u));
+  if (do_k) {
+    if (KM == K_BF16) {
+      issue_rows(slot, map, sg.k_row0 + t0, bar);
+    } else {
+      bulk_g2s(slot, sg.kc + (size_t)t0 * 16 * BITS, kc_bytes, bar);
+      bulk_g2s(slot + TL::km_off, sg.km + (size_t)t0 * kmb, km_bytes, bar);
+    }
   }
-  bulk_g2s(slot + TL::vc_off, sg.vc + (size_t)t0 * 16 * BITS, vc_bytes, bar);
-  bulk_g2s(slot + TL::vm_off, sg.vm + (size_t)t0 * vmb, vm_bytes, bar);
+  if (do_v) {
+    bulk_g2s(slot + TL::vc_off, sg.vc + (size_t)t0 * 16 * BITS, vc_bytes, bar);
+    bulk_g2s(slot + TL::vm_off, sg.vm + (size_t)t0 * vmb, vm_bytes, bar);
+  }
 }
 
 // Bounded wait for a phase of a slot's mbarrier.  On timeout, or once another
@@ -308,9 +316,102 @@ __device__ __forceinline__ bool wait_tile(uint32_t bar, uint32_t parity, volatil
   return false;
 }
 
+// A warp's pipeline over its token range [wb, we): fill i uses slot i % SLOTS
+// and phase i / SLOTS of that slot's mbarrier; fills are consumed in order.
+template <int BITS, int NT, int KM, int VM, int MB, bool COLS>
+struct WarpPipe {
+  using TL = Tile<BITS, KM, VM, MB, COLS>;
+  static constexpr int SLOTS = TL::slots, FPT = TL::SPLIT ? 2 : 1;  // fills per tile
+  const Seg& sg;
+  const DecodeParams& p;
+  int wb, we, n_tiles, n_fills, issued;
+  int fs, fp;  // slot and phase parity of the next fill to consume
+  char* buf;
+  uint32_t buf0, bars;
+  volatile int* abort;
+
+  // The warp's quarter of the chunk [tb, te), in whole units of GRAN tokens.
+  // Only the first tile goes in flight now: with every CTA of the launch
+  // starting at once, first tiles alone make a burst the memory system serves
+  // quickly, so compute starts early; the other slots are filled once the
+  // first tile has landed.  (Filling them all at once measured the same, also
+  // in launches of a few dozen CTAs.)
+  __device__ __forceinline__ WarpPipe(char* smem, int warp, const Seg& s, const DecodeParams& dp, int tb, int te,
+                                      int gran)
+      : sg(s), p(dp), fs(0), fp(0) {
+    const int span = (max(te - tb, 0) + kWarps * gran - 1) / (kWarps * gran) * gran;
+    wb = min(tb + warp * span, te);
+    we = min(wb + span, te);
+    n_tiles = (max(we - wb, 0) + TL::tokens - 1) / TL::tokens;
+    n_fills = n_tiles * FPT;
+    buf = smem + kStageOff + warp * kWarpBuf;
+    buf0 = smem_u32(buf);
+    bars = smem_u32(smem + SmemLayout<NT>::bar) + warp * (8 * kMaxSlots);
+    abort = reinterpret_cast<volatile int*>(smem + SmemLayout<NT>::bar + 8 * kMaxSlots * kWarps);
+    issued = min(n_fills, FPT);
+    if (elect_one())
+      for (int i = 0; i < issued; ++i) issue(i, i);
+  }
+  __device__ __forceinline__ void issue(int slot, int i) {
+    issue_fill<BITS, KM, VM, MB, COLS>(buf0 + slot * TL::slot_bytes, bars + 8 * slot, sg, i, wb, we, &p.arena_map);
+  }
+  __device__ __forceinline__ int tile_tokens(int it) const { return min(TL::tokens, we - wb - it * TL::tokens); }
+  __device__ __forceinline__ const char* slot() const { return buf + fs * TL::slot_bytes; }
+  __device__ __forceinline__ const char* next_slot() const {
+    return buf + (fs + 1 == SLOTS ? 0 : fs + 1) * TL::slot_bytes;
+  }
+  // Wait for the next fill; false when a wait of the CTA ran out.
+  __device__ __forceinline__ bool landed() {
+    if (__all_sync(kFull, mbar_try_wait(bars + 8 * fs, fp))) return true;
+    return (bool)__all_sync(kFull, wait_tile(bars + 8 * fs, fp, abort, p.status));
+  }
+  // The first tile landed: fill the other slots.
+  __device__ __forceinline__ void fill_rest() {
+    const int upto = min(n_fills, SLOTS);
+    if (elect_one())
+      for (int i = issued; i < upto; ++i) issue(i, i);
+    issued = upto;
+  }
+  // Every lane has read the consumed fill: refill its slot and move on.
+  __device__ __forceinline__ void refill() {
+    __syncwarp();
+    if (issued < n_fills) {
+      if (elect_one()) {
+        fence_proxy_async_shared();
+        issue(fs, issued);
+      }
+      ++issued;
+    }
+    if (++fs == SLOTS) {
+      fs = 0;
+      fp ^= 1;
+    }
+  }
+  // After a wait ran out: a slot is refilled only after its previous fill
+  // landed, so only the last SLOTS fills can still be in flight; let them land
+  // (bounded) before the buffer is reused or the CTA exits.
+  __device__ __forceinline__ void drain(int lane) {
+    if (*abort && lane == 0) {
+      for (int t = (issued > SLOTS ? issued - SLOTS : 0); t < issued; ++t)
+        for (uint32_t i = 0; i < kWaitRounds && !mbar_try_wait_sleep(bars + 8 * (t % SLOTS), (t / SLOTS) & 1,
+                                                                      kWaitSleepNs);
+             ++i) {
+        }
+    }
+  }
+};
+
 // ---------------------------------------------------------------------------
 // Query fragments
 // ---------------------------------------------------------------------------
+// hi + lo FP16 split of an fp32 pair below FP16's largest value (x = hi + lo to
+// 22 significant bits, 2^-25 at least)
+__device__ __forceinline__ void split_pair16(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+  hi = pack_half2(x0, x1);
+  const float2 h = half2_bits_to_float2(hi);
+  lo = pack_half2(x0 - h.x, x1 - h.y);
+}
+
 // hi + lo BF16 split of an fp32 pair (x = hi + lo to ~16 significant bits)
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
   hi = pack_bf16x2(x0, x1);
@@ -353,52 +454,38 @@ __device__ __forceinline__ void token_channels(int tq, int j, int (&c)[4]) {
   }
 }
 
-// Query fragments for coded per-token keys.  2-bit: k-step j carries q / 4^(j % 3)
-// to match the scaled key pairs.  Also returns, per query column of this
-// thread, s1 = sum of the fragment values as the MMA sees them (for removing
-// the 128 offset of the key codes) and s0 = sum of the unscaled queries.
+// Query fragments (FP16) for coded per-token keys from the staged, scaled rows:
+// k-step j's k-slots carry q times the unit of the codes they meet.  Rotated
+// queries are not BF16 values any more and take a hi + lo pair; the others are
+// exact in one.  s0 = sum of the (scaled) query of this thread's columns.
 template <int BITS, int NT, bool ROT>
 __device__ __forceinline__ void qfrag_token(uint32_t (&qb)[NT][8][2], uint32_t (&ql)[NT][8][2],
-                                            float (&s1)[NT][2], float (&s0)[NT][2],
-                                            const float* q_s, int g, int tq) {
+                                            float (&s0)[NT][2], const float* q_s, int g, int tq) {
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
     const int r = nt * 8 + g;
-    float a1 = 0.f, a0 = 0.f;
+    float a0 = 0.f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       int c[4];
       token_channels<BITS>(tq, j, c);
-      const float f = (BITS != 4) ? 1.0f / (float)(1 << pos3(j)) : 1.0f;  // exact
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
-        const float x0 = q_s[qidx(r, c[2 * hh])] * f, x1 = q_s[qidx(r, c[2 * hh + 1])] * f;
-        uint32_t hi, lo = 0u;
+        const float f = code_unit<BITS>(BITS == 4 ? hh : j);
+        const float x0 = q_s[qidx(r, c[2 * hh])], x1 = q_s[qidx(r, c[2 * hh + 1])];
+        a0 += x0 + x1;
         if (ROT) {
-          split_pair(x0, x1, hi, lo);
+          split_pair16(x0 * f, x1 * f, qb[nt][j][hh], ql[nt][j][hh]);
         } else {
-          hi = pack_bf16x2(x0, x1);  // exact: the queries are BF16
+          qb[nt][j][hh] = pack_half2(x0 * f, x1 * f);
         }
-        qb[nt][j][hh] = hi;
-        ql[nt][j][hh] = lo;
-        float h0, h1, l0, l1;
-        bf16x2_to_f32(hi, h0, h1);
-        bf16x2_to_f32(lo, l0, l1);
-        const float part = (h0 + l0) + (h1 + l1);
-        a1 += part;
-        a0 += part * (1.0f / f);
       }
     }
-    // totals for query g, then the values of this thread's columns 2tq, 2tq+1
-    a1 += __shfl_xor_sync(kFull, a1, 1);
-    a1 += __shfl_xor_sync(kFull, a1, 2);
+    // the total for query g, then the values of this thread's columns 2tq, 2tq+1
     a0 += __shfl_xor_sync(kFull, a0, 1);
     a0 += __shfl_xor_sync(kFull, a0, 2);
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      s1[nt][e] = __shfl_sync(kFull, a1, (2 * tq + e) << 2);
-      s0[nt][e] = __shfl_sync(kFull, a0, (2 * tq + e) << 2);
-    }
+    for (int e = 0; e < 2; ++e) s0[nt][e] = __shfl_sync(kFull, a0, (2 * tq + e) << 2);
   }
 }
 
@@ -434,8 +521,6 @@ __device__ __forceinline__ void softmax_update(WarpState<NT, NZ>& ws, float (&sc
           ws.o[nt][mt][e] *= a;
           ws.o[nt][mt][2 + e] *= a;
         }
-        ws.corr[nt][e] *= a;
-        ws.corr[nt][2 + e] *= a;
       }
     }
   }
@@ -478,6 +563,67 @@ __device__ __forceinline__ void pfrag16(const float (&p)[4], float fg, float fg8
   b[1] = movtrans(pack_half2(p[2] * fg8, p[3] * fg8));
 }
 
+// O^T += V^T . P^T over one slice of coded values in channel order: tokens ta,
+// tb (k-slots 2tq, 2tq + 1) and tc, td (2tq + 8, 2tq + 9) of this lane.  M-tile
+// mt's rows g and g + 8 are channels 16g + mt and 16g + 8 + mt, in units of
+// code_unit(mt) 2^24 (4 bits: of m-tile mt % 4).
+template <int BITS, int NT>
+__device__ __forceinline__ void pv_codes(float (&o)[NT][8][4], const uint32_t* vc32, int ta, int tb, int tc, int td,
+                                         int g, const uint32_t (&b)[NT][2]) {
+  const int t[4] = {ta, tb, tc, td};
+  if (BITS != 4) {
+    // word g of a token row holds channels 16g..16g+15
+    constexpr int RW = 4 * BITS;  // words per token row
+    const uint32_t w0 = vc32[t[0] * RW + g], w1 = vc32[t[1] * RW + g];
+    const uint32_t w8 = vc32[t[2] * RW + g], w9 = vc32[t[3] * RW + g];
+    const uint32_t x[4] = {prmt(w0, w1, 0x5410), prmt(w0, w1, 0x7632), prmt(w8, w9, 0x5410),
+                           prmt(w8, w9, 0x7632)};
+    // 3 bits: bit 2 of word g's codes 0-7 is byte g % 2 of plane word
+    // 8 + g / 2, codes 8-15 byte 2 + g % 2; two tokens side by side
+    uint32_t hp[4] = {0u, 0u, 0u, 0u};
+    if (BITS == 3) {
+      const int pw = 8 + (g >> 1), bs = g & 1;
+      const uint32_t p0 = vc32[t[0] * RW + pw], p1 = vc32[t[1] * RW + pw];
+      const uint32_t p8 = vc32[t[2] * RW + pw], p9 = vc32[t[3] * RW + pw];
+      hp[0] = prmt(p0, p1, plane_sel(bs));
+      hp[1] = prmt(p0, p1, plane_sel(2 + bs));
+      hp[2] = prmt(p8, p9, plane_sel(bs));
+      hp[3] = prmt(p8, p9, plane_sel(2 + bs));
+    }
+#pragma unroll
+    for (int mt = 0; mt < 8; ++mt) {
+      uint32_t a[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        a[k] = code_pair<BITS>(x[k], mt);
+        if (BITS == 3) a[k] |= plane_pair(hp[k], mt, code_pos<BITS>(mt));
+      }
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) mma_f16(o[nt][mt], a, b[nt][0], b[nt][1]);
+    }
+  } else {
+    // word 2g holds channels 16g..16g+7 (codes 0-3 low half, 4-7 high), 2g+1 the next 8
+    const uint2 v0 = *reinterpret_cast<const uint2*>(vc32 + t[0] * 16 + 2 * g);
+    const uint2 v1 = *reinterpret_cast<const uint2*>(vc32 + t[1] * 16 + 2 * g);
+    const uint2 v8 = *reinterpret_cast<const uint2*>(vc32 + t[2] * 16 + 2 * g);
+    const uint2 v9 = *reinterpret_cast<const uint2*>(vc32 + t[3] * 16 + 2 * g);
+    const uint32_t xa = prmt(v0.x, v1.x, 0x5410), ya = prmt(v0.x, v1.x, 0x7632);
+    const uint32_t xb = prmt(v0.y, v1.y, 0x5410), yb = prmt(v0.y, v1.y, 0x7632);
+    const uint32_t xc = prmt(v8.x, v9.x, 0x5410), yc = prmt(v8.x, v9.x, 0x7632);
+    const uint32_t xd = prmt(v8.y, v9.y, 0x5410), yd = prmt(v8.y, v9.y, 0x7632);
+#pragma unroll
+    for (int mt = 0; mt < 8; ++mt) {
+      uint32_t a[4];
+      a[0] = code_pair<4>(mt < 4 ? xa : ya, mt & 3);
+      a[1] = code_pair<4>(mt < 4 ? xb : yb, mt & 3);
+      a[2] = code_pair<4>(mt < 4 ? xc : yc, mt & 3);
+      a[3] = code_pair<4>(mt < 4 ? xd : yd, mt & 3);
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) mma_f16(o[nt][mt], a, b[nt][0], b[nt][1]);
+    }
+  }
+}
+
 template <int NT, int NZ>
 __device__ __forceinline__ void vscale_update(WarpState<NT, NZ>& ws, float smax) {
   if (__any_sync(kFull, smax > ws.vb)) {
@@ -489,8 +635,6 @@ __device__ __forceinline__ void vscale_update(WarpState<NT, NZ>& ws, float smax)
       for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
         for (int i = 0; i < 4; ++i) ws.o[nt][mt][i] *= a;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) ws.corr[nt][i] *= a;
     }
     ws.vb = nb;
   }
@@ -505,7 +649,7 @@ template <int BITS, int NT, int KM, int VM, bool ROT, int MB, class F>
 __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws, const char* kst, const char* vst,
                                              int nvalid, const uint32_t (&qb)[NT][8][2],
                                              const uint32_t (&ql)[NT][8][2], const float* q_s,
-                                             const float (&s1)[NT][2], const float (&s0)[NT][2],
+                                             const float (&kq)[NT][2], const float (&s0)[NT][2],
                                              float scale_log2, int lane, F&& between) {
   using TL = Tile<BITS, KM, VM, MB>;
   constexpr int NZ = NZOf<VM>::value;
@@ -581,25 +725,19 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
           pl[2] = pa >> 8;
           pl[3] = pb >> 8;
         }
-        uint32_t w6[4], w12[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          w6[k] = w[k] >> 6;
-          w12[k] = w[k] >> 12;
-        }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           uint32_t a[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            a[k] = pair2_scaled(w[k], w6[k], w12[k], j);
-            if (BITS == 3) a[k] |= plane_pair(pl[k], j, pos3(j));
+            a[k] = code_pair<BITS>(w[k], j);
+            if (BITS == 3) a[k] |= plane_pair(pl[k], j, code_pos<BITS>(j));
           }
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
             float (&dst)[4] = (j & 1) ? acc2[nt] : acc[0][nt];
-            mma_bf16(dst, a, qb[nt][j][0], qb[nt][j][1]);
-            if (ROT) mma_bf16(dst, a, ql[nt][j][0], ql[nt][j][1]);
+            mma_f16(dst, a, qb[nt][j][0], qb[nt][j][1]);
+            if (ROT) mma_f16(dst, a, ql[nt][j][0], ql[nt][j][1]);
           }
         }
       } else {
@@ -611,15 +749,15 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
         for (int j = 0; j < 8; ++j) {
           const int wi = j >> 1, i = 2 * (j & 1);
           uint32_t a[4];
-          a[0] = pair2_off<4>(wa[wi] >> (4 * i));
-          a[1] = pair2_off<4>(wb[wi] >> (4 * i));
-          a[2] = pair2_off<4>(wa[wi] >> (4 * i + 4));
-          a[3] = pair2_off<4>(wb[wi] >> (4 * i + 4));
+          a[0] = code_pair<4>(wa[wi], i);
+          a[1] = code_pair<4>(wb[wi], i);
+          a[2] = code_pair<4>(wa[wi], i + 1);
+          a[3] = code_pair<4>(wb[wi], i + 1);
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
             float (&dst)[4] = (j & 1) ? acc2[nt] : acc[0][nt];
-            mma_bf16(dst, a, qb[nt][j][0], qb[nt][j][1]);
-            if (ROT) mma_bf16(dst, a, ql[nt][j][0], ql[nt][j][1]);
+            mma_f16(dst, a, qb[nt][j][0], qb[nt][j][1]);
+            if (ROT) mma_f16(dst, a, ql[nt][j][0], ql[nt][j][1]);
           }
         }
       }
@@ -694,10 +832,10 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
           uint32_t a[4];
           if (BITS == 2) {
             // the word's low half holds tokens 16s..16s+7, its high half the next 8
-            a[0] = pair2<2>(prmt(w[0][0], w[1][0], 0x5410) >> (2 * g));
-            a[1] = pair2<2>(prmt(w[0][0], w[1][0], 0x7632) >> (2 * g));
-            a[2] = pair2<2>(prmt(w[2][0], w[3][0], 0x5410) >> (2 * g));
-            a[3] = pair2<2>(prmt(w[2][0], w[3][0], 0x7632) >> (2 * g));
+            a[0] = codes_bf16x2((prmt(w[0][0], w[1][0], 0x5410) >> (2 * g)) & pair_mask<2>());
+            a[1] = codes_bf16x2((prmt(w[0][0], w[1][0], 0x7632) >> (2 * g)) & pair_mask<2>());
+            a[2] = codes_bf16x2((prmt(w[2][0], w[3][0], 0x5410) >> (2 * g)) & pair_mask<2>());
+            a[3] = codes_bf16x2((prmt(w[2][0], w[3][0], 0x7632) >> (2 * g)) & pair_mask<2>());
           } else if (BITS == 3) {
             // bit 2 of token 16s + i: plane byte s (i < 8) or 2 + s (i >= 8), bit i % 8
             const uint32_t lo0 = prmt(w[0][0], w[1][0], 0x5410) >> (2 * g);
@@ -708,17 +846,17 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
             const uint32_t h1 = prmt(w[0][1], w[1][1], plane_sel(2 + s)) >> g;
             const uint32_t h2 = prmt(w[2][1], w[3][1], plane_sel(s)) >> g;
             const uint32_t h3 = prmt(w[2][1], w[3][1], plane_sel(2 + s)) >> g;
-            a[0] = pair2<3>((lo0 & 0x00030003u) | ((h0 & 0x00010001u) << 2));
-            a[1] = pair2<3>((lo1 & 0x00030003u) | ((h1 & 0x00010001u) << 2));
-            a[2] = pair2<3>((lo2 & 0x00030003u) | ((h2 & 0x00010001u) << 2));
-            a[3] = pair2<3>((lo3 & 0x00030003u) | ((h3 & 0x00010001u) << 2));
+            a[0] = codes_bf16x2((lo0 & 0x00030003u) | ((h0 & 0x00010001u) << 2));
+            a[1] = codes_bf16x2((lo1 & 0x00030003u) | ((h1 & 0x00010001u) << 2));
+            a[2] = codes_bf16x2((lo2 & 0x00030003u) | ((h2 & 0x00010001u) << 2));
+            a[3] = codes_bf16x2((lo3 & 0x00030003u) | ((h3 & 0x00010001u) << 2));
           } else {
             // words 2s, 2s+1 of a channel: tokens 16s..16s+7 and 16s+8..16s+15
             const int sh = 4 * (g & 1);
-            a[0] = pair2<4>(prmt(w[0][0], w[1][0], sel4) >> sh);
-            a[1] = pair2<4>(prmt(w[0][1], w[1][1], sel4) >> sh);
-            a[2] = pair2<4>(prmt(w[2][0], w[3][0], sel4) >> sh);
-            a[3] = pair2<4>(prmt(w[2][1], w[3][1], sel4) >> sh);
+            a[0] = codes_bf16x2((prmt(w[0][0], w[1][0], sel4) >> sh) & pair_mask<4>());
+            a[1] = codes_bf16x2((prmt(w[0][1], w[1][1], sel4) >> sh) & pair_mask<4>());
+            a[2] = codes_bf16x2((prmt(w[2][0], w[3][0], sel4) >> sh) & pair_mask<4>());
+            a[3] = codes_bf16x2((prmt(w[2][1], w[3][1], sel4) >> sh) & pair_mask<4>());
           }
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
@@ -729,16 +867,14 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
       }
       float sc[NT][4];
       if (KM == K_TOKEN) {
-        // acc = sum_d (128 + f c_d) (q_d / f) = 128 s1 + q.c, so
-        // score = s (acc - 128 s1) + z s0
+        // score = s (q.c) + z sum(q), kq and s0 with the units and the softmax scale
         const float2 mg = meta_pair<MB>(kmp, tok0 + g), mg8 = meta_pair<MB>(kmp, tok0 + g + 8);
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            const float off = -128.f * s1[nt][e];
-            sc[nt][e] = fmaf(mg.x, acc[s][nt][e] + off, mg.y * s0[nt][e]) * scale_log2;
-            sc[nt][2 + e] = fmaf(mg8.x, acc[s][nt][2 + e] + off, mg8.y * s0[nt][e]) * scale_log2;
+            sc[nt][e] = fmaf(mg.x, acc[s][nt][e] * kq[nt][e], mg.y * s0[nt][e]);
+            sc[nt][2 + e] = fmaf(mg8.x, acc[s][nt][2 + e] * kq[nt][e], mg8.y * s0[nt][e]);
           }
         }
       } else if (KM == K_KIVI) {
@@ -802,72 +938,8 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
 #pragma unroll
           for (int e = 0; e < 2; ++e) ws.z[nt][e][0] += p[nt][e] * vg.y + p[nt][2 + e] * vg8.y;
         }
-        // value codes enter as 1024 + f c; the 1024 part is collected in ws.corr
-        // by one MMA on a constant tile and removed at the end (f: see pair2_scaled)
-        {
-          const uint32_t c1024[4] = {0x64006400u, 0x64006400u, 0x64006400u, 0x64006400u};
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) mma_f16(ws.corr[nt], c1024, b[nt][0], b[nt][1]);
-        }
         const int t0 = tok0 + 2 * tq;
-        if (BITS != 4) {
-          // word g of a token row holds channels 16g..16g+15
-          constexpr int RW = 4 * BITS;  // words per token row
-          const uint32_t w0 = vc32[t0 * RW + g], w1 = vc32[(t0 + 1) * RW + g];
-          const uint32_t w8 = vc32[(t0 + 8) * RW + g], w9 = vc32[(t0 + 9) * RW + g];
-          const uint32_t x[4] = {prmt(w0, w1, 0x5410), prmt(w0, w1, 0x7632), prmt(w8, w9, 0x5410),
-                                 prmt(w8, w9, 0x7632)};
-          // 3 bits: bit 2 of word g's codes 0-7 is byte g % 2 of plane word
-          // 8 + g / 2, codes 8-15 byte 2 + g % 2; two tokens side by side
-          uint32_t hp[4] = {0u, 0u, 0u, 0u};
-          if (BITS == 3) {
-            const int pw = 8 + (g >> 1), bs = g & 1;
-            const uint32_t p0 = vc32[t0 * RW + pw], p1 = vc32[(t0 + 1) * RW + pw];
-            const uint32_t p8 = vc32[(t0 + 8) * RW + pw], p9 = vc32[(t0 + 9) * RW + pw];
-            hp[0] = prmt(p0, p1, plane_sel(bs));
-            hp[1] = prmt(p0, p1, plane_sel(2 + bs));
-            hp[2] = prmt(p8, p9, plane_sel(bs));
-            hp[3] = prmt(p8, p9, plane_sel(2 + bs));
-          }
-          uint32_t x6[4], x12[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            x6[k] = x[k] >> 6;
-            x12[k] = x[k] >> 12;
-          }
-#pragma unroll
-          for (int mt = 0; mt < 8; ++mt) {
-            uint32_t a[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              a[k] = pair2_scaled_h(x[k], x6[k], x12[k], mt);
-              if (BITS == 3) a[k] |= plane_pair(hp[k], mt, pos3(mt));
-            }
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) mma_f16(ws.o[nt][mt], a, b[nt][0], b[nt][1]);
-          }
-        } else {
-          // word 2g holds channels 16g..16g+7 (codes 0-3 low half, 4-7 high), 2g+1 the next 8
-          const uint2 v0 = *reinterpret_cast<const uint2*>(vc32 + t0 * 16 + 2 * g);
-          const uint2 v1 = *reinterpret_cast<const uint2*>(vc32 + (t0 + 1) * 16 + 2 * g);
-          const uint2 v8 = *reinterpret_cast<const uint2*>(vc32 + (t0 + 8) * 16 + 2 * g);
-          const uint2 v9 = *reinterpret_cast<const uint2*>(vc32 + (t0 + 9) * 16 + 2 * g);
-          const uint32_t xa = prmt(v0.x, v1.x, 0x5410), ya = prmt(v0.x, v1.x, 0x7632);
-          const uint32_t xb = prmt(v0.y, v1.y, 0x5410), yb = prmt(v0.y, v1.y, 0x7632);
-          const uint32_t xc = prmt(v8.x, v9.x, 0x5410), yc = prmt(v8.x, v9.x, 0x7632);
-          const uint32_t xd = prmt(v8.y, v9.y, 0x5410), yd = prmt(v8.y, v9.y, 0x7632);
-#pragma unroll
-          for (int mt = 0; mt < 8; ++mt) {
-            const int sh = 4 * (mt & 3);
-            uint32_t a[4];
-            a[0] = pair2_off_h<4>((mt < 4 ? xa : ya) >> sh);
-            a[1] = pair2_off_h<4>((mt < 4 ? xb : yb) >> sh);
-            a[2] = pair2_off_h<4>((mt < 4 ? xc : yc) >> sh);
-            a[3] = pair2_off_h<4>((mt < 4 ? xd : yd) >> sh);
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) mma_f16(ws.o[nt][mt], a, b[nt][0], b[nt][1]);
-          }
-        }
+        pv_codes<BITS, NT>(ws.o, vc32, t0, t0 + 1, t0 + 8, t0 + 9, g, b);
       } else {  // V_KIVI: 4 value groups of 32 channels; m-tile mt = channels 16mt..16mt+15
         float sv_g[4], zv_g[4], sv_g8[4], zv_g8[4];
         {
@@ -907,10 +979,10 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
           if (BITS == 2) {
             const uint32_t w0 = vc32[t0 * W + mt], w1 = vc32[(t0 + 1) * W + mt];
             const uint32_t w8 = vc32[(t0 + 8) * W + mt], w9 = vc32[(t0 + 9) * W + mt];
-            a[0] = pair2_h<2>(prmt(w0, w1, 0x5410) >> (2 * g));
-            a[1] = pair2_h<2>(prmt(w0, w1, 0x7632) >> (2 * g));
-            a[2] = pair2_h<2>(prmt(w8, w9, 0x5410) >> (2 * g));
-            a[3] = pair2_h<2>(prmt(w8, w9, 0x7632) >> (2 * g));
+            a[0] = codes_f16x2((prmt(w0, w1, 0x5410) >> (2 * g)) & pair_mask<2>());
+            a[1] = codes_f16x2((prmt(w0, w1, 0x7632) >> (2 * g)) & pair_mask<2>());
+            a[2] = codes_f16x2((prmt(w8, w9, 0x5410) >> (2 * g)) & pair_mask<2>());
+            a[3] = codes_f16x2((prmt(w8, w9, 0x7632) >> (2 * g)) & pair_mask<2>());
           } else if (BITS == 3) {
             // channels 16mt + g and 16mt + 8 + g: bit 2 in byte mt % 2 and
             // 2 + mt % 2 of plane word 8 + mt / 2, bit g
@@ -921,40 +993,25 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
             const uint32_t p8 = vc32[(t0 + 8) * W + pw], p9 = vc32[(t0 + 9) * W + pw];
             const uint32_t h0 = prmt(p0, p1, plane_sel(bs)) >> g, h1 = prmt(p0, p1, plane_sel(2 + bs)) >> g;
             const uint32_t h2 = prmt(p8, p9, plane_sel(bs)) >> g, h3 = prmt(p8, p9, plane_sel(2 + bs)) >> g;
-            a[0] = pair2_h<3>(((prmt(w0, w1, 0x5410) >> (2 * g)) & 0x00030003u) | ((h0 & 0x00010001u) << 2));
-            a[1] = pair2_h<3>(((prmt(w0, w1, 0x7632) >> (2 * g)) & 0x00030003u) | ((h1 & 0x00010001u) << 2));
-            a[2] = pair2_h<3>(((prmt(w8, w9, 0x5410) >> (2 * g)) & 0x00030003u) | ((h2 & 0x00010001u) << 2));
-            a[3] = pair2_h<3>(((prmt(w8, w9, 0x7632) >> (2 * g)) & 0x00030003u) | ((h3 & 0x00010001u) << 2));
+            a[0] = codes_f16x2(((prmt(w0, w1, 0x5410) >> (2 * g)) & 0x00030003u) | ((h0 & 0x00010001u) << 2));
+            a[1] = codes_f16x2(((prmt(w0, w1, 0x7632) >> (2 * g)) & 0x00030003u) | ((h1 & 0x00010001u) << 2));
+            a[2] = codes_f16x2(((prmt(w8, w9, 0x5410) >> (2 * g)) & 0x00030003u) | ((h2 & 0x00010001u) << 2));
+            a[3] = codes_f16x2(((prmt(w8, w9, 0x7632) >> (2 * g)) & 0x00030003u) | ((h3 & 0x00010001u) << 2));
           } else {
             const uint2 u0 = *reinterpret_cast<const uint2*>(vc32 + t0 * W + 2 * mt);
             const uint2 u1 = *reinterpret_cast<const uint2*>(vc32 + (t0 + 1) * W + 2 * mt);
             const uint2 u8 = *reinterpret_cast<const uint2*>(vc32 + (t0 + 8) * W + 2 * mt);
             const uint2 u9 = *reinterpret_cast<const uint2*>(vc32 + (t0 + 9) * W + 2 * mt);
             const int sh = 4 * (g & 1);
-            a[0] = pair2_h<4>(prmt(u0.x, u1.x, sel4) >> sh);
-            a[1] = pair2_h<4>(prmt(u0.y, u1.y, sel4) >> sh);
-            a[2] = pair2_h<4>(prmt(u8.x, u9.x, sel4) >> sh);
-            a[3] = pair2_h<4>(prmt(u8.y, u9.y, sel4) >> sh);
+            a[0] = codes_f16x2((prmt(u0.x, u1.x, sel4) >> sh) & pair_mask<4>());
+            a[1] = codes_f16x2((prmt(u0.y, u1.y, sel4) >> sh) & pair_mask<4>());
+            a[2] = codes_f16x2((prmt(u8.x, u9.x, sel4) >> sh) & pair_mask<4>());
+            a[3] = codes_f16x2((prmt(u8.y, u9.y, sel4) >> sh) & pair_mask<4>());
           }
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) mma_f16(ws.o[nt][mt], a, b[nt][mt >> 1][0], b[nt][mt >> 1][1]);
         }
       }
-    }
-  }
-  if (VM == V_TOKEN) {
-    // Fold the tile's 1024 offsets into the accumulators.  Both grow with the
-    // segment while their difference (the value sum) stays small; left to the
-    // end of a long segment (thousands of tokens in one CTA), the fp32
-    // accumulation error of the large common part would show in the result.
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-      for (int mt = 0; mt < 8; ++mt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) ws.o[nt][mt][i] -= ws.corr[nt][i];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) ws.corr[nt][i] = 0.f;
     }
   }
 }
@@ -1055,6 +1112,40 @@ struct QPieces {
   static constexpr int n = (NT * 8 * 16 + kThreads - 1) / kThreads;
 };
 
+// The queries as fp32 rows in shared memory (rows >= G zero).  TOP >= 0: each
+// row divided by a power of two (exact) that brings its largest element to
+// 2^TOP at most, kept in qn[row].
+template <int NT, int TOP>
+__device__ __forceinline__ void stage_queries(float* q_s, float* qn, const uint4 (&qv)[QPieces<NT>::n], int tid) {
+#pragma unroll
+  for (int k = 0; k < QPieces<NT>::n; ++k) {
+    const int i = tid + k * kThreads;
+    if (i < NT * 8 * 16) {  // whole warps
+      // piece i: row i / 16, channels 8 (i % 16) .. + 7
+      float4* dst = reinterpret_cast<float4*>(q_s + qidx(i >> 4, 8 * (i & 15)));
+      float f[8];
+      bf16x2_to_f32(qv[k].x, f[0], f[1]);
+      bf16x2_to_f32(qv[k].y, f[2], f[3]);
+      bf16x2_to_f32(qv[k].z, f[4], f[5]);
+      bf16x2_to_f32(qv[k].w, f[6], f[7]);
+      if (TOP >= 0) {
+        float m = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) m = fmaxf(m, fabsf(f[e]));
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));  // the row's 16 threads
+        const float n = pow2_ceil(fminf(fmaxf(m, kScaleLow), kScaleTop)) * (1.0f / (float)(1 << (TOP < 0 ? 0 : TOP)));
+        const float inv = pow2_inv(n);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) f[e] *= inv;
+        if ((i & 15) == 0) qn[i >> 4] = n;
+      }
+      dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+      dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+  }
+}
+
 template <int BITS, int NT, int KM, int VM, bool ROT, int MB>
 __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int te, const DecodeParams& p,
                                          const uint4 (&qv)[QPieces<NT>::n], int G, float* parts) {
@@ -1067,47 +1158,16 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
   const int g = lane >> 2, tq = lane & 3;
   float* q_s = reinterpret_cast<float*>(smem + SmemLayout<NT>::q);
   const float scale_log2 = p.scale_log2;
-  constexpr int QV = QPieces<NT>::n;
 
-  // This warp's quarter of the chunk (whole 16-token slices, KIVI-style key
-  // groups) and its pipeline: fill i uses slot i % SLOTS and phase i / SLOTS
-  // of that slot's mbarrier.
-  constexpr int SLOTS = TL::slots, FPT = TL::SPLIT ? 2 : 1;  // fills per tile
-  constexpr int GRAN = (KM == K_KIVI) ? kKiviGroup : 16;
-  const int span = (max(te - tb, 0) + kWarps * GRAN - 1) / (kWarps * GRAN) * GRAN;
-  const int wb = min(tb + warp * span, te), we = min(wb + span, te);
-  const int n_tiles = (max(we - wb, 0) + TL::tokens - 1) / TL::tokens;
-  const int n_fills = n_tiles * FPT;
-  char* buf = smem + kStageOff + warp * kWarpBuf;
-  const uint32_t buf0 = smem_u32(buf);
-  const uint32_t bars = smem_u32(smem + SmemLayout<NT>::bar) + warp * (8 * kMaxSlots);
-  volatile int* abort = reinterpret_cast<volatile int*>(smem + SmemLayout<NT>::bar + 8 * kMaxSlots * kWarps);
-  // Only the first tile goes in flight now: with every CTA of the launch
-  // starting at once, first tiles alone make a burst the memory system serves
-  // quickly, so compute starts early; the other slots are filled once the
-  // first tile has landed.
-  int issued = min(n_fills, FPT);
-  if (elect_one())
-    for (int i = 0; i < issued; ++i)
-      issue_fill<BITS, KM, VM, MB>(buf0 + i * TL::slot_bytes, bars + 8 * i, sg, i, wb, we, &p.arena_map);
+  WarpPipe<BITS, NT, KM, VM, MB, false> pipe(smem, warp, sg, p, tb, te, (KM == K_KIVI) ? kKiviGroup : 16);
 
   // Queries of this KV head's group (fp32, rows >= G zero), rotated for
   // AKVQ-style coded keys.
-#pragma unroll
-  for (int k = 0; k < QV; ++k) {
-    const int i = tid + k * kThreads;
-    if (i < NT * 8 * 16) {
-      // piece i: row i / 16, channels 8 (i % 16) .. + 7
-      float4* dst = reinterpret_cast<float4*>(q_s + qidx(i >> 4, 8 * (i & 15)));
-      float f[8];
-      bf16x2_to_f32(qv[k].x, f[0], f[1]);
-      bf16x2_to_f32(qv[k].y, f[2], f[3]);
-      bf16x2_to_f32(qv[k].z, f[4], f[5]);
-      bf16x2_to_f32(qv[k].w, f[6], f[7]);
-      dst[0] = make_float4(f[0], f[1], f[2], f[3]);
-      dst[1] = make_float4(f[4], f[5], f[6], f[7]);
-    }
-  }
+  // Per-token coded keys: rows scaled so that every staged and rotated element (at most
+  // sqrt(128) times the row's largest) is below FP16's 65504.
+  constexpr int TOP = KM == K_TOKEN ? (ROT ? 11 : 15) : -1;
+  float* qn = reinterpret_cast<float*>(smem + SmemLayout<NT>::qn);
+  stage_queries<NT, TOP>(q_s, qn, qv, tid);
   __syncthreads();
   if (ROT) {
     for (int j = warp; j < G; j += kWarps) {
@@ -1125,11 +1185,23 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
   for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
     for (int j = 0; j < 8; ++j) qb[nt][j][0] = qb[nt][j][1] = ql[nt][j][0] = ql[nt][j][1] = 0u;
-  float s1[NT][2], s0[NT][2];
+  // per-token coded keys, per column: unit of the key MMAs' results and sum of
+  // the query, both with the softmax scale
+  float kq[NT][2], s0[NT][2];
 #pragma unroll
-  for (int nt = 0; nt < NT; ++nt) s1[nt][0] = s1[nt][1] = s0[nt][0] = s0[nt][1] = 0.f;
+  for (int nt = 0; nt < NT; ++nt) kq[nt][0] = kq[nt][1] = s0[nt][0] = s0[nt][1] = 0.f;
   if (KM == K_BF16) qfrag_natural<NT>(qb, q_s, g, tq);
-  if (KM == K_TOKEN) qfrag_token<BITS, NT, ROT>(qb, ql, s1, s0, q_s, g, tq);
+  if (KM == K_TOKEN) {
+    qfrag_token<BITS, NT, ROT>(qb, ql, s0, q_s, g, tq);
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float n = qn[nt * 8 + 2 * tq + e] * scale_log2;
+        s0[nt][e] *= n;
+        kq[nt][e] = n * kCodeUnit;
+      }
+  }
 
   WarpState<NT, NZ> ws;
 #pragma unroll
@@ -1145,66 +1217,25 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
     for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
       for (int i = 0; i < 4; ++i) ws.o[nt][mt][i] = 0.f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) ws.corr[nt][i] = 0.f;
   }
   ws.vb = __uint_as_float(0x00800000u);  // 2^-126: no value scale seen yet
 
-  // Wait for fill f (in slot fs, phase parity fp), then move on to the next.
-  int fs = 0, fp = 0;
-  auto landed = [&]() {
-    if (__all_sync(kFull, mbar_try_wait(bars + 8 * fs, fp))) return true;
-    return (bool)__all_sync(kFull, wait_tile(bars + 8 * fs, fp, abort, p.status));
-  };
-  auto next = [&]() {
-    if (++fs == SLOTS) {
-      fs = 0;
-      fp ^= 1;
-    }
-  };
-  // Refill the slot just consumed (every lane has read it).
-  auto refill = [&]() {
-    __syncwarp();
-    if (issued < n_fills) {
-      if (elect_one()) {
-        fence_proxy_async_shared();
-        issue_fill<BITS, KM, VM, MB>(buf0 + fs * TL::slot_bytes, bars + 8 * fs, sg, issued, wb, we, &p.arena_map);
-      }
-      ++issued;
-    }
-    next();
-  };
 #pragma unroll 1
-  for (int it = 0; it < n_tiles; ++it) {
-    if (!landed()) break;
-    if (it == 0) {  // tile 0 landed: fill the other slots
-      const int upto = min(n_fills, SLOTS);
-      if (elect_one())
-        for (int i = issued; i < upto; ++i)
-          issue_fill<BITS, KM, VM, MB>(buf0 + i * TL::slot_bytes, bars + 8 * i, sg, i, wb, we, &p.arena_map);
-      issued = upto;
-    }
-    const char* kst = buf + fs * TL::slot_bytes;
-    const char* vst = TL::SPLIT ? buf + (fs + 1 == SLOTS ? 0 : fs + 1) * TL::slot_bytes : kst;
+  for (int it = 0; it < pipe.n_tiles; ++it) {
+    if (!pipe.landed()) break;
+    if (it == 0) pipe.fill_rest();
+    const char* kst = pipe.slot();
+    const char* vst = TL::SPLIT ? pipe.next_slot() : kst;
     bool ok = true;
-    compute_tile<BITS, NT, KM, VM, ROT, MB>(ws, kst, vst, min(TL::tokens, we - wb - it * TL::tokens), qb, ql, q_s, s1,
-                                            s0, scale_log2, lane, [&]() {
-                                              refill();
-                                              return ok = landed();
+    compute_tile<BITS, NT, KM, VM, ROT, MB>(ws, kst, vst, pipe.tile_tokens(it), qb, ql, q_s, kq, s0, scale_log2, lane,
+                                            [&]() {
+                                              pipe.refill();
+                                              return ok = pipe.landed();
                                             });
     if (TL::SPLIT && !ok) break;
-    refill();
+    pipe.refill();
   }
-  if (*abort && lane == 0) {
-    // A slot is refilled only after its previous fill landed, so only the
-    // last SLOTS fills can still be in flight: let them land (bounded) before
-    // the buffer is reused or the CTA exits.
-    for (int t = (issued > SLOTS ? issued - SLOTS : 0); t < issued; ++t)
-      for (uint32_t i = 0; i < kWaitRounds && !mbar_try_wait_sleep(bars + 8 * (t % SLOTS), (t / SLOTS) & 1,
-                                                                    kWaitSleepNs);
-           ++i) {
-      }
-  }
+  pipe.drain(lane);
   __syncthreads();  // the warps' buffers are reused for the reduction below
 
   // ---- per-warp results: reduce l and the value-zero terms over the 8 rows g ----
@@ -1235,22 +1266,362 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
       for (int mt = 0; mt < 8; ++mt) {
         int c_lo, c_hi;  // channels of rows g and g+8 of m-tile mt
         if (VM == V_TOKEN) {
-          // remove the 128 offset and the 4^(mt % 3) factor of 2-bit value pairs
           c_lo = 16 * g + mt;
           c_hi = 16 * g + 8 + mt;
-          // and the units (vb) of the coded-value accumulators
-          const float f = ((BITS != 4) ? 1.0f / (float)(1 << pos3(mt)) : 1.0f) * ws.vb;
-          orow[c_lo] = (ws.o[nt][mt][e] - ws.corr[nt][e]) * f + ws.z[nt][e][0];
-          orow[c_hi] = (ws.o[nt][mt][2 + e] - ws.corr[nt][2 + e]) * f + ws.z[nt][e][0];
+          // units of the codes (a position's factor, 2^24), then of the scales (vb)
+          const float f = code_unit<BITS>(BITS == 4 ? mt % 4 : mt) * kCodeUnit;
+          orow[c_lo] = fmaf(ws.o[nt][mt][e] * f, ws.vb, ws.z[nt][e][0]);
+          orow[c_hi] = fmaf(ws.o[nt][mt][2 + e] * f, ws.vb, ws.z[nt][e][0]);
         } else {
           c_lo = 16 * mt + g;
           c_hi = 16 * mt + 8 + g;
           const float z = (VM == V_KIVI) ? ws.z[nt][e][(mt >> 1) % NZ] : 0.f;
-          const float f = (VM == V_KIVI) ? ws.vb : 1.0f;  // units of coded values
-          orow[c_lo] = ws.o[nt][mt][e] * f + z;
-          orow[c_hi] = ws.o[nt][mt][2 + e] * f + z;
+          if (VM == V_KIVI) {
+            orow[c_lo] = fmaf(ws.o[nt][mt][e], ws.vb, z);
+            orow[c_hi] = fmaf(ws.o[nt][mt][2 + e], ws.vb, z);
+          } else {
+            orow[c_lo] = ws.o[nt][mt][e];
+            orow[c_hi] = ws.o[nt][mt][2 + e];
+          }
         }
       }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// KIVI-style items with QC = 1 or 2 queries per KV head (multi-head attention):
+// the eight MMA columns hold what run_item leaves to lane-dependent shifts.
+//
+// Keys, 64 tokens (two 32-token groups) at a time.  Row g of every m-tile is
+// half g / 4 of code word g % 4 (16 tokens: word s of group r is 2r + s), and
+// the m-tile picks the position inside the half, so a lane expands its words
+// at fixed bit positions (three shifts for eight of them, see code_pair) instead of shifting every pair by its own amount.  The rows of one m-tile
+// then belong to both groups, whose scaled queries q_c s_c differ: column
+// 4r + 2k + h holds group r's, h the FP16 hi or lo part, k the query (QC = 2)
+// or the parity of the k-steps the lane scales (QC = 1: each lane builds half
+// of them, the other columns see zeros).  Row g reads columns 4r .. 4r + 3 of
+// its group r = (g / 2) % 2.
+// The 64 scores pass through shared memory, so the softmax works on two tokens
+// per lane instead of four columns of which one or two are real.
+//
+// Values: column 4q + j holds p_t s_tj of value group j, so every row takes the
+// channel-order expansion of per-token codes (pv_codes) and reads the column of
+// its own group (channels 16g .. 16g + 15: group g / 2).  Tokens tq, tq + 4,
+// tq + 8, tq + 12 of a slice sit in one lane's k-slots (codes and metadata of
+// the four tq lanes on different banks).
+//
+// Issue-bound before: 772 warp instructions per 16-token slice in run_item
+// (one query in eight columns), 32 KV heads of 3,120 tokens in 16 rows at 109 us
+// a layer, 0.39 of the measured copy rate; here 278 and 55 us, 0.77.  Error
+// against 64 bits as before (with BF16 128 + c and FP16 1024 + c operands, the
+// offsets removed by MMAs over constant tiles, it grew from 1.71e-3 to 2.1e-3).
+// ---------------------------------------------------------------------------
+template <int QC>
+struct ColState {
+  float o[1][8][4];   // as WarpState, in units of vb
+  float vb;
+  float kb;      // power-of-two bound of the key channel scales seen so far
+  float z;       // column g: sum_t p_t z_t of value group g % 4, query g / 4
+  float m[QC], l[QC];  // running maxima (the warp's), sums of this lane's tokens
+};
+
+// Scores of the tile's tokens 2 lane, 2 lane + 1 (x[q][i], log2 units, -inf past
+// the end) -> probabilities into ps[q][token], a slice's 16 tokens permuted so
+// that lane tq's four are contiguous (token t of a slice at 4 (t % 4) + t / 4).
+template <int QC>
+__device__ __forceinline__ void cols_softmax(ColState<QC>& ws, const float (&x)[QC][2], float* ps, int lane) {
+  bool need = false;
+#pragma unroll
+  for (int q = 0; q < QC; ++q) need |= fmaxf(x[q][0], x[q][1]) > ws.m[q] + 8.0f;
+  if (__any_sync(kFull, need)) {
+    float a[QC];
+#pragma unroll
+    for (int q = 0; q < QC; ++q) {
+      const float mn = fmaxf(ws.m[q], warp_max(fmaxf(x[q][0], x[q][1])));
+      a[q] = (ws.m[q] == -INFINITY) ? 0.f : fast_exp2(ws.m[q] - mn);
+      ws.m[q] = mn;
+      ws.l[q] *= a[q];
+    }
+    const float az = (QC == 2 && (lane & 16)) ? a[QC - 1] : a[0];  // this lane's column g: query g / 4
+    const float ao = (QC == 2 && (lane & 2)) ? a[QC - 1] : a[0];   // its accumulator columns 2tq, 2tq + 1
+    ws.z *= az;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int mt = 0; mt < 8; ++mt) ws.o[0][mt][i] *= ao;
+  }
+  __syncwarp();  // the scores have been read
+  const int t = 2 * lane;
+  float* dst = ps + (t & ~15) + 4 * (t & 3) + ((t >> 2) & 3);
+#pragma unroll
+  for (int q = 0; q < QC; ++q) {
+    const float p0 = fast_exp2(x[q][0] - ws.m[q]), p1 = fast_exp2(x[q][1] - ws.m[q]);
+    ws.l[q] += p0 + p1;
+    dst[64 * q] = p0;
+    dst[64 * q + 4] = p1;
+  }
+  __syncwarp();
+}
+
+// Raw scores of a 64-token tile of KIVI-style keys: kst its codes and metadata,
+// x[q][i] the scores of tokens 2 lane + i, in units of the staged query rows
+// and without the softmax scale.
+template <int BITS, int QC, int MB>
+__device__ __forceinline__ void cols_scores(const char* kst, const char* kmeta, const float* q_s, float* ps, float& kb,
+                                            bool two_groups, int lane, float (&x)[QC][2]) {
+  const int g = lane >> 2, tq = lane & 3;
+  const int sel = (g >> 1) & 1, lo = g & 1;  // this lane's column: k-step parity or query; hi or lo part
+  // scaled queries of group g / 4, this lane's column
+  constexpr int NB = QC == 1 ? 4 : 8;
+  uint32_t own[NB][2];
+  float zk = 0.f;
+  {
+    // in units of kb, a power of two no smaller than any channel scale so far
+    float top = 0.f;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      float2 m[4];
+      meta_quad<MB>(kmeta, (g >> 2) * kD + 16 * (QC == 1 ? 2 * i + sel : i) + 4 * tq, m);
+      top = fmaxf(top, fmaxf(fmaxf(m[0].x, m[1].x), fmaxf(m[2].x, m[3].x)));
+    }
+    if (!two_groups && lane >= 16) top = 0.f;  // stale metadata of an absent second group
+    if (__any_sync(kFull, top > kb)) kb = pow2_ceil(fminf(warp_max(top), kScaleTop));
+  }
+  const float inv = pow2_inv(kb);
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int c0 = 16 * (QC == 1 ? 2 * i + sel : i) + 4 * tq;
+    float2 m[4];
+    meta_quad<MB>(kmeta, (g >> 2) * kD + c0, m);
+    const float4 qv = *reinterpret_cast<const float4*>(q_s + (QC == 1 ? 0 : sel) * kQRow + c0);
+    uint32_t hi, rest;
+    split_pair16(qv.x * (m[0].x * inv), qv.y * (m[1].x * inv), hi, rest);
+    own[i][0] = lo ? rest : hi;
+    split_pair16(qv.z * (m[2].x * inv), qv.w * (m[3].x * inv), hi, rest);
+    own[i][1] = lo ? rest : hi;
+    zk = fmaf(qv.x, m[0].y, zk);
+    zk = fmaf(qv.y, m[1].y, zk);
+    zk = fmaf(qv.z, m[2].y, zk);
+    zk = fmaf(qv.w, m[3].y, zk);
+  }
+  zk += __shfl_xor_sync(kFull, zk, 1);
+  zk += __shfl_xor_sync(kFull, zk, 2);
+  const float zo = __shfl_xor_sync(kFull, zk, 8);  // the other parity's part, or the other query's term
+
+  const int r = (g >> 1) & 1, s = g & 1;  // group and word of this lane's rows
+  const bool upper = g >= 4;              // half of the word
+  const uint32_t half = upper ? 0x7632u : 0x5410u;
+  const uint32_t* gc = reinterpret_cast<const uint32_t*>(kst) + r * (kD * BITS);
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int mt = 0; mt < 4; ++mt) acc[mt][i] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    // k-slots 2tq, 2tq + 1, 2tq + 8, 2tq + 9 of k-step j <-> channels 16j + 4tq + 0..3
+    const int c0 = 16 * j + 4 * tq;
+    uint32_t b0 = own[QC == 1 ? j >> 1 : j][0], b1 = own[QC == 1 ? j >> 1 : j][1];
+    if (QC == 1 && sel != (j & 1)) b0 = b1 = 0u;
+    uint32_t y[2][2], hp[2] = {0u, 0u};  // per channel pair: codes of its half word(s), bit-2 planes
+#pragma unroll
+    for (int cp = 0; cp < 2; ++cp) {
+      const uint32_t* w = gc + (c0 + 2 * cp) * BITS;
+      if (BITS == 4) {
+        const int i = 2 * s + (upper ? 1 : 0);
+        y[cp][0] = prmt(w[i], w[4 + i], 0x5410);
+        y[cp][1] = prmt(w[i], w[4 + i], 0x7632);
+      } else {
+        y[cp][0] = y[cp][1] = prmt(w[s], w[BITS + s], half);
+        if (BITS == 3) hp[cp] = prmt(w[2], w[BITS + 2], plane_sel(0) + 0x1111u * (s + (upper ? 2 : 0)));
+      }
+    }
+#pragma unroll
+    for (int mt = 0; mt < 4; ++mt) {
+      uint32_t a[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int pos = mt + 4 * (k & 1);  // rows g: positions 0..3, rows g + 8: 4..7
+        a[k] = code_pair<BITS>(y[k >> 1][BITS == 4 ? k & 1 : 0], BITS == 4 ? mt : pos);
+        if (BITS == 3) a[k] |= plane_pair(hp[k >> 1], pos, code_pos<BITS>(pos));
+      }
+      mma_f16(acc[mt], a, b0, b1);
+    }
+  }
+  // rows g and g + 8 of m-tile mt: tokens 16 (g % 4) + 8 (g / 4) + mt and + 4
+  if ((tq >> 1) == r) {
+    float v[8];
+#pragma unroll
+    for (int mt = 0; mt < 4; ++mt) {
+      const float unit = kb * kCodeUnit;
+      v[mt] = (acc[mt][0] + acc[mt][1]) * (code_unit<BITS>(mt) * unit);
+      v[4 + mt] = (acc[mt][2] + acc[mt][3]) * (code_unit<BITS>(BITS == 4 ? mt : mt + 4) * unit);
+    }
+    float4* dst = reinterpret_cast<float4*>(ps + 64 * (tq & 1) + 16 * (g & 3) + 8 * (g >> 2));
+    dst[0] = make_float4(v[0], v[1], v[2], v[3]);
+    dst[1] = make_float4(v[4], v[5], v[6], v[7]);
+  }
+  __syncwarp();
+  // tokens 2 lane, 2 lane + 1 are of group lane / 16, as is this lane's zk
+  const float2 u0 = *reinterpret_cast<const float2*>(ps + 2 * lane);
+  const float2 u1 = *reinterpret_cast<const float2*>(ps + 64 + 2 * lane);
+  if (QC == 1) {
+    x[0][0] = (u0.x + u1.x) + (zk + zo);
+    x[0][1] = (u0.y + u1.y) + (zk + zo);
+  } else {
+    const float z0 = sel ? zo : zk, z1 = sel ? zk : zo;
+    x[0][0] = u0.x + z0;
+    x[0][1] = u0.y + z0;
+    x[QC - 1][0] = u1.x + z1;
+    x[QC - 1][1] = u1.y + z1;
+  }
+}
+
+// KM: K_KIVI (quantized heads) or K_BF16 (image keys of keys-only heads).
+template <int BITS, int QC, int KM, int MB>
+__device__ __forceinline__ void run_item_cols(char* smem, const Seg& sg, int tb, int te, const DecodeParams& p,
+                                              const uint4 (&qv)[QPieces<1>::n], float* parts) {
+  using TL = Tile<BITS, KM, V_KIVI, MB, true>;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(kFull, tid >> 5, 0);
+  const int g = lane >> 2, tq = lane & 3;
+  float* q_s = reinterpret_cast<float*>(smem + SmemLayout<1>::q);
+  // scores and probabilities of the warp's tile, [2][64], behind the QC query rows
+  static_assert((2 * kQRow + kWarps * 128) * 4 <= 8 * kQRow * 4, "the query rows above the first two hold the scores");
+  float* ps = q_s + 2 * kQRow + warp * 128;
+  WarpPipe<BITS, 1, KM, V_KIVI, MB, true> pipe(smem, warp, sg, p, tb, te, (KM == K_KIVI) ? kKiviGroup : 16);
+
+  float* qn = reinterpret_cast<float*>(smem + SmemLayout<1>::qn);
+  stage_queries<1, KM == K_BF16 ? -1 : 15>(q_s, qn, qv, tid);
+  __syncthreads();
+  float unit[QC];  // of the scores: the staged rows' and the softmax scale
+#pragma unroll
+  for (int q = 0; q < QC; ++q) unit[q] = (KM == K_BF16 ? 1.f : qn[q]) * p.scale_log2;
+  uint32_t qb[1][8][2];
+  if (KM == K_BF16) {
+    qfrag_natural<1>(qb, q_s, g, tq);
+    __syncthreads();  // rows 2.. hold the scores from here on
+  }
+  ColState<QC> ws;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int mt = 0; mt < 8; ++mt) ws.o[0][mt][i] = 0.f;
+#pragma unroll
+  for (int q = 0; q < QC; ++q) {
+    ws.m[q] = -INFINITY;
+    ws.l[q] = 0.f;
+  }
+  ws.z = 0.f;
+  ws.vb = __uint_as_float(0x00800000u);  // 2^-126: no value scale seen yet
+  ws.kb = kScaleLow;
+
+#pragma unroll 1
+  for (int it = 0; it < pipe.n_tiles; ++it) {
+    if (!pipe.landed()) break;
+    if (it == 0) pipe.fill_rest();
+    const char* kst = pipe.slot();
+    const char* vst = pipe.next_slot();
+    const int nvalid = pipe.tile_tokens(it);  // whole slices: coded tokens come in groups of 32
+    float x[QC][2];
+    if constexpr (KM == K_KIVI) {
+      cols_scores<BITS, QC, MB>(kst, kst + TL::km_off, q_s, ps, ws.kb, nvalid > kKiviGroup, lane, x);
+    } else {
+      const uint32_t rbase = smem_u32(kst) + ((lane & 7) + 8 * ((lane >> 3) & 1)) * 128;
+      const int rsw = lane & 7, ch = lane >> 4;
+      float acc[2][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[0][i] = acc[1][i] = 0.f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        uint32_t a[4];
+        ldsm_x4(a, rbase + (j >> 2) * (TL::tokens * 128) + (((2 * (j & 3) + ch) ^ rsw) << 4));
+        mma_bf16(acc[j & 1], a, qb[0][j][0], qb[0][j][1]);
+      }
+      if (tq == 0) {  // columns 0, 1: the queries
+        ps[g] = acc[0][0] + acc[1][0];
+        ps[g + 8] = acc[0][2] + acc[1][2];
+        if (QC == 2) {
+          ps[64 + g] = acc[0][1] + acc[1][1];
+          ps[64 + g + 8] = acc[0][3] + acc[1][3];
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < QC; ++q) {
+        const float2 u = *reinterpret_cast<const float2*>(ps + 64 * q + (2 * lane & 15));
+        x[q][0] = u.x;
+        x[q][1] = u.y;
+      }
+    }
+    pipe.refill();
+    const bool in = 2 * lane < nvalid;
+#pragma unroll
+    for (int q = 0; q < QC; ++q)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) x[q][i] = in ? x[q][i] * unit[q] : -INFINITY;
+    cols_softmax<QC>(ws, x, ps, lane);
+    if (!pipe.landed()) break;
+
+    const uint32_t* vc32 = reinterpret_cast<const uint32_t*>(vst);
+    const char* vmp = vst + TL::vm_off;
+#pragma unroll 1
+    for (int t0 = 0; t0 < nvalid; t0 += 16) {
+      const float4 pt = *reinterpret_cast<const float4*>(ps + (QC == 2 ? 64 * (g >> 2) : 0) + t0 + 4 * tq);
+      const int t = t0 + tq;  // and t + 4, + 8, + 12
+      float2 vm[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) vm[i] = meta_pair<MB>(vmp, (t + 4 * i) * 4 + (g & 3));
+      const float smax = fmaxf(fmaxf(vm[0].x, vm[1].x), fmaxf(vm[2].x, vm[3].x));
+      if (__any_sync(kFull, smax > ws.vb)) {
+        const float nb = pow2_ceil(warp_max(smax));
+        const float a = ws.vb * pow2_inv(nb);  // a power of two: exact
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int mt = 0; mt < 8; ++mt) ws.o[0][mt][i] *= a;
+        ws.vb = nb;
+      }
+      const float inv = pow2_inv(ws.vb);
+      uint32_t b[1][2];
+      b[0][0] = pack_half2(pt.x * (vm[0].x * inv), pt.y * (vm[1].x * inv));
+      b[0][1] = pack_half2(pt.z * (vm[2].x * inv), pt.w * (vm[3].x * inv));
+      ws.z = fmaf(pt.x, vm[0].y, ws.z);
+      ws.z = fmaf(pt.y, vm[1].y, ws.z);
+      ws.z = fmaf(pt.z, vm[2].y, ws.z);
+      ws.z = fmaf(pt.w, vm[3].y, ws.z);
+      pv_codes<BITS, 1>(ws.o, vc32, t, t + 4, t + 8, t + 12, g, b);
+    }
+    pipe.refill();
+  }
+  pipe.drain(lane);
+  __syncthreads();  // the warps' buffers are reused for the reduction below
+
+  ws.z += __shfl_xor_sync(kFull, ws.z, 1);
+  ws.z += __shfl_xor_sync(kFull, ws.z, 2);
+#pragma unroll
+  for (int q = 0; q < QC; ++q) {
+    const float l = warp_sum(ws.l[q]);
+    float* prow = parts + (warp * kMaxG + q) * kPartialStride;  // (m, l, -, -, o[128])
+    if (lane == 0) {
+      prow[0] = ws.m[q];
+      prow[1] = l;
+    }
+    // rows g, g + 8 of m-tile mt: channels 16g + mt, 16g + 8 + mt, value group g / 2
+    const int col = 4 * q + (g >> 1);
+    const float z = __shfl_sync(kFull, ws.z, col << 2);
+    if (tq == (col >> 1)) {
+      float v[16];
+#pragma unroll
+      for (int mt = 0; mt < 8; ++mt) {
+        const float f = code_unit<BITS>(BITS == 4 ? mt % 4 : mt) * kCodeUnit;
+        v[mt] = fmaf(((col & 1) ? ws.o[0][mt][1] : ws.o[0][mt][0]) * f, ws.vb, z);
+        v[8 + mt] = fmaf(((col & 1) ? ws.o[0][mt][3] : ws.o[0][mt][2]) * f, ws.vb, z);
+      }
+      float4* dst = reinterpret_cast<float4*>(prow + 4 + 16 * g);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
     }
   }
 }
@@ -1289,7 +1660,9 @@ __device__ __forceinline__ void locate_item(const DecodeParams& p, int x, int& l
   h = all ? n : nth_bit(prot ? mask : ~mask, n);
 }
 
-template <int BITS, int NT, int BASE, int MB>
+// NT: 8-query column tiles of the MMAs.  QC: queries per KV head where
+// run_item_cols serves the KIVI-style items (1 or 2), else 0.
+template <int BITS, int NT, int BASE, int MB, int QC>
 __global__ void __launch_bounds__(kThreads, NT == 1 ? 4 : 2)
 decode_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ __align__(1024) char smem_raw[];
@@ -1382,7 +1755,9 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
     sg.k_row0 = (int)((p.lt.base[li] + hd.kimg + b * hd.kimg_bs) >> 8);
     sg.vc = Lb + hd.vq + b * hd.vq_bs;
     sg.vm = Lb + hd.vqm + b * hd.vqm_bs;
-    if (BASE == kKivi)
+    if constexpr (QC > 0)
+      run_item_cols<BITS, QC, K_BF16, MB>(smem, sg, tb, te, p, qv, parts);
+    else if constexpr (BASE == kKivi)
       run_item<BITS, NT, K_BF16, V_KIVI, false, MB>(smem, sg, tb, te, p, qv, G, parts);
     else
       run_item<BITS, NT, K_BF16, V_TOKEN, false, MB>(smem, sg, tb, te, p, qv, G, parts);
@@ -1392,9 +1767,11 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
     sg.km = Lb + hd.kqm + b * hd.kqm_bs;
     sg.vc = Lb + hd.vq + b * hd.vq_bs;
     sg.vm = Lb + hd.vqm + b * hd.vqm_bs;
-    if (BASE == kKivi)
+    if constexpr (QC > 0)
+      run_item_cols<BITS, QC, K_KIVI, MB>(smem, sg, tb, te, p, qv, parts);
+    else if constexpr (BASE == kKivi)
       run_item<BITS, NT, K_KIVI, V_KIVI, false, MB>(smem, sg, tb, te, p, qv, G, parts);
-    else if (BASE == kAkvq)
+    else if constexpr (BASE == kAkvq)
       run_item<BITS, NT, K_TOKEN, V_TOKEN, true, MB>(smem, sg, tb, te, p, qv, G, parts);
     else
       run_item<BITS, NT, K_TOKEN, V_TOKEN, false, MB>(smem, sg, tb, te, p, qv, G, parts);
@@ -1453,7 +1830,7 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
   if (ni > 1 && tid == 0) atomicExch(p.counters + head_lin, 0u);
 }
 
-template <int BITS, int NT, int BASE, int MB>
+template <int BITS, int NT, int BASE, int MB, int QC>
 cudaError_t launch_t(const DecodeParams& p, int grid_x, cudaStream_t s) {
   // set once per device; host threads that race here both set the same
   // attributes, and the flags themselves are atomic
@@ -1462,11 +1839,11 @@ cudaError_t launch_t(const DecodeParams& p, int grid_x, cudaStream_t s) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev].load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(decode_kernel<BITS, NT, BASE, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(decode_kernel<BITS, NT, BASE, MB, QC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              SmemLayout<NT>::bytes);
     if (e != cudaSuccess) return e;
     // four CTAs of 54 KB share an SM: ask for the full shared-memory carve-out
-    e = cudaFuncSetAttribute(decode_kernel<BITS, NT, BASE, MB>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(decode_kernel<BITS, NT, BASE, MB, QC>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
@@ -1482,7 +1859,7 @@ cudaError_t launch_t(const DecodeParams& p, int grid_x, cudaStream_t s) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, decode_kernel<BITS, NT, BASE, MB>, p);
+  e = cudaLaunchKernelEx(&cfg, decode_kernel<BITS, NT, BASE, MB, QC>, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -1490,9 +1867,14 @@ cudaError_t launch_t(const DecodeParams& p, int grid_x, cudaStream_t s) {
 template <int BITS, int NT, int MB>
 cudaError_t launch_base(const DecodeParams& p, int grid_x, cudaStream_t s) {
   switch (p.d.base) {
-    case kKivi: return launch_t<BITS, NT, kKivi, MB>(p, grid_x, s);
-    case kAkvq: return launch_t<BITS, NT, kAkvq, MB>(p, grid_x, s);
-    default: return launch_t<BITS, NT, kMinMax, MB>(p, grid_x, s);
+    case kKivi:
+      if constexpr (NT == 1) {
+        if (p.d.G == 1) return launch_t<BITS, NT, kKivi, MB, 1>(p, grid_x, s);
+        if (p.d.G == 2) return launch_t<BITS, NT, kKivi, MB, 2>(p, grid_x, s);
+      }
+      return launch_t<BITS, NT, kKivi, MB, 0>(p, grid_x, s);
+    case kAkvq: return launch_t<BITS, NT, kAkvq, MB, 0>(p, grid_x, s);
+    default: return launch_t<BITS, NT, kMinMax, MB, 0>(p, grid_x, s);
   }
 }
 

@@ -219,7 +219,6 @@ HG_HD int head_chunks(int cls, const ChunkCounts& c, int* n_bf16) {
 // Position of the n-th set bit of m (n from 0; m has more than n set bits).
 HG_HD int nth_bit(uint64_t m, int n) {
   int pos = 0;
-#pragma unroll
   for (int w = 32; w >= 1; w >>= 1) {
     const int c = popc64(m & ((1ull << w) - 1ull));
     if (n >= c) {

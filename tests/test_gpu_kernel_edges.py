@@ -76,3 +76,55 @@ def test_decode_layers_with_different_appended_counts(base, keys_only, prefix):
         for row in range(w.batch):
             ref = _row_reference(runner, layer, row, *kept[layer], q, news[:n])
             assert_close(bits16(out[layer, row:row + 1]), ref, "layer %d row %d" % (layer, row))
+
+
+def _decode_against_oracle(w, kept, steps, q_scale=1.0, v_max=1.0):
+    """Append `steps` tokens in fused steps on a cache quantized from `kept`; the last step's outputs, every row.
+    The tolerance is the suite's (2e-3 + 1e-2 |r| for values of order one) with its absolute part in units of
+    the largest value: weights times value scales are FP16 products, so an output that cancels is off by up to
+    2^-11 of the values that went into it, whatever its own size."""
+    runner = CacheRunner(w)
+    hg.hg_quantize_kv(runner.cache, 0, [k for k, _ in kept], [v for _, v in kept])
+    news = []
+    for step in range(steps):
+        k_new, v_new = wl.step_new_kv(w, step, "cuda")
+        q = (wl.step_query(w, step, "cuda").float() * q_scale).bfloat16()
+        out = runner.decode_step(step, q=q, k_new=k_new, v_new=v_new)
+        news.append((k_new, v_new))
+    for layer in range(w.layers):
+        for row in range(w.batch):
+            ref = _row_reference(runner, layer, row, *kept[layer], q, news)
+            got = out[layer, row:row + 1].double().cpu().numpy()
+            err = np.abs(got - ref)
+            bad = ~(err <= 2e-3 * max(1.0, v_max) + 1e-2 * np.abs(ref))
+            assert not bad.any(), (w.name, layer, row, int(bad.sum()), float(err.max()))
+
+
+@pytest.mark.parametrize("meta_bits", [64, 32])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("group", [1, 2])
+def test_kivi_few_queries_per_head(group, bits, meta_bits):
+    """One or two queries per KV head over KIVI-style codes: a single 32-token group (half a tile), an odd
+    number of groups, and more than one tile per warp; quantized and keys-only heads."""
+    for image, keys_only in ((33, 1), (100, 0), (1000, 1)):
+        w = wl.custom("cols%d" % image, 1, 2, 4 * group, 4, 7, image, 37, wl.BASE_KIVI, bits, keys_only,
+                      decode_steps=2, seed=3, protected=[(0, 2)], meta_bits=meta_bits)
+        _decode_against_oracle(w, [wl.layer_kv(w, 0, "cuda")], 2)
+
+
+@pytest.mark.parametrize("base,bits,group", [(wl.BASE_KIVI, 2, 1), (wl.BASE_KIVI, 3, 2), (wl.BASE_KIVI, 4, 1),
+                                             (wl.BASE_MINMAX, 2, 4), (wl.BASE_MINMAX, 4, 12), (wl.BASE_AKVQ, 3, 7)])
+def test_decode_scales_over_many_binades(base, bits, group):
+    """Key and value scales that change by 2^16 between 32-token groups, grow along the sequence, vanish
+    (constant groups) and meet zero and large queries: the power-of-two units of the FP16 operands."""
+    w = wl.custom("binades", 1, 1, 2 * group, 2, 8, 640, 40, base, bits, 0, decode_steps=1, seed=9, protected=[])
+    g = torch.Generator(device="cuda").manual_seed(4)
+    e = torch.randint(-8, 9, (1, 2, w.seq_len // 32 + 1, 1), generator=g, device="cuda")
+    e = e.sort(dim=2).values.repeat_interleave(32, 2)[:, :, :w.seq_len].float()
+    k, v = wl.layer_kv(w, 0, "cuda")
+    k = (k.float() * torch.exp2(-2 - e.abs())).bfloat16()
+    v = (v.float() * torch.exp2(e)).bfloat16()
+    k[:, :, 104:136] = 0.25  # a constant group: scale 0
+    v[:, :, 200:232, 32:64] = -3.0
+    for q_scale in (0.0, 1.0, 512.0):
+        _decode_against_oracle(w, [(k, v)], 1, q_scale, float(v.abs().max()))
