@@ -36,6 +36,7 @@ struct DequantParams {
   int out_fp32;
   void* k_out;   // [n_layers][B][H][T + appended][128]
   void* v_out;
+  uint64_t neg_zero2;  // two fp32 -0 (see scale_add)
 };
 
 struct AppendParams {

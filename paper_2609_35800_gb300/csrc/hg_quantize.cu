@@ -13,6 +13,7 @@
 // (round half to even of the IEEE quotient, no contraction).
 #include <algorithm>
 #include <climits>
+#include <cmath>
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -1001,17 +1002,33 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __grid_const
 // ---------------------------------------------------------------------------
 // Reconstruction (Sec. 4: codes to floats, code * scale + zero; AKVQ-style keys
 // rotated back; BF16 entries copied), every layer of the launch in original
-// token order followed by the appended tokens.  One CTA per (32-token tile,
-// batch row, KV head, layer); a half-warp owns one token row of K or of V,
-// lane j of it channels 8j..8j+7, so every output row is one 256-byte (BF16)
-// or 512-byte (fp32) store of 16 lanes and each lane issues its code,
-// metadata and row loads independently (all four units of a thread at once).
-// A BF16 entry written as BF16 is copied as it is.  The AKVQ-style inverse rotation runs
-// its first three butterfly stages inside a lane and the last four across the
-// half-warp, in the same order as the forward transform.
+// token order followed by the appended tokens.  One CTA per span of 32-token
+// tiles of a (batch row, KV head, layer), tiles aligned with the image start;
+// warps 0-3 take eight rows each of K, warps 4-7 of V.  Almost every such run
+// of eight rows is of one kind -- coded tokens, or BF16 rows that lie one after
+// the other -- and is found so once per warp: its loads and stores are then at
+// constant strides from one address.  The rest (a run across a span's end, or
+// in an image span with salient tokens) resolve each row.
+//   Rows: a half-warp per row, lane j channels 8j..8j+7, the warp's eight rows
+// in flight together; a BF16 entry written as BF16 is copied as it is.
+//   KIVI-style keys: lane l has channels 4l..4l+3 of the group, reads their
+// words and metadata once and writes the warp's eight tokens from registers (a
+// half-warp per token instead read every word and pair of the group sixteen
+// times).
+// The AKVQ-style inverse rotation runs its first three butterfly stages inside
+// a lane and the last four across the half-warp, in the same order as the
+// forward transform.
+//
+// Before, every row found its own place (146 warp instructions per pair of
+// rows: issue-bound on small caches).  Qwen2.5-VL-7B-shaped, 28 layers: 30.8 ->
+// 22.6 us; a LLaVA-NeXT-7B-shaped layer of 16 rows: 378 -> 167 us, 0.98 of the
+// measured copy rate (BF16 output).
 // ---------------------------------------------------------------------------
 constexpr int kDqThreads = 256;
 constexpr int kDqTile = 32;
+constexpr int kDqRows = 8;   // rows of one warp in a tile
+// First token of the first tile (0 or less).
+HG_HD int dq_origin(const Dims& d) { return d.s % kDqTile ? d.s % kDqTile - kDqTile : 0; }
 
 // Two floats to BF16 bits (round to nearest even, low half first): one cvt.
 __device__ __forceinline__ uint32_t pack_bf16x2_rn(float lo, float hi) {
@@ -1026,98 +1043,61 @@ __device__ __forceinline__ void bf16x8_to_f32(const uint4& w, float (&x)[8]) {
   bf16x2_to_f32(w.w, x[6], x[7]);
 }
 
-// Codes of channels 8c..8c+7 of a per-token packed row (channel order; 3 bits:
-// the 2-bit half-word, then the plane byte of channels 8c..8c+7, which holds
-// them in order at byte ((c >> 1) & 1) | ((c & 1) << 1) of plane word c / 4).
-__device__ __forceinline__ void row_codes8(const uint32_t* row, int bits, int c, uint32_t (&code)[8]) {
-  if (bits == 4) {
-    const uint32_t w = __ldg(row + c);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) code[i] = (w >> (4 * i)) & 15u;
-    return;
-  }
-  const uint32_t half = (__ldg(row + (c >> 1)) >> (16 * (c & 1))) & 0xffffu;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) code[i] = (half >> (2 * i)) & 3u;
-  if (bits == 3) {
-    const uint32_t pl = __ldg(row + 8 + (c >> 2)) >> (8 * (((c >> 1) & 1) | ((c & 1) << 1)));
-#pragma unroll
-    for (int i = 0; i < 8; ++i) code[i] |= ((pl >> i) & 1u) << 2;
-  }
-}
-
-// Code of token e (0..31) of one KIVI-style key group row (one channel, token order).
-__device__ __forceinline__ uint32_t kivi_code(const uint32_t* row, int bits, int e) {
-  if (bits == 3) {
-    const uint32_t lo = (__ldg(row + e / 16) >> (2 * (e % 16))) & 3u;
-    const int pp = (e & 7) | (((e >> 4) & 1) << 3) | (((e >> 3) & 1) << 4);
-    return lo | (((__ldg(row + 2) >> pp) & 1u) << 2);
-  }
-  const int per = 32 / bits;
-  return (__ldg(row + e / per) >> (bits * (e % per))) & ((1u << bits) - 1u);
-}
-
-// Codes of token e of eight consecutive KIVI-style key rows (channels
-// 8j..8j+7: BITS words each, contiguous): at 2 and 3 bits the 16 or 24 words
-// arrive as 16-byte loads and each channel's word is selected in registers;
-// at 4 bits the one word a channel needs is loaded alone.
+// Codes of channels 8c..8c+7 of a per-token packed row: `lo` their 32 (4-bit)
+// or 16 (2- and 3-bit) low bits in channel order, `hi` (3 bits) the plane byte
+// of channels 8c..8c+7, which holds them in order at byte
+// ((c >> 1) & 1) | ((c & 1) << 1) of plane word c / 4.
+struct Codes8 {
+  uint32_t lo, hi;
+};
 template <int BITS>
-__device__ __forceinline__ void kivi_codes8(const uint32_t* rows, int e, uint32_t (&code)[8]) {
-  if constexpr (BITS == 4) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) code[i] = kivi_code(rows + i * BITS, BITS, e);
+__device__ __forceinline__ Codes8 load_codes8(const char* row, int c) {
+  Codes8 r = {0u, 0u};
+  if (BITS == 4) {
+    r.lo = __ldg(reinterpret_cast<const uint32_t*>(row) + c);
   } else {
-    uint32_t w[8 * BITS];
-#pragma unroll
-    for (int v = 0; v < 2 * BITS; ++v) {
-      const uint4 x = ldg16(rows + 4 * v);
-      w[4 * v] = x.x;
-      w[4 * v + 1] = x.y;
-      w[4 * v + 2] = x.z;
-      w[4 * v + 3] = x.w;
-    }
-    const bool hi = e >= 16;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t lo = ((hi ? w[i * BITS + 1] : w[i * BITS]) >> (2 * (e & 15))) & 3u;
-      if (BITS == 3) {
-        const int pp = (e & 7) | (((e >> 4) & 1) << 3) | (((e >> 3) & 1) << 4);
-        code[i] = lo | (((w[i * BITS + 2] >> pp) & 1u) << 2);
-      } else {
-        code[i] = lo;
-      }
-    }
+    r.lo = __ldg(reinterpret_cast<const uint16_t*>(row) + c);
+    if (BITS == 3)
+      r.hi = __ldg(reinterpret_cast<const uint8_t*>(row) + 32 + 4 * (c >> 2) + (((c >> 1) & 1) | ((c & 1) << 1)));
   }
+  return r;
 }
 
-// Metadata pairs of eight consecutive KIVI-style key rows from index i0 (a
-// multiple of 8, so 64 or 32 contiguous bytes on a 16-byte boundary).
-template <bool M16>
-__device__ __forceinline__ void kivi_meta8(const char* base, size_t i0, float2 (&m)[8]) {
-  if (M16) {
-    const uint4* p = reinterpret_cast<const uint4*>(base + i0 * 4);
+// The integer c < 2^23 as a float: 2^23 + c in the mantissa, less 2^23 (exact).
+__device__ __forceinline__ uint32_t int_magic(uint32_t c) { return c | 0x4B000000u; }
+__device__ __forceinline__ uint64_t magic_pair() { return f32x2(0x4B000000u, 0x4B000000u); }
+
+// fl(fl(x s) + z) of two elements.  The product is an FMA with nz = (-0, -0),
+// the same value: the compiler contracts a packed multiply and add, explicitly
+// rounded or not, into one FMA, so nz is a launch parameter it cannot see through.
+__device__ __forceinline__ uint64_t scale_add(uint64_t x, uint64_t s, uint64_t z, uint64_t nz) {
+  return f32x2_add(f32x2_fma(x, s, nz), z);
+}
+
+// fl(fl(code * scale) + zero) of eight codes.
+template <int BITS>
+__device__ __forceinline__ void dequant8(const Codes8& k, float scale, float zero, uint64_t nz, float (&x)[8]) {
+  const uint64_t s2 = f32x2(__float_as_uint(scale), __float_as_uint(scale));
+  const uint64_t z2 = f32x2(__float_as_uint(zero), __float_as_uint(zero));
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const uint4 x = __ldg(p + v);
-      m[4 * v] = half2_bits_to_float2(x.x);
-      m[4 * v + 1] = half2_bits_to_float2(x.y);
-      m[4 * v + 2] = half2_bits_to_float2(x.z);
-      m[4 * v + 3] = half2_bits_to_float2(x.w);
-    }
-  } else {
-    const float4* p = reinterpret_cast<const float4*>(base + i0 * 8);
+  for (int i = 0; i < 8; i += 2) {
+    uint32_t c[2];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const float4 x = __ldg(p + v);
-      m[2 * v] = make_float2(x.x, x.y);
-      m[2 * v + 1] = make_float2(x.z, x.w);
+    for (int e = 0; e < 2; ++e) {
+      c[e] = (k.lo >> ((BITS == 4 ? 4 : 2) * (i + e))) & (BITS == 4 ? 15u : 3u);
+      if (BITS == 3) c[e] |= ((k.hi >> (i + e)) & 1u) << 2;
     }
+    const uint64_t v = f32x2_sub(f32x2(int_magic(c[0]), int_magic(c[1])), magic_pair());
+    const uint64_t r = scale_add(v, s2, z2, nz);
+    x[i] = __uint_as_float((uint32_t)r);
+    x[i + 1] = __uint_as_float((uint32_t)(r >> 32));
   }
 }
 
 // Normalised Hadamard-128 of a vector spread over a half-warp, lane j holding
 // channels 8j..8j+7: stages h = 1, 2, 4 in the lane, h = 8..64 with lane
 // j ^ (h / 8); butterflies (a, b) -> (a + b, a - b), one multiply at the end.
+// (fma(x, +-1, p) is p + x or p - x, rounded once.)
 __device__ __forceinline__ void fwht128_half(float (&x)[8], int j) {
 #pragma unroll
   for (int h = 1; h < 8; h <<= 1) {
@@ -1131,141 +1111,231 @@ __device__ __forceinline__ void fwht128_half(float (&x)[8], int j) {
   }
 #pragma unroll
   for (int m = 1; m < 16; m <<= 1) {
-    const bool upper = (j & m) != 0;
+    const float sgn = (j & m) ? -1.f : 1.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float p = __shfl_xor_sync(kFull, x[i], m);
-      x[i] = upper ? __fsub_rn(p, x[i]) : __fadd_rn(x[i], p);
-    }
+    for (int i = 0; i < 8; ++i) x[i] = __fmaf_rn(x[i], sgn, __shfl_xor_sync(kFull, x[i], m));
   }
   const float c = hadamard_c();
 #pragma unroll
   for (int i = 0; i < 8; ++i) x[i] = __fmul_rn(x[i], c);
 }
 
+// Eight reconstructed channels, or the BF16 entry w (raw), to row element o
+// (this lane's first channel) of an output, where ok; called by whole warps.
+// fp32: lanes 2i and 2i + 1 exchange halves, so that each of the two stores
+// writes whole 32-byte sectors.
+__device__ __forceinline__ void store8(const DequantParams& p, void* dst, size_t o, bool raw, uint4 w, float (&x)[8],
+                                       bool ok = true) {
+  if (p.out_fp32) {
+    if (raw) bf16x8_to_f32(w, x);
+    const bool odd = threadIdx.x & 1;
+    float r[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = __shfl_xor_sync(kFull, odd ? x[i] : x[4 + i], 1);
+    float4* f = reinterpret_cast<float4*>(static_cast<float*>(dst) + (odd ? o - 4 : o));
+    if (ok) {
+      f[0] = odd ? make_float4(r[0], r[1], r[2], r[3]) : make_float4(x[0], x[1], x[2], x[3]);
+      f[2] = odd ? make_float4(x[4], x[5], x[6], x[7]) : make_float4(r[0], r[1], r[2], r[3]);
+    }
+  } else {
+    if (!raw)
+      w = make_uint4(pack_bf16x2_rn(x[0], x[1]), pack_bf16x2_rn(x[2], x[3]), pack_bf16x2_rn(x[4], x[5]),
+                     pack_bf16x2_rn(x[6], x[7]));
+    if (ok) *reinterpret_cast<uint4*>(static_cast<uint16_t*>(dst) + o) = w;
+  }
+}
+
+// Tokens 8u..8u+7 (u = 0..3, the warp's) of one KIVI-style key group: codes and
+// metadata of its 128 channels, first output element o (lane l: channels
+// 4l..4l+3 of each token).
+template <int BITS, bool M16>
+__device__ __forceinline__ void dequant_key_group(const DequantParams& p, const char* codes, const char* meta, int u,
+                                                  int lane, size_t o) {
+  // each channel's BITS words; the eight tokens' codes are in one half of a
+  // 2-bit word, or one 4-bit word, and at bits plane_bit + i of the 3-bit plane
+  const uint4* cw = reinterpret_cast<const uint4*>(codes) + lane * BITS;
+  uint32_t w[4 * BITS];
+#pragma unroll
+  for (int v = 0; v < BITS; ++v) {
+    const uint4 q = __ldg(cw + v);
+    w[4 * v] = q.x;
+    w[4 * v + 1] = q.y;
+    w[4 * v + 2] = q.z;
+    w[4 * v + 3] = q.w;
+  }
+  float2 m[4];
+  if (M16) {
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(meta) + lane);
+    m[0] = half2_bits_to_float2(q.x);
+    m[1] = half2_bits_to_float2(q.y);
+    m[2] = half2_bits_to_float2(q.z);
+    m[3] = half2_bits_to_float2(q.w);
+  } else {
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const float4 q = __ldg(reinterpret_cast<const float4*>(meta) + 2 * lane + v);
+      m[2 * v] = make_float2(q.x, q.y);
+      m[2 * v + 1] = make_float2(q.z, q.w);
+    }
+  }
+  Codes8 k[4];  // eight tokens of each channel, in the layout of a row's eight channels
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const uint32_t* x = w + c * BITS;
+    if (BITS == 4) {
+      k[c].lo = (u & 2) ? ((u & 1) ? x[3 % BITS] : x[2 % BITS]) : ((u & 1) ? x[1] : x[0]);
+    } else {
+      k[c].lo = ((u & 2) ? x[1] : x[0]) >> (16 * (u & 1));
+      // token 8u + i: index bits 3 and 4 (of u) exchanged
+      if (BITS == 3) k[c].hi = x[2 % BITS] >> (8 * ((u >> 1) | ((u & 1) << 1)));
+    }
+  }
+  const uint64_t s01 = f32x2(__float_as_uint(m[0].x), __float_as_uint(m[1].x));
+  const uint64_t s23 = f32x2(__float_as_uint(m[2].x), __float_as_uint(m[3].x));
+  const uint64_t z01 = f32x2(__float_as_uint(m[0].y), __float_as_uint(m[1].y));
+  const uint64_t z23 = f32x2(__float_as_uint(m[2].y), __float_as_uint(m[3].y));
+#pragma unroll
+  for (int i = 0; i < kDqRows; ++i) {
+    uint32_t c[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      c[e] = (k[e].lo >> ((BITS == 4 ? 4 : 2) * i)) & (BITS == 4 ? 15u : 3u);
+      if (BITS == 3) c[e] |= ((k[e].hi >> i) & 1u) << 2;
+    }
+    const uint64_t a = scale_add(f32x2_sub(f32x2(int_magic(c[0]), int_magic(c[1])), magic_pair()), s01, z01, p.neg_zero2);
+    const uint64_t b = scale_add(f32x2_sub(f32x2(int_magic(c[2]), int_magic(c[3])), magic_pair()), s23, z23, p.neg_zero2);
+    const size_t e0 = o + (size_t)i * kD + 4 * lane;
+    if (p.out_fp32)
+      *reinterpret_cast<float4*>(static_cast<float*>(p.k_out) + e0) =
+          make_float4(pair_lo(a), pair_hi(a), pair_lo(b), pair_hi(b));
+    else
+      *reinterpret_cast<uint2*>(static_cast<uint16_t*>(p.k_out) + e0) =
+          make_uint2(pack_bf16x2_rn(pair_lo(a), pair_hi(a)), pack_bf16x2_rn(pair_lo(b), pair_hi(b)));
+  }
+}
+
 // BITS, BASE and M16 are compile-time, so each (code width, base, metadata
-// width) runs code of its own; a CTA takes a span of consecutive tiles of one
-// (row, head, layer), so the head's region map and its barrier are paid once
-// per span.
+// width) runs code of its own.
 template <int BITS, int BASE, bool M16>
 __global__ void __launch_bounds__(kDqThreads, 6) dequantize_kernel(const __grid_constant__ DequantParams p) {
   const Dims& d = p.d;
   const int li = blockIdx.z, bh = blockIdx.y;
   const int b = bh / d.H, h = bh % d.H;
   const int Tt = d.T + p.appended;
-  // the head's region map, computed once for the CTA (64-bit arithmetic that
-  // would otherwise cost every warp more instructions than its four units)
+  // the head's region map, computed once for the CTA (64-bit arithmetic)
   __shared__ HeadGeom s_hd;
   if (threadIdx.x == 0) s_hd = head_geom(d, layer_geom(d, p.lt.mask[li]), h);
   __syncthreads();
   const HeadGeom& hd = s_hd;
+  const int cls = hd.cls;
+  const int warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const bool is_k = warp < 4;
+  const int j = lane & 15, hw = lane >> 4;  // a half-warp's row: channels 8j..8j+7
   const char* Lb = p.arena + p.lt.base[li];
   const int qs = d.s, qe = d.s + d.nq;
-  constexpr int W = kD * BITS / 32;
-  const int j = threadIdx.x & 15;  // channels 8j..8j+7
-  const size_t out_row0 = (((size_t)li * d.B + b) * d.H + h) * (size_t)Tt;
-  const int ntiles = (Tt + kDqTile - 1) / kDqTile;
+  constexpr int CB = kD * BITS / 8;  // code bytes of a token
+  constexpr int MB = M16 ? 4 : 8;
+  constexpr int VG = BASE == kKivi ? 4 : 1;
+  const bool has_salient = BASE == kAkvq && d.ns > 0 && cls != kProtected;
+  // this warp's operand: BF16 rows, and codes + metadata (or the keys-only
+  // head's BF16 image keys) of the coded tokens
+  const char* rows = Lb + (is_k ? hd.kb : hd.vb) + b * hd.kb_bs;
+  const bool coded_here = cls != kProtected && !(is_k && cls == kKeysOnly);
+  const char* img = Lb + hd.kimg + b * hd.kimg_bs;  // keys-only heads
+  const char* codes = Lb + (is_k ? hd.kq : hd.vq) + b * (is_k ? hd.kq_bs : hd.vq_bs);
+  const char* meta = Lb + (is_k ? hd.kqm : hd.vqm) + b * (is_k ? hd.kqm_bs : hd.vqm_bs);
+  void* out = is_k ? p.k_out : p.v_out;
+  const size_t out0 = (((size_t)li * d.B + b) * d.H + h) * (size_t)Tt * kD;
+  const int shift = cls == kProtected ? 0 : d.nq - d.ns;  // token - position of the rows past the image
+  const int origin = dq_origin(d);
+  const int ntiles = (Tt - origin + kDqTile - 1) / kDqTile;
   const int span = (ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
   const int x1 = min(((int)blockIdx.x + 1) * span, ntiles);
 
 #pragma unroll 1
   for (int x = blockIdx.x * span; x < x1; ++x) {
-    // a thread's two tokens (rows 16 apart), each with its K and V unit: the
-    // token's coded slot and BF16 position found once for both
-    int tk[2], ck[2], pk[2];
-    bool codedk[2], salk[2];
+    const int a = origin + x * kDqTile + (warp & 3) * kDqRows, e = a + kDqRows;  // the warp's tokens [a, e)
+    if (e <= 0 || a >= Tt) continue;
+    const bool whole = a >= 0 && e <= Tt;
+    const bool in_image = a >= qs && e <= qe, outside = cls == kProtected || e <= qs || a >= qe;
+    // ---- eight BF16 rows one after the other ----
+    if (whole && (outside || (in_image && !coded_here && !has_salient))) {
+      const char* src = (outside ? rows + (size_t)(a >= qe ? a - shift : a) * 256 : img + (size_t)(a - qs) * 256) +
+                        hw * 256 + j * 16;
+      uint4 w[kDqRows / 2];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int t = x * kDqTile + ((threadIdx.x >> 4) + 16 * r);
-      const bool coded = (t >= qs) && (t < qe);
-      const int ti = t - qs;
-      int ci = ti, spos = 0;  // coded slot; BF16 position of a salient token (Sec. 4)
-      bool sal = false;
-      if (BASE == kAkvq && coded && d.ns > 0 && hd.cls != kProtected) {
+      for (int i = 0; i < kDqRows / 2; ++i) w[i] = ldg16(src + i * 512);
+      const size_t o = out0 + (size_t)(a + hw) * kD + 8 * j;
+#pragma unroll
+      for (int i = 0; i < kDqRows / 2; ++i) {
+        float x8[8];
+        store8(p, out, o + i * 2 * kD, true, w[i], x8);
+      }
+      continue;
+    }
+    // ---- eight coded tokens ----
+    if (whole && in_image && coded_here && !has_salient) {
+      const int ti = a - qs;
+      if (BASE == kKivi && is_k) {
+        const int grp = ti / kKiviGroup;
+        dequant_key_group<BITS, M16>(p, codes + (size_t)grp * (kD * BITS * 4), meta + (size_t)grp * (kD * MB),
+                                     (ti >> 3) & 3, lane, out0 + (size_t)a * kD);
+        continue;
+      }
+      Codes8 c[kDqRows / 2];
+      float2 m[kDqRows / 2];
+      const char* cr = codes + (size_t)(ti + hw) * CB;
+      const char* mr = meta + ((size_t)(ti + hw) * VG + (BASE == kKivi ? (j >> 2) : 0)) * MB;
+#pragma unroll
+      for (int i = 0; i < kDqRows / 2; ++i) {
+        c[i] = load_codes8<BITS>(cr + i * 2 * CB, j);
+        m[i] = load_meta(mr + i * 2 * VG * MB, 0, M16);
+      }
+      const size_t o = out0 + (size_t)(a + hw) * kD + 8 * j;
+#pragma unroll
+      for (int i = 0; i < kDqRows / 2; ++i) {
+        float x8[8];
+        dequant8<BITS>(c[i], m[i].x, m[i].y, p.neg_zero2, x8);
+        if (BASE == kAkvq && is_k) fwht128_half(x8, j);  // inverse rotation (H is self-inverse)
+        store8(p, out, o + i * 2 * kD, false, make_uint4(0u, 0u, 0u, 0u), x8);
+      }
+      continue;
+    }
+    // ---- each row for itself; two rows' loads in flight per lane ----
+#pragma unroll 2
+    for (int i = 0; i < kDqRows / 2; ++i) {
+      const int t = a + 2 * i + hw;
+      const bool ok = t >= 0 && t < Tt;
+      bool coded = t >= qs && t < qe;  // an image token: code, BF16 image key, or salient
+      int ci = t - qs, pos = (t < qs || cls == kProtected) ? t : t - shift;
+      if (has_salient && ok && coded) {
         const char* sm = Lb + hd.sal + b * hd.sal_bs;
-        const int w = ti >> 5, e = ti & 31;
+        const int w = ci >> 5, k = ci & 31;
         const uint32_t sb = __ldg(reinterpret_cast<const uint32_t*>(sm) + w);
         const int rank = __ldg(reinterpret_cast<const int*>(sm + (size_t)sal_blocks(d) * 4) + w) +
-                         __popc(sb & ((1u << e) - 1u));
-        sal = (sb >> e) & 1u;
-        ci = ti - rank;
-        spos = qs + rank;
+                         __popc(sb & ((1u << k) - 1u));
+        if ((sb >> k) & 1u) {
+          coded = false;
+          pos = qs + rank;
+        }
+        ci -= rank;
       }
-      tk[r] = t;
-      ck[r] = ci;
-      codedk[r] = coded;
-      salk[r] = sal;
-      pk[r] = (t >= d.T) ? hd.bf16_prefill + (t - d.T) : (sal ? spos : bf16_pos(d, hd.cls, t));
-    }
-    // unit u: K (u < 16 * kDqTile) or V, token (u >> 4) % kDqTile of the
-    // tile; unrolled so that the loads of a thread's four units are in flight
-    // together
-#pragma unroll
-    for (int u = threadIdx.x; u < 2 * kDqTile * 16; u += kDqThreads) {
-      const bool is_k = u < kDqTile * 16;
-      const int r = ((u - threadIdx.x) / kDqThreads) & 1;  // the thread's token of this unit
-      const int t = tk[r];
-      if (t >= Tt) continue;  // uniform over the half-warp
-      const bool coded = codedk[r], sal = salk[r];
-      const int ti = t - qs, ci = ck[r], pos = pk[r];
-      const size_t o = (out_row0 + t) * kD + 8 * j;
-      void* dst = is_k ? p.k_out : p.v_out;
-      float x8[8];
-      bool raw = false;  // a BF16 entry: `w` holds its 16 bytes
+      const bool code = coded && coded_here;
       uint4 w = make_uint4(0u, 0u, 0u, 0u);
-      if (is_k) {
-        if (coded && hd.cls == kQuantized && !sal) {
-          uint32_t code[8];
-          float2 m[8];
-          if (BASE == kKivi) {
-            const int grp = ti / kKiviGroup, e = ti % kKiviGroup;
-            const uint32_t* codes = reinterpret_cast<const uint32_t*>(Lb + hd.kq + b * hd.kq_bs) +
-                                    ((size_t)grp * kD + 8 * j) * BITS;
-            kivi_codes8<BITS>(codes, e, code);
-            kivi_meta8<M16>(Lb + hd.kqm + b * hd.kqm_bs, (size_t)grp * kD + 8 * j, m);
-          } else {
-            row_codes8(reinterpret_cast<const uint32_t*>(Lb + hd.kq + b * hd.kq_bs) + (size_t)ci * W, BITS, j,
-                       code);
-            const float2 m0 = load_meta(Lb + hd.kqm + b * hd.kqm_bs, ci, M16);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) m[i] = m0;
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) x8[i] = dequant1(code[i], m[i].x, m[i].y);
-          if (BASE == kAkvq) fwht128_half(x8, j);  // inverse rotation (H is self-inverse)
-        } else {
-          const char* src = (coded && hd.cls == kKeysOnly && !sal)
-                                ? Lb + hd.kimg + b * hd.kimg_bs + (size_t)ci * 256
-                                : Lb + hd.kb + b * hd.kb_bs + (size_t)pos * 256;
-          w = ldg16(src + j * 16);
-          raw = true;
-        }
-      } else {
-        if (coded && hd.cls != kProtected && !sal) {
-          uint32_t code[8];
-          row_codes8(reinterpret_cast<const uint32_t*>(Lb + hd.vq + b * hd.vq_bs) + (size_t)ci * W, BITS, j,
-                     code);
-          // KIVI-style: 32-channel groups, channels 8j.. in group j / 4
-          const float2 m = load_meta(Lb + hd.vqm + b * hd.vqm_bs,
-                                     (size_t)ci * vgroups(d) + (BASE == kKivi ? (j >> 2) : 0), M16);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) x8[i] = dequant1(code[i], m.x, m.y);
-        } else {
-          w = ldg16(Lb + hd.vb + b * hd.kb_bs + (size_t)pos * 256 + j * 16);
-          raw = true;
+      Codes8 c = {0u, 0u};
+      float2 m = make_float2(0.f, 0.f);
+      if (ok) {
+        if (!code) {
+          w = ldg16(((coded && cls == kKeysOnly) ? img + (size_t)ci * 256 : rows + (size_t)pos * 256) + j * 16);
+        } else if (!(BASE == kKivi && is_k)) {
+          c = load_codes8<BITS>(codes + (size_t)ci * CB, j);
+          m = load_meta(meta, (size_t)ci * VG + (BASE == kKivi ? (j >> 2) : 0), M16);
         }
       }
-      if (p.out_fp32) {
-        if (raw) bf16x8_to_f32(w, x8);
-        float4* f = reinterpret_cast<float4*>(static_cast<float*>(dst) + o);
-        f[0] = make_float4(x8[0], x8[1], x8[2], x8[3]);
-        f[1] = make_float4(x8[4], x8[5], x8[6], x8[7]);
-      } else {
-        if (!raw)
-          w = make_uint4(pack_bf16x2_rn(x8[0], x8[1]), pack_bf16x2_rn(x8[2], x8[3]),
-                         pack_bf16x2_rn(x8[4], x8[5]), pack_bf16x2_rn(x8[6], x8[7]));
-        *reinterpret_cast<uint4*>(static_cast<uint16_t*>(dst) + o) = w;
-      }
+      float x8[8];
+      dequant8<BITS>(c, m.x, m.y, p.neg_zero2, x8);
+      if (BASE == kAkvq && is_k) fwht128_half(x8, j);  // by every lane: rows that are not coded drop it
+      store8(p, out, out0 + (size_t)t * kD + 8 * j, !code, w, x8, ok);
     }
   }
 }
@@ -1361,12 +1431,21 @@ cudaError_t launch_dequantize_bits(const DequantParams& p, dim3 grid, cudaStream
 
 cudaError_t launch_dequantize(const DequantParams& p, int sm_count, cudaStream_t s) {
   const int Tt = p.d.T + p.appended;
-  const int ntiles = (Tt + kDqTile - 1) / kDqTile;
-  // spans of several tiles once the grid holds more than 16 waves of 6 CTAs
-  // per SM (at most 8 tiles a CTA)
-  const long long groups = (long long)p.d.B * p.d.H * p.n_layers;
-  const long long waves16 = 16LL * 6 * (sm_count > 0 ? sm_count : 1);
-  const int span = (int)std::max(1LL, std::min(8LL, groups * ntiles / waves16));
+  const int ntiles = (Tt - dq_origin(p.d) + kDqTile - 1) / kDqTile;
+  // Tiles per CTA (1 to 4): whole waves of 6 CTAs per SM, each as long as its
+  // tiles and a start worth 0.4 of one.  (Qwen2.5-VL-7B-shaped, 28 layers: 24.7
+  // us with one tile per CTA, 22.6 with two; a LLaVA-NeXT-7B-shaped layer of 16
+  // rows 179 us with two, 175 with four, 179 with eight.)
+  const double groups = (double)p.d.B * p.d.H * p.n_layers, wave = 6.0 * (sm_count > 0 ? sm_count : 1);
+  int span = 1;
+  double best = 0.0;
+  for (int n = 1; n <= 4; ++n) {
+    const double t = std::ceil(groups * ((ntiles + n - 1) / n) / wave) * (n + 0.4);
+    if (n == 1 || t < best) {
+      best = t;
+      span = n;
+    }
+  }
   dim3 grid((ntiles + span - 1) / span, p.d.B * p.d.H, p.n_layers);
   if (p.d.bits == 2) return launch_dequantize_bits<2>(p, grid, s);
   if (p.d.bits == 3) return launch_dequantize_bits<3>(p, grid, s);

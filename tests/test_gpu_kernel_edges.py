@@ -11,6 +11,7 @@ from paper_2609_35800_gb300 import workloads as wl
 from paper_2609_35800_gb300.runner import CacheRunner
 
 from parity import assert_close, attention_reference, bits16, n_salient
+from test_gpu_parity import _dequantize_bit_exact
 
 pytestmark = pytest.mark.gpu
 
@@ -128,3 +129,14 @@ def test_decode_scales_over_many_binades(base, bits, group):
     v[:, :, 200:232, 32:64] = -3.0
     for q_scale in (0.0, 1.0, 512.0):
         _decode_against_oracle(w, [(k, v)], 1, q_scale, float(v.abs().max()))
+
+
+@pytest.mark.parametrize("meta_bits", [64, 32])
+@pytest.mark.parametrize("base,bits,salient", [(wl.BASE_MINMAX, 3, 0), (wl.BASE_KIVI, 2, 0), (wl.BASE_KIVI, 3, 0),
+                                               (wl.BASE_KIVI, 4, 0), (wl.BASE_AKVQ, 2, 0), (wl.BASE_AKVQ, 4, 30)])
+@pytest.mark.parametrize("prefix,image,suffix", [(0, 1, 0), (3, 2, 1), (31, 33, 0), (1, 40, 64), (33, 257, 5)])
+def test_dequantize_run_edges(prefix, image, suffix, base, bits, salient, meta_bits):
+    """Eight-row runs that straddle the start, the image span's end and the last token, bit for bit."""
+    w = wl.custom("runs", 2, 1, 4, 2, prefix, image, suffix, base, bits, int(image == 33), seed=2,
+                  protected=[(0, 1)], residual=0, meta_bits=meta_bits, salient_permille=salient)
+    _dequantize_bit_exact(w)
