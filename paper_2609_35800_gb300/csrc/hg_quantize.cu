@@ -847,53 +847,88 @@ __global__ void __launch_bounds__(32) quantize_tiles_kernel(const __grid_constan
 }
 
 // ---------------------------------------------------------------------------
-// AKVQ-style salient tokens (Sec. 4): one CTA per (batch row, KV head, layer);
-// protected K+V heads (no coded image entries) return.  Squared key norms of the
-// image tokens in the fixed binary32 order (a warp per token: lane l sums
-// channels 4l..4l+3, then five butterfly rounds of pairwise sums), ns rounds
-// of a CTA-wide arg-max (largest score, ties to the lower index), then the
-// map: a bit per image token and the salient count before each 32-token block.
+// AKVQ-style salient tokens (Sec. 4), two launches; protected K+V heads (no
+// coded image entries) are left out.  First the squared key norms of the image
+// tokens in the fixed binary32 order (32 partial sums of channels 4l..4l+3, then
+// five butterfly rounds): a half-warp per row, eight rows per warp in flight,
+// CTAs of 64 tokens over the whole GPU; the scores go to the head's own code
+// (or BF16) rows, which the quantizer fills after the selection.  Then one CTA
+// per (batch row, KV head, layer) selects the ns largest scores (ties to the
+// lower index) and writes the map: a bit per image token and the salient count
+// before each 32-token block.
+//
+// One CTA per head for both read the keys with 8 KB in flight: 88 us for a
+// layer of 32 rows, 8 KV heads and 3,328 image tokens (191 MB of keys read, 28 us
+// at the measured copy rate); now 33 us and 12 us.
 // ---------------------------------------------------------------------------
-constexpr int kSalThreads = 256;
+constexpr int kNormThreads = 256, kNormRows = 8, kNormTokens = kNormThreads / 32 * kNormRows;
+constexpr int kSalThreads = 512;
 
-__global__ void __launch_bounds__(kSalThreads) salient_kernel(const __grid_constant__ QuantizeParams p) {
+// Where the scores of one row of a head with coded values wait for the
+// selection: its value codes, or its BF16 rows when nearly every token is
+// salient (nc tokens of 16 BITS bytes, ns of 256, for nc + ns scores of 4).
+__device__ __forceinline__ float* salient_scores(const Dims& d, const HeadGeom& hd, char* Lb, int b) {
+  const bool codes = (long long)ncoded(d) * 16 * d.bits >= (long long)d.nq * 4;
+  return reinterpret_cast<float*>(codes ? Lb + hd.vq + b * hd.vq_bs : Lb + hd.kb + b * hd.kb_bs);
+}
+
+__global__ void __launch_bounds__(kNormThreads) salient_norm_kernel(const __grid_constant__ QuantizeParams p) {
+  const Dims& d = p.d;
+  const int li = blockIdx.z, b = blockIdx.y / d.H, h = blockIdx.y % d.H;
+  if (head_class(d, p.lt.mask[li], h) == kProtected) return;
+  const int lane = threadIdx.x & 31, j = lane & 15;
+  const int r0 = blockIdx.x * kNormTokens + (threadIdx.x >> 5) * kNormRows + (lane >> 4);
+  const uint16_t* K = p.k[li] + (((size_t)b * d.H + h) * d.T + d.s) * kD + 8 * j;
+  uint4 w[kNormRows / 2];
+#pragma unroll
+  for (int i = 0; i < kNormRows / 2; ++i) {
+    const int r = r0 + 2 * i;
+    w[i] = r < d.nq ? ldg16(K + (size_t)r * kD) : make_uint4(0u, 0u, 0u, 0u);
+  }
+  __shared__ float* s_out;
+  if (threadIdx.x == 0)
+    s_out = salient_scores(d, head_geom(d, layer_geom(d, p.lt.mask[li]), h), p.arena + p.lt.base[li], b);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kNormRows / 2; ++i) {
+    // partial sums 2j and 2j + 1; round m of the butterfly is lane j ^ (m / 2),
+    // the last one inside the lane
+    float a[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      float x[4];
+      bf16x4_to_f32(e ? make_uint2(w[i].z, w[i].w) : make_uint2(w[i].x, w[i].y), x);
+      a[e] = __fmul_rn(x[0], x[0]);
+      a[e] = __fadd_rn(a[e], __fmul_rn(x[1], x[1]));
+      a[e] = __fadd_rn(a[e], __fmul_rn(x[2], x[2]));
+      a[e] = __fadd_rn(a[e], __fmul_rn(x[3], x[3]));
+    }
+#pragma unroll
+    for (int m = 8; m >= 1; m >>= 1) {
+      a[0] = __fadd_rn(a[0], __shfl_xor_sync(kFull, a[0], m));
+      a[1] = __fadd_rn(a[1], __shfl_xor_sync(kFull, a[1], m));
+    }
+    const int r = r0 + 2 * i;
+    if (j == 0 && r < d.nq) s_out[r] = __fadd_rn(a[0], a[1]);
+  }
+}
+
+__global__ void __launch_bounds__(kSalThreads) salient_select_kernel(const __grid_constant__ QuantizeParams p) {
   const Dims& d = p.d;
   const int bh = blockIdx.x, li = blockIdx.y;
   const int b = bh / d.H, h = bh % d.H;
-  const LayerGeom g = layer_geom(d, p.lt.mask[li]);
-  const HeadGeom hd = head_geom(d, g, h);
-  if (hd.cls == kProtected || d.ns <= 0) return;
+  if (head_class(d, p.lt.mask[li], h) == kProtected) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nq = d.nq, nblk = sal_blocks(d);
   extern __shared__ __align__(16) float sal_smem[];
   float* score = sal_smem;                                     // [nq]
   uint32_t* bits = reinterpret_cast<uint32_t*>(sal_smem + nq);  // [nblk]
-
-  const uint16_t* K = p.k[li] + (((size_t)b * d.H + h) * d.T + d.s) * kD;
-  // four rows per warp in flight: their loads first, then each row's sum in
-  // the same order as one row at a time
-  constexpr int kRows = 4, kWarps = kSalThreads / 32;
-  for (int i0 = warp; i0 < nq; i0 += kRows * kWarps) {
-    uint2 w[kRows];
-#pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      const int i = i0 + u * kWarps;
-      w[u] = (i < nq) ? ldg8(K + (size_t)i * kD + lane * 4) : make_uint2(0u, 0u);
-    }
-#pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      const int i = i0 + u * kWarps;
-      float x[4];
-      bf16x4_to_f32(w[u], x);
-      float a = __fmul_rn(x[0], x[0]);
-      a = __fadd_rn(a, __fmul_rn(x[1], x[1]));
-      a = __fadd_rn(a, __fmul_rn(x[2], x[2]));
-      a = __fadd_rn(a, __fmul_rn(x[3], x[3]));
-#pragma unroll
-      for (int m = 16; m >= 1; m >>= 1) a = __fadd_rn(a, __shfl_xor_sync(kFull, a, m));
-      if (lane == 0 && i < nq) score[i] = a;
-    }
-  }
+  __shared__ HeadGeom s_hd;
+  if (tid == 0) s_hd = head_geom(d, layer_geom(d, p.lt.mask[li]), h);
+  __syncthreads();
+  const HeadGeom& hd = s_hd;
+  const float* src = salient_scores(d, hd, p.arena + p.lt.base[li], b);
+  for (int i = tid; i < nq; i += kSalThreads) score[i] = src[i];
   __syncthreads();
 
   // The ns largest scores, ties to the lower index -- the set that ns rounds
@@ -903,14 +938,14 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __grid_const
   // match the digits chosen so far and the digit where the count of larger
   // keys reaches ns.  Then every key above the final threshold T is taken,
   // and of the keys equal to T the first `need` by index.
-  static_assert(kSalThreads == 256, "one histogram bin per thread");
+  static_assert(kSalThreads >= 256, "a thread per histogram bin");
   __shared__ uint32_t hist[256];
   __shared__ uint32_t s_prefix, s_need, s_eq;
   uint32_t prefix = 0u, pmask = 0u, need = (uint32_t)d.ns;
 #pragma unroll 1
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
-    hist[tid] = 0u;  // kSalThreads == 256 bins
+    if (tid < 256) hist[tid] = 0u;
     __syncthreads();
     for (int i0 = warp * 32; i0 < nq; i0 += kSalThreads) {  // warp-uniform: lane i0 + lane
       const int i = i0 + lane;
@@ -990,11 +1025,18 @@ __global__ void __launch_bounds__(kSalThreads) salient_kernel(const __grid_const
   uint32_t* out_bits = reinterpret_cast<uint32_t*>(dst);
   int* out_rank = reinterpret_cast<int*>(dst + (size_t)nblk * 4);
   for (int w = tid; w < nblk; w += kSalThreads) out_bits[w] = bits[w];
-  if (tid == 0) {
-    int acc = 0;
-    for (int w = 0; w < nblk; ++w) {
-      out_rank[w] = acc;
-      acc += __popc(bits[w]);
+  if (warp == 0) {
+    int before = 0;
+    for (int w0 = 0; w0 < nblk; w0 += 32) {
+      const int c = w0 + lane < nblk ? __popc(bits[w0 + lane]) : 0;
+      int incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (w0 + lane < nblk) out_rank[w0 + lane] = before + incl - c;
+      before += __shfl_sync(kFull, incl, 31);
     }
   }
 }
@@ -1404,11 +1446,14 @@ cudaError_t launch_salient(const QuantizeParams& p, cudaStream_t s) {
   const size_t smem = salient_smem_bytes(p.d);
   if (smem > 48 * 1024) {
     const cudaError_t e =
-        cudaFuncSetAttribute(salient_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(salient_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  dim3 grid(p.d.B * p.d.H, p.n_layers, 1);
-  salient_kernel<<<grid, kSalThreads, smem, s>>>(p);
+  const unsigned heads = (unsigned)(p.d.B * p.d.H), layers = (unsigned)p.n_layers;
+  salient_norm_kernel<<<dim3((p.d.nq + kNormTokens - 1) / kNormTokens, heads, layers), kNormThreads, 0, s>>>(p);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  salient_select_kernel<<<dim3(heads, layers, 1), kSalThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
 

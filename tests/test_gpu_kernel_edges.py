@@ -11,7 +11,7 @@ from paper_2609_35800_gb300 import workloads as wl
 from paper_2609_35800_gb300.runner import CacheRunner
 
 from parity import assert_close, attention_reference, bits16, n_salient
-from test_gpu_parity import _dequantize_bit_exact
+from test_gpu_parity import _dequantize_bit_exact, _run_and_check
 
 pytestmark = pytest.mark.gpu
 
@@ -140,3 +140,13 @@ def test_dequantize_run_edges(prefix, image, suffix, base, bits, salient, meta_b
     w = wl.custom("runs", 2, 1, 4, 2, prefix, image, suffix, base, bits, int(image == 33), seed=2,
                   protected=[(0, 1)], residual=0, meta_bits=meta_bits, salient_permille=salient)
     _dequantize_bit_exact(w)
+
+
+@pytest.mark.parametrize("bits,permille,image", [(2, 10, 63), (2, 500, 65), (2, 870, 129), (2, 880, 128), (3, 930, 200),
+                                                 (4, 930, 200), (4, 970, 96), (2, 1000, 33)])
+def test_salient_scores_beside_codes_or_rows(bits, permille, image):
+    """The selection's scores wait in the head's value codes, or in its BF16 rows when the coded tokens are too
+    few to hold them: both sides of the line, spans around the 64 tokens of a block; keys-only heads too."""
+    w = wl.custom("scores", 2, 2, 8, 4, 5, image, 9, wl.BASE_AKVQ, bits, 1, decode_steps=1, seed=6,
+                  protected=[(0, 1), (1, 2)], salient_permille=permille)
+    _run_and_check(w)
