@@ -27,6 +27,8 @@ struct hg_cache {
   Dims d;
   std::vector<uint64_t> layer_mask;
   std::vector<uint64_t> layer_base;
+  std::vector<LayerOffsets> layer_off;
+  GeomConsts gc;
   std::vector<int> appended;
   char* arena;
   size_t arena_bytes;
@@ -452,6 +454,8 @@ hg_status hg_cache_create(const hg_shape* shape, const hg_quant_config* config,
     delete c;
     return HG_ERR_ARENA_TOO_SMALL;
   }
+  for (uint64_t m : c->layer_mask) c->layer_off.push_back(layer_offsets(layer_geom(d, m)));
+  c->gc = geom_consts(d);
   c->appended.assign(d.L, 0);
   c->arena = static_cast<char*>(arena);
   c->arena_bytes = arena_bytes;
@@ -519,7 +523,9 @@ hg_status hg_quantize_kv(hg_cache* c, int32_t layer_begin, int32_t layer_count,
     p.n_layers = n;
     p.tile_origin = d.s % 32;
     fill_table(c, layer_begin + done, n, &p.lt);
+    p.gt.gc = c->gc;
     for (int i = 0; i < n; ++i) {
+      p.gt.off[i] = c->layer_off[layer_begin + done + i];
       p.k[i] = static_cast<const uint16_t*>(k[done + i]);
       p.v[i] = static_cast<const uint16_t*>(v[done + i]);
     }

@@ -16,6 +16,13 @@ struct LayerTable {
   uint64_t base[kMaxLayersPerLaunch];
   uint64_t mask[kMaxLayersPerLaunch];
 };
+// Strides and region offsets for head_geom_at (the quantizer's launches; where a
+// CTA works for microseconds on one head, reading them cost more than the
+// arithmetic they save: per-layer decode launches 2%, reconstruction 3%).
+struct GeomTable {
+  GeomConsts gc;
+  LayerOffsets off[kMaxLayersPerLaunch];
+};
 
 struct QuantizeParams {
   Dims d;
@@ -23,6 +30,7 @@ struct QuantizeParams {
   int n_layers;
   int tile_origin;  // s mod 32: KIVI-style tile i covers [tile_origin - 32 + 64 i, +64) clipped to [0, T)
   LayerTable lt;
+  GeomTable gt;
   const uint16_t* k[kMaxLayersPerLaunch];
   const uint16_t* v[kMaxLayersPerLaunch];
 };

@@ -171,6 +171,74 @@ HG_HD HeadGeom head_geom(const Dims& d, const LayerGeom& g, int h) {
   return r;
 }
 
+// The same for kernels, from quantities of the launch that the host works out
+// once: per layer the region offsets, per cache the strides.  A head is then a
+// few multiply-adds on uniform values (layer_geom and head_geom take some 300
+// instructions, most of them 64-bit products, which a one-warp CTA of the
+// quantizer spent on every 32 rows).
+struct LayerOffsets {
+  uint64_t kb, vb, kq, kqm, vq, vqm, kimg, sal;  // from the layer's base
+};
+struct GeomConsts {
+  uint64_t kq_bs, kqm_bs, vqm_bs, kimg_bs, sal_bs;                   // per batch row (vq_bs is kq_bs)
+  uint64_t kq_head, kqm_head, vqm_head, kimg_head, sal_head;         // per head with the region
+  uint64_t bf16_head, bf16_extra;  // BF16 bytes of a head, and of a protected K+V head beyond that
+  int bf16_U, cap_U, extra;        // BF16 prefill tokens and capacity of a head, tokens beyond that
+};
+
+HG_HD LayerOffsets layer_offsets(const LayerGeom& g) {
+  return {g.kb, g.vb, g.kq, g.kqm, g.vq, g.vqm, g.kimg, g.sal};
+}
+
+HG_HD GeomConsts geom_consts(const Dims& d) {
+  GeomConsts c;
+  const uint64_t B = (uint64_t)d.B, nc = (uint64_t)ncoded(d);
+  c.kq_bs = nc * code_bytes_per_token(d);
+  c.kqm_bs = kmeta_stride(d);
+  c.vqm_bs = vmeta_stride(d);
+  c.kimg_bs = nc * kD * 2;
+  c.sal_bs = sal_stride(d);
+  c.kq_head = B * c.kq_bs;
+  c.kqm_head = B * c.kqm_bs;
+  c.vqm_head = B * c.vqm_bs;
+  c.kimg_head = B * c.kimg_bs;
+  c.sal_head = B * c.sal_bs;
+  c.bf16_head = B * (uint64_t)cap_unprot(d) * kD * 2;
+  c.bf16_extra = B * nc * kD * 2;
+  c.bf16_U = d.T - d.nq + d.ns;
+  c.cap_U = cap_unprot(d);
+  c.extra = (int)nc;
+  return c;
+}
+
+HG_HD HeadGeom head_geom_at(const Dims& d, const GeomConsts& c, const LayerOffsets& o, uint64_t mask, int h) {
+  HeadGeom r;
+  const int prot_below = popc64(mask & ((1ull << h) - 1ull));
+  const uint32_t pkv_below = d.keys_only ? 0u : (uint32_t)prot_below;
+  const uint32_t u = (uint32_t)(h - prot_below), vr = d.keys_only ? (uint32_t)h : u;
+  r.cls = head_class(d, mask, h);
+  const int more = (r.cls == kProtected) ? c.extra : 0;
+  r.bf16_prefill = c.bf16_U + more;
+  r.cap = c.cap_U + more;
+  r.kb_bs = (uint64_t)(uint32_t)r.cap * (kD * 2);
+  const uint64_t rows = (uint32_t)h * c.bf16_head + pkv_below * c.bf16_extra;
+  r.kb = o.kb + rows;
+  r.vb = o.vb + rows;
+  r.kq_bs = r.vq_bs = c.kq_bs;
+  r.kqm_bs = c.kqm_bs;
+  r.vqm_bs = c.vqm_bs;
+  r.kimg_bs = c.kimg_bs;
+  r.sal_bs = c.sal_bs;
+  // regions the head does not have are not looked at
+  r.kq = o.kq + u * c.kq_head;
+  r.kqm = o.kqm + u * c.kqm_head;
+  r.vq = o.vq + vr * c.kq_head;
+  r.vqm = o.vqm + vr * c.vqm_head;
+  r.kimg = o.kimg + (uint32_t)prot_below * c.kimg_head;
+  r.sal = o.sal + vr * c.sal_head;
+  return r;
+}
+
 // Position of prefill token t in a head's BF16 region, or -1 when the token is
 // an image token of a head whose image tokens are coded (the salient ones of
 // a quantized head sit at d.s + their rank among the salient tokens; the

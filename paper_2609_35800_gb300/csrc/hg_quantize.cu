@@ -633,6 +633,11 @@ __device__ __forceinline__ void copy_rows_warp(char* dst, const StagedRows& rows
   }
 }
 
+// Region map of KV head h of the launch's layer li.
+__device__ __forceinline__ HeadGeom quantize_head(const QuantizeParams& p, int li, int h) {
+  return head_geom_at(p.d, p.gt.gc, p.gt.off[li], p.lt.mask[li], h);
+}
+
 // Token span of a tile: rows r < n hold tokens t0 + r.
 struct TileSpan {
   int t0, n, tlo;  // tlo: the unclipped tile start (KIVI-style tiles)
@@ -830,7 +835,6 @@ struct KiviTiles {
 template <class TP>
 __global__ void __launch_bounds__(32) quantize_tiles_kernel(const __grid_constant__ QuantizeParams p) {
   __shared__ __align__(16) StagedRows rows;
-  __shared__ HeadGeom s_hd;
   const int pi = blockIdx.x % TP::kNParts, tx = blockIdx.x / TP::kNParts;
   const int li = blockIdx.z, b = blockIdx.y / p.d.H, h = blockIdx.y % p.d.H;
   const int kv = TP::part(pi);
@@ -838,12 +842,10 @@ __global__ void __launch_bounds__(32) quantize_tiles_kernel(const __grid_constan
   if (sp.n <= 0) return;
   stage_rows(p, li, b, h, kv, sp, rows);
   cp_async_commit();
-  // the head's region map, once for the CTA while its copies are in flight
-  // (64-bit arithmetic that would otherwise run in every thread)
-  if (threadIdx.x == 0) s_hd = head_geom(p.d, layer_geom(p.d, p.lt.mask[li]), h);
+  const HeadGeom hd = quantize_head(p, li, h);
   cp_async_wait<0>();
   __syncwarp();
-  TP::process(p, li, b, kv, sp, rows, s_hd);
+  TP::process(p, li, b, kv, sp, rows, hd);
 }
 
 // ---------------------------------------------------------------------------
@@ -863,6 +865,11 @@ __global__ void __launch_bounds__(32) quantize_tiles_kernel(const __grid_constan
 // ---------------------------------------------------------------------------
 constexpr int kNormThreads = 256, kNormRows = 8, kNormTokens = kNormThreads / 32 * kNormRows;
 constexpr int kSalThreads = 512;
+// Spans up to this length: the selection's CTA sums the norms itself, one
+// launch (a layer of 8 heads in 4 rows, prefill in one and two launches before
+// the quantizer's: 26.8 and 27.3 us with 512 image tokens, 38.9 and 34.3 with
+// 1,024; 256 heads: 56.1 and 59.9, 85.9 and 85.4).
+constexpr int kSalOneLaunch = 512;
 
 // Where the scores of one row of a head with coded values wait for the
 // selection: its value codes, or its BF16 rows when nearly every token is
@@ -870,6 +877,28 @@ constexpr int kSalThreads = 512;
 __device__ __forceinline__ float* salient_scores(const Dims& d, const HeadGeom& hd, char* Lb, int b) {
   const bool codes = (long long)ncoded(d) * 16 * d.bits >= (long long)d.nq * 4;
   return reinterpret_cast<float*>(codes ? Lb + hd.vq + b * hd.vq_bs : Lb + hd.kb + b * hd.kb_bs);
+}
+
+// Squared norm of the key whose channels 8j..8j+7 lane j of a half-warp holds
+// (in its lane 0), in the fixed order: partial sums 2j and 2j + 1, round m of
+// the butterfly with lane j ^ (m / 2), the last one inside the lane.
+__device__ __forceinline__ float key_norm2(const uint4& w) {
+  float a[2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    float x[4];
+    bf16x4_to_f32(e ? make_uint2(w.z, w.w) : make_uint2(w.x, w.y), x);
+    a[e] = __fmul_rn(x[0], x[0]);
+    a[e] = __fadd_rn(a[e], __fmul_rn(x[1], x[1]));
+    a[e] = __fadd_rn(a[e], __fmul_rn(x[2], x[2]));
+    a[e] = __fadd_rn(a[e], __fmul_rn(x[3], x[3]));
+  }
+#pragma unroll
+  for (int m = 8; m >= 1; m >>= 1) {
+    a[0] = __fadd_rn(a[0], __shfl_xor_sync(kFull, a[0], m));
+    a[1] = __fadd_rn(a[1], __shfl_xor_sync(kFull, a[1], m));
+  }
+  return __fadd_rn(a[0], a[1]);
 }
 
 __global__ void __launch_bounds__(kNormThreads) salient_norm_kernel(const __grid_constant__ QuantizeParams p) {
@@ -885,34 +914,16 @@ __global__ void __launch_bounds__(kNormThreads) salient_norm_kernel(const __grid
     const int r = r0 + 2 * i;
     w[i] = r < d.nq ? ldg16(K + (size_t)r * kD) : make_uint4(0u, 0u, 0u, 0u);
   }
-  __shared__ float* s_out;
-  if (threadIdx.x == 0)
-    s_out = salient_scores(d, head_geom(d, layer_geom(d, p.lt.mask[li]), h), p.arena + p.lt.base[li], b);
-  __syncthreads();
+  float* out = salient_scores(d, quantize_head(p, li, h), p.arena + p.lt.base[li], b);
 #pragma unroll
   for (int i = 0; i < kNormRows / 2; ++i) {
-    // partial sums 2j and 2j + 1; round m of the butterfly is lane j ^ (m / 2),
-    // the last one inside the lane
-    float a[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      float x[4];
-      bf16x4_to_f32(e ? make_uint2(w[i].z, w[i].w) : make_uint2(w[i].x, w[i].y), x);
-      a[e] = __fmul_rn(x[0], x[0]);
-      a[e] = __fadd_rn(a[e], __fmul_rn(x[1], x[1]));
-      a[e] = __fadd_rn(a[e], __fmul_rn(x[2], x[2]));
-      a[e] = __fadd_rn(a[e], __fmul_rn(x[3], x[3]));
-    }
-#pragma unroll
-    for (int m = 8; m >= 1; m >>= 1) {
-      a[0] = __fadd_rn(a[0], __shfl_xor_sync(kFull, a[0], m));
-      a[1] = __fadd_rn(a[1], __shfl_xor_sync(kFull, a[1], m));
-    }
+    const float norm = key_norm2(w[i]);
     const int r = r0 + 2 * i;
-    if (j == 0 && r < d.nq) s_out[r] = __fadd_rn(a[0], a[1]);
+    if (j == 0 && r < d.nq) out[r] = norm;
   }
 }
 
+template <bool NORMS>
 __global__ void __launch_bounds__(kSalThreads) salient_select_kernel(const __grid_constant__ QuantizeParams p) {
   const Dims& d = p.d;
   const int bh = blockIdx.x, li = blockIdx.y;
@@ -923,12 +934,28 @@ __global__ void __launch_bounds__(kSalThreads) salient_select_kernel(const __gri
   extern __shared__ __align__(16) float sal_smem[];
   float* score = sal_smem;                                     // [nq]
   uint32_t* bits = reinterpret_cast<uint32_t*>(sal_smem + nq);  // [nblk]
-  __shared__ HeadGeom s_hd;
-  if (tid == 0) s_hd = head_geom(d, layer_geom(d, p.lt.mask[li]), h);
-  __syncthreads();
-  const HeadGeom& hd = s_hd;
-  const float* src = salient_scores(d, hd, p.arena + p.lt.base[li], b);
-  for (int i = tid; i < nq; i += kSalThreads) score[i] = src[i];
+  const HeadGeom hd = quantize_head(p, li, h);
+  if (NORMS) {
+    const uint16_t* K = p.k[li] + (((size_t)b * d.H + h) * d.T + d.s) * kD + 8 * (lane & 15);
+    constexpr int kStep = kSalThreads / 16;  // rows of one sweep, four sweeps in flight
+    for (int r0 = tid >> 4; r0 - (lane >> 4) < nq; r0 += 4 * kStep) {  // whole warps
+      uint4 w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = r0 + i * kStep;
+        w[i] = r < nq ? ldg16(K + (size_t)r * kD) : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = r0 + i * kStep;
+        const float norm = key_norm2(w[i]);
+        if ((lane & 15) == 0 && r < nq) score[r] = norm;
+      }
+    }
+  } else {
+    const float* src = salient_scores(d, hd, p.arena + p.lt.base[li], b);
+    for (int i = tid; i < nq; i += kSalThreads) score[i] = src[i];
+  }
   __syncthreads();
 
   // The ns largest scores, ties to the lower index -- the set that ns rounds
@@ -1442,19 +1469,25 @@ cudaError_t launch_quantize(const QuantizeParams& p, cudaStream_t s) {
   return m16 ? launch_quantize_bits<4, true>(p, s) : launch_quantize_bits<4, false>(p, s);
 }
 
-cudaError_t launch_salient(const QuantizeParams& p, cudaStream_t s) {
+template <bool NORMS>
+cudaError_t launch_salient_select(const QuantizeParams& p, cudaStream_t s) {
   const size_t smem = salient_smem_bytes(p.d);
   if (smem > 48 * 1024) {
     const cudaError_t e =
-        cudaFuncSetAttribute(salient_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(salient_select_kernel<NORMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  const unsigned heads = (unsigned)(p.d.B * p.d.H), layers = (unsigned)p.n_layers;
-  salient_norm_kernel<<<dim3((p.d.nq + kNormTokens - 1) / kNormTokens, heads, layers), kNormThreads, 0, s>>>(p);
+  salient_select_kernel<NORMS><<<dim3((unsigned)(p.d.B * p.d.H), (unsigned)p.n_layers, 1), kSalThreads, smem, s>>>(p);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_salient(const QuantizeParams& p, cudaStream_t s) {
+  if (p.d.nq <= kSalOneLaunch) return launch_salient_select<true>(p, s);
+  salient_norm_kernel<<<dim3((p.d.nq + kNormTokens - 1) / kNormTokens, (unsigned)(p.d.B * p.d.H), (unsigned)p.n_layers),
+                        kNormThreads, 0, s>>>(p);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  salient_select_kernel<<<dim3(heads, layers, 1), kSalThreads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_salient_select<false>(p, s);
 }
 
 template <int BITS, int BASE, bool M16>

@@ -150,3 +150,11 @@ def test_salient_scores_beside_codes_or_rows(bits, permille, image):
     w = wl.custom("scores", 2, 2, 8, 4, 5, image, 9, wl.BASE_AKVQ, bits, 1, decode_steps=1, seed=6,
                   protected=[(0, 1), (1, 2)], salient_permille=permille)
     _run_and_check(w)
+
+
+@pytest.mark.parametrize("image", [511, 512, 513])
+def test_salient_selection_in_one_or_two_launches(image):
+    """Around the span length up to which the selection sums the key norms itself."""
+    w = wl.custom("launches", 1, 2, 8, 4, 6, image, 9, wl.BASE_AKVQ, 4, 0, decode_steps=1, seed=8,
+                  protected=[(0, 1)], salient_permille=20)
+    _run_and_check(w)
