@@ -10,7 +10,7 @@ import paper_2609_35800_gb300 as hg
 from paper_2609_35800_gb300 import workloads as wl
 from paper_2609_35800_gb300.runner import CacheRunner
 
-from parity import assert_close, attention_reference, bits16, n_salient
+from parity import assert_close, attention_reference, bits16, check_arena_layer, n_salient, oracle_layer
 from test_gpu_parity import _dequantize_bit_exact, _run_and_check
 
 pytestmark = pytest.mark.gpu
@@ -158,3 +158,36 @@ def test_salient_selection_in_one_or_two_launches(image):
     w = wl.custom("launches", 1, 2, 8, 4, 6, image, 9, wl.BASE_AKVQ, 4, 0, decode_steps=1, seed=8,
                   protected=[(0, 1)], salient_permille=20)
     _run_and_check(w)
+
+
+@pytest.mark.parametrize("meta_bits", [64, 32])
+@pytest.mark.parametrize("base", [wl.BASE_MINMAX, wl.BASE_KIVI, wl.BASE_AKVQ])
+def test_two_bit_codes_by_comparison(base, meta_bits):
+    """2-bit groups for the comparison rule and around what it leaves to the general one, bit for bit: one
+    sign, boundaries at and next to zero and on BF16 values, signed zeros, constants, steps too small and too
+    large, values many binades apart."""
+    w = wl.custom("compare", 1, 1, 4, 2, 0, 32 * 14, 0, base, 2, 0, seed=12, protected=[], residual=0,
+                  meta_bits=meta_bits)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r = torch.randn(14, 2, 2, 32, 128, generator=g, device="cuda")
+    r[0] = r[0].abs() + 0.01
+    r[1] = -r[1].abs() - 0.01
+    r[2] = torch.where(r[2] > 0, 1.5, -1.5)                                   # middle boundary at zero
+    r[3, ..., ::2], r[3, ..., 1::2] = -3.0, 3.0078125                         # ... and next to it
+    r[4] = torch.randint(-6, 7, r[4].shape, generator=g, device="cuda") * 0.5  # quotients on half-integers
+    r[5] = torch.where(r[5] > 0, 0.0, -0.0)
+    r[6] = 0.375
+    r[7] *= 1e-36
+    r[8] *= 1e36
+    r[9] *= torch.exp2(torch.randint(-30, 30, r[9].shape, generator=g, device="cuda").float())
+    r[10] = torch.where(r[10].abs() < 1, r[10] * 1e-4, r[10])                 # many values around zero
+    r[11] = r[11] * 0.01 + 100.0
+    r[12] = r[12] * 0.01 - 100.0
+    r[13, ..., :] = torch.linspace(-1.0, 2.0, 128, device="cuda")
+    k = r[:, 0].permute(1, 0, 2, 3).reshape(1, 2, -1, 128).bfloat16().contiguous()
+    v = r[:, 1].permute(1, 0, 2, 3).reshape(1, 2, -1, 128).bfloat16().contiguous()
+    k, v = k.clone(), v.clone()
+    runner = CacheRunner(w)
+    hg.hg_quantize_kv(runner.cache, 0, [k], [v])
+    torch.cuda.synchronize()
+    check_arena_layer(runner, 0, bits16(k), bits16(v), oracle_layer(runner, 0, bits16(k), bits16(v)))
