@@ -11,6 +11,7 @@ the compute functions without the built library raises.
 """
 import ctypes
 import os
+import struct
 
 from . import build as _build
 
@@ -132,6 +133,19 @@ def _devs(where, *specs):
     first -- and live on a CUDA device; an int is taken as a raw device
     address whose extent the caller vouches for, None as a null pointer
     (which the library rejects)."""
+    out = []
+    for x, nbytes, _ in specs:
+        if x is None or isinstance(x, int):
+            out.append(x)
+        elif x.is_cuda and x.is_contiguous() and x.nbytes >= nbytes:
+            out.append(x.data_ptr())
+        else:
+            _refuse(where, specs)
+    return out
+
+
+def _refuse(where, specs):
+    """Raise for the first argument that _devs does not take."""
     for x, nbytes, name in specs:
         if x is None or isinstance(x, int):
             continue
@@ -144,14 +158,13 @@ def _devs(where, *specs):
     for x, _, name in specs:
         if x is not None and not isinstance(x, int) and not x.is_cuda:
             raise ValueError("%s: %s must be a CUDA tensor" % (where, name))
-    return [x if (x is None or isinstance(x, int)) else x.data_ptr() for x, _, _ in specs]
 
 
 def _extent(cache, *dims, elem=2):
     """Bytes of a dense [dims...][head_dim] array of `elem`-byte entries."""
     n = elem * cache.shape.head_dim
     for d in dims:
-        n *= max(int(d), 0)
+        n *= int(d) if d > 0 else 0
     return n
 
 
@@ -159,6 +172,8 @@ def _stream(stream):
     """cudaStream_t handle: a torch.cuda.Stream, an int, or None (current torch stream)."""
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():  # the handle alone, without a Stream object around it
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -238,12 +253,18 @@ def hg_quantize_kv(cache, layer_begin, k_list, v_list, stream=None):
         raise ValueError("hg_quantize_kv: %d key and %d value tensors" % (n, len(v_list)))
     sh = cache.shape
     need = _extent(cache, sh.batch, sh.num_kv_heads, sh.seq_len)
-    ptrs = _devs("hg_quantize_kv", *([(k, need, "k[%d]" % i) for i, k in enumerate(k_list)] +
-                                     [(v, need, "v[%d]" % i) for i, v in enumerate(v_list)]))
-    karr = (ctypes.c_void_p * n)(*ptrs[:n])
-    varr = (ctypes.c_void_p * n)(*ptrs[n:])
-    _check(library().hg_quantize_kv(cache.handle, layer_begin, n, karr, varr, _stream(stream)),
-           "hg_quantize_kv")
+    ptrs = []
+    for x in (*k_list, *v_list):
+        if x is None or isinstance(x, int):
+            ptrs.append(x or 0)
+        elif x.is_cuda and x.is_contiguous() and x.nbytes >= need:
+            ptrs.append(x.data_ptr())
+        else:
+            _refuse("hg_quantize_kv", [(k, need, "k[%d]" % i) for i, k in enumerate(k_list)] +
+                    [(v, need, "v[%d]" % i) for i, v in enumerate(v_list)])
+    # two arrays of n pointers, as bytes
+    _check(library().hg_quantize_kv(cache.handle, layer_begin, n, struct.pack("%dQ" % n, *ptrs[:n]),
+                                    struct.pack("%dQ" % n, *ptrs[n:]), _stream(stream)), "hg_quantize_kv")
 
 
 def hg_dequantize_kv(cache, layer_begin, layer_count, k_out, v_out, out_fp32, stream=None):
@@ -317,7 +338,7 @@ def hg_select_heads(g_scores, o_scores, num_layers, num_q_heads, num_kv_heads, k
 def hg_decode_attention(cache, layer_begin, layer_count, q, out, softmax_scale, workspace,
                         workspace_bytes=None, stream=None):
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
+        workspace_bytes = workspace.nbytes
     sh = cache.shape
     need = _extent(cache, layer_count, sh.batch, sh.num_q_heads)
     qp, op, wp = _devs("hg_decode_attention", (q, need, "q"), (out, need, "out"),
@@ -331,10 +352,10 @@ def hg_decode_step(cache, layer_begin, layer_count, q, k_new, v_new, out, softma
                    workspace_bytes=None, stream=None):
     """Append the step's K/V and run decode attention including it, in one launch."""
     if workspace_bytes is None:
-        workspace_bytes = workspace.numel() * workspace.element_size()
+        workspace_bytes = workspace.nbytes
     sh = cache.shape
-    nq = _extent(cache, layer_count, sh.batch, sh.num_q_heads)
-    nkv = _extent(cache, layer_count, sh.batch, sh.num_kv_heads)
+    per = _extent(cache, layer_count, sh.batch)
+    nq, nkv = per * sh.num_q_heads, per * sh.num_kv_heads
     qp, kp, vp, op, wp = _devs("hg_decode_step", (q, nq, "q"), (k_new, nkv, "k_new"),
                                (v_new, nkv, "v_new"), (out, nq, "out"),
                                (workspace, workspace_bytes, "workspace"))

@@ -35,6 +35,8 @@ struct hg_cache {
   size_t needed_bytes;
   // The arena as a BF16 tensor [arena_bytes / 256][128] for the decode
   // kernel's TMA loads; encoded by the first decode call.
+  mutable int least_layers = 0, least_sms = 0;  // decode_least_workspace's last answer
+  mutable size_t least_bytes = 0;
   mutable CUtensorMap arena_map;
   mutable bool arena_map_ready;
 };
@@ -670,12 +672,18 @@ int fill_runs(const Dims& d, const HeadCounts& hc, DecodeParams* p) {
   return total;
 }
 
+// The work plans of a call's first launch (usually its only one).
+struct Planned {
+  DecodePlan plan, least;
+};
+
 // Decode attention over layers [layer_begin, +layer_count); with k_new / v_new
 // the step's new tokens (already counted in the cache's appended state) are
 // read from the inputs and stored into the arena by the same launch.
+// planned: what decode_checks worked out.
 hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_count, const void* q,
                         const void* k_new, const void* v_new, void* out, float softmax_scale,
-                        void* ws, size_t ws_bytes_given, hg_stream_t stream) {
+                        void* ws, size_t ws_bytes_given, const Planned& planned, hg_stream_t stream) {
   const Dims& d = c->d;
   const hg_status mst = arena_tensor_map(c);
   if (mst != HG_OK) return mst;
@@ -689,9 +697,9 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     p.d = d;
     p.arena = c->arena;
     p.n_layers = n;
-    DecodePlan least;
-    p.plan = plan_decode(c, layer_begin + done, n, &least);
-    if (plan_ws_bytes(d, n, p.plan) > ws_bytes_given) p.plan = least;
+    Planned pl = planned;
+    if (done > 0) pl.plan = plan_decode(c, layer_begin + done, n, &pl.least);
+    p.plan = plan_ws_bytes(d, n, pl.plan) <= ws_bytes_given ? pl.plan : pl.least;
     p.max_items = max_items_of(d, p.plan);
     p.scale_log2 = scale * 1.4426950408889634f;
     p.q = static_cast<const uint16_t*>(q) + (size_t)done * layer_elems;
@@ -726,13 +734,16 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
 }
 
 hg_status decode_checks(const hg_cache* c, int32_t layer_begin, int32_t layer_count, const void* q,
-                        void* out, float softmax_scale, void* ws, size_t ws_bytes_given) {
+                        void* out, float softmax_scale, void* ws, size_t ws_bytes_given, Planned* planned) {
   if (!range_ok(c, layer_begin, layer_count) || !q || !out || !ws) return HG_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(out) || !aligned16(ws)) return HG_ERR_ALIGNMENT;
   if (!(softmax_scale == softmax_scale)) return HG_ERR_INVALID_ARG;  // NaN
   for (int done = 0; done < layer_count; done += kMaxLayersPerLaunch) {
     const int n = std::min(kMaxLayersPerLaunch, layer_count - done);
-    if (ws_bytes_given < ws_least_for(c, layer_begin + done, n)) return HG_ERR_WORKSPACE_TOO_SMALL;
+    Planned pl;
+    pl.plan = plan_decode(c, layer_begin + done, n, &pl.least);
+    if (ws_bytes_given < plan_ws_bytes(c->d, n, pl.least)) return HG_ERR_WORKSPACE_TOO_SMALL;
+    if (done == 0) *planned = pl;
   }
   return HG_OK;
 }
@@ -744,16 +755,18 @@ extern "C" {
 hg_status hg_decode_attention(const hg_cache* c, int32_t layer_begin, int32_t layer_count,
                               const void* q, void* out, float softmax_scale, void* ws,
                               size_t ws_bytes_given, hg_stream_t stream) {
-  const hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given);
+  Planned planned;
+  const hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given, &planned);
   if (st != HG_OK) return st;
   return decode_launch(c, layer_begin, layer_count, q, nullptr, nullptr, out, softmax_scale, ws,
-                       ws_bytes_given, stream);
+                       ws_bytes_given, planned, stream);
 }
 
 hg_status hg_decode_step(hg_cache* c, int32_t layer_begin, int32_t layer_count, const void* q,
                          const void* k_new, const void* v_new, void* out, float softmax_scale,
                          void* ws, size_t ws_bytes_given, hg_stream_t stream) {
-  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given);
+  Planned planned;
+  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given, &planned);
   if (st != HG_OK) return st;
   if (!k_new || !v_new) return HG_ERR_INVALID_ARG;
   if (!aligned16(k_new) || !aligned16(v_new)) return HG_ERR_ALIGNMENT;
@@ -761,7 +774,7 @@ hg_status hg_decode_step(hg_cache* c, int32_t layer_begin, int32_t layer_count, 
     if (c->appended[layer_begin + i] >= c->d.S_new) return HG_ERR_CAPACITY;
   for (int i = 0; i < layer_count; ++i) c->appended[layer_begin + i] += 1;
   st = decode_launch(c, layer_begin, layer_count, q, k_new, v_new, out, softmax_scale, ws,
-                     ws_bytes_given, stream);
+                     ws_bytes_given, planned, stream);
   if (st != HG_OK)
     for (int i = 0; i < layer_count; ++i) c->appended[layer_begin + i] -= 1;
   return st;
@@ -772,13 +785,25 @@ hg_status hg_decode_step(hg_cache* c, int32_t layer_begin, int32_t layer_count, 
 namespace hg {
 
 hg_status decode_least_workspace(const hg_cache* c, int32_t layer_count, size_t* bytes) {
-  return workspace_bound(c, layer_count, bytes, ws_least_for);
+  // a plan per placement of the range: kept for the count asked last
+  if (c && c->least_layers == layer_count && c->least_sms == sm_count()) {
+    *bytes = c->least_bytes;
+    return HG_OK;
+  }
+  const hg_status st = workspace_bound(c, layer_count, bytes, ws_least_for);
+  if (st == HG_OK) {
+    c->least_layers = layer_count;
+    c->least_sms = sm_count();
+    c->least_bytes = *bytes;
+  }
+  return st;
 }
 
 hg_status decode_attention_on_scratch(const hg_cache* c, int32_t layer_begin, int32_t layer_count,
                                       const void* q, void* out, float softmax_scale, void* scratch,
                                       size_t scratch_bytes, hg_stream_t stream) {
-  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, scratch, scratch_bytes);
+  Planned planned;
+  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, scratch, scratch_bytes, &planned);
   if (st != HG_OK) return st;
   st = arena_tensor_map(c);
   if (st != HG_OK) return st;
@@ -789,7 +814,7 @@ hg_status decode_attention_on_scratch(const hg_cache* c, int32_t layer_begin, in
                       reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
     return HG_ERR_CUDA;
   return decode_launch(c, layer_begin, layer_count, q, nullptr, nullptr, out, softmax_scale, scratch,
-                       scratch_bytes, stream);
+                       scratch_bytes, planned, stream);
 }
 
 }  // namespace hg
