@@ -312,7 +312,7 @@ hg_status hg_decode_step(hg_cache *cache, int32_t layer_begin, int32_t layer_cou
  *             the array's device address with cudaGetSymbolAddress; make that
  *             first call before any stream capture.
  *   Sharing   every call uses the same array and clears its split counters
- *             (cudaMemsetAsync) before launching; calls that overlap on the
+ *             (a small kernel) before launching; calls that overlap on the
  *             GPU (different streams, or threads on the same device) race.
  *   Errors    the argument checks and the size limit run before anything is
  *             enqueued.  A bounded wait that runs out (see Errors above) sets

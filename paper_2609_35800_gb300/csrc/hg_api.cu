@@ -810,9 +810,9 @@ hg_status decode_attention_on_scratch(const hg_cache* c, int32_t layer_begin, in
   // launches over more than kMaxLayersPerLaunch layers reuse the counters of
   // the first group, and every launch leaves them at zero again
   const size_t counters = ws_counter_bytes(c->d, std::min<int>(layer_count, kMaxLayersPerLaunch));
-  if (cudaMemsetAsync(static_cast<char*>(scratch) + kWsHeaderBytes, 0, counters,
-                      reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return HG_ERR_CUDA;
+  st = cuda_status(launch_clear(static_cast<char*>(scratch) + kWsHeaderBytes, counters,
+                                reinterpret_cast<cudaStream_t>(stream)));
+  if (st != HG_OK) return st;
   return decode_launch(c, layer_begin, layer_count, q, nullptr, nullptr, out, softmax_scale, scratch,
                        scratch_bytes, planned, stream);
 }

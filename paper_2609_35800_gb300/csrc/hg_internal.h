@@ -125,6 +125,9 @@ constexpr size_t kMaxSalientSmem = 200 * 1024;
 // Reconstruction of the launch's layers; sm_count sizes the tile spans.
 cudaError_t launch_dequantize(const DequantParams& p, int sm_count, cudaStream_t s);
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s);
+// Zero `bytes` (a multiple of 16, 16-byte aligned) in stream order, as a
+// programmatic dependent launch (a memset between two would serialise them).
+cudaError_t launch_clear(void* words, size_t bytes, cudaStream_t s);
 cudaError_t launch_decode(const DecodeParams& p, int grid_x, cudaStream_t s);
 cudaError_t launch_wait_probe(uint32_t* result, uint32_t rounds, cudaStream_t s);
 // The decode kernels for binary16 metadata pairs (called by launch_decode).

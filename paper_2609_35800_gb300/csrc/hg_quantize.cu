@@ -1602,8 +1602,14 @@ __global__ void __launch_bounds__(kDqThreads, 6) dequantize_kernel(const __grid_
   }
 }
 
-// One decode token per (layer, row, head) into the head's BF16 region.
+// One decode token per (layer, row, head) into the head's BF16 region.  Part of
+// the programmatic dependent launches of a decode loop: the next launch may be
+// scheduled at once, and everything before the first store comes from the
+// launch parameters.  Appending and attending without a workspace, layer by
+// layer (append, clear, decode: 6 layers of 5 KV heads, 2 tokens): 246 -> 182 us
+// with the three overlapping; before, append and a memset each ran alone.
 __global__ void __launch_bounds__(64) append_kernel(const __grid_constant__ AppendParams p) {
+  grid_launch_dependents();
   const Dims& d = p.d;
   const int li = blockIdx.x, bh = blockIdx.y;
   const int b = bh / d.H, h = bh % d.H;
@@ -1613,13 +1619,17 @@ __global__ void __launch_bounds__(64) append_kernel(const __grid_constant__ Appe
   const int pos = hd.bf16_prefill + p.appended[li];
   const size_t src = (((size_t)li * d.B + b) * d.H + h) * kD;
   const int lane = threadIdx.x & 31;
-  if (threadIdx.x < 32) {
-    *reinterpret_cast<uint2*>(Lb + hd.kb + b * hd.kb_bs + ((size_t)pos * kD + lane * 4) * 2) =
-        ldg8(p.k_new + src + lane * 4);
-  } else {
-    *reinterpret_cast<uint2*>(Lb + hd.vb + b * hd.kb_bs + ((size_t)pos * kD + lane * 4) * 2) =
-        ldg8(p.v_new + src + lane * 4);
-  }
+  const bool is_k = threadIdx.x < 32;
+  char* dst = Lb + (is_k ? hd.kb : hd.vb) + b * hd.kb_bs + ((size_t)pos * kD + lane * 4) * 2;
+  grid_dependency_wait();
+  *reinterpret_cast<uint2*>(dst) = ldg8((is_k ? p.k_new : p.v_new) + src + lane * 4);
+}
+
+// Zeroes n 16-byte words between two decode launches of the same chain.
+__global__ void __launch_bounds__(256) clear_kernel(uint4* words, int n) {
+  grid_launch_dependents();
+  grid_dependency_wait();
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) words[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 }  // namespace
@@ -1723,10 +1733,30 @@ cudaError_t launch_dequantize(const DequantParams& p, int sm_count, cudaStream_t
   return launch_dequantize_bits<4>(p, grid, s);
 }
 
+// A launch that may be scheduled while the kernel before it still runs.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 cudaError_t launch_append(const AppendParams& p, cudaStream_t s) {
-  dim3 grid(p.n_layers, p.d.B * p.d.H, 1);
-  append_kernel<<<grid, 64, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_dependent(append_kernel, dim3(p.n_layers, p.d.B * p.d.H, 1), 64, s, p);
+}
+
+cudaError_t launch_clear(void* words, size_t bytes, cudaStream_t s) {
+  const int n = (int)(bytes / 16);
+  return launch_dependent(clear_kernel, dim3(std::max(1, std::min(64, (n + 255) / 256)), 1, 1), 256, s,
+                          static_cast<uint4*>(words), n);
 }
 
 }  // namespace hg

@@ -191,3 +191,26 @@ def test_two_bit_codes_by_comparison(base, meta_bits):
     hg.hg_quantize_kv(runner.cache, 0, [k], [v])
     torch.cuda.synchronize()
     check_arena_layer(runner, 0, bits16(k), bits16(v), oracle_layer(runner, 0, bits16(k), bits16(v)))
+
+
+@pytest.mark.parametrize("base,group", [(wl.BASE_MINMAX, 7), (wl.BASE_KIVI, 1), (wl.BASE_AKVQ, 12)])
+def test_append_and_allocation_free_attention_back_to_back(base, group):
+    """Tokens appended and attended layer by layer with nothing waiting in between (append, counter clear and
+    decode overlap as programmatic dependent launches), against the oracle at the last token."""
+    w = wl.custom("chain", 3, 2, 4 * group, 4, 20, 700, 40, base, 2, 0, decode_steps=8, seed=13,
+                  protected=[(0, 1), (2, 3)])
+    runner = CacheRunner(w)
+    kept = runner.quantize_all(keep=True)
+    news = [wl.step_new_kv(w, s, "cuda") for s in range(8)]
+    qs = [wl.step_query(w, s, "cuda") for s in range(8)]
+    outs = [torch.empty_like(q) for q in qs]
+    torch.cuda.synchronize()
+    for (k_new, v_new), q, out in zip(news, qs, outs):
+        for layer in range(3):
+            hg.hg_append_kv(runner.cache, layer, 1, k_new[layer], v_new[layer])
+            hg.hg_decode_attention_noalloc(runner.cache, layer, 1, q[layer], out[layer], SIGMA)
+    torch.cuda.synchronize()
+    for step in (0, 7):
+        for layer in range(3):
+            ref = _row_reference(runner, layer, 1, *kept[layer], qs[step], news[:step + 1])
+            assert_close(bits16(outs[step][layer, 1:2]), ref, "step %d layer %d" % (step, layer))
