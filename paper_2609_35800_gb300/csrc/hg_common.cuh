@@ -94,8 +94,8 @@ __device__ __forceinline__ float2 half2_bits_to_float2(uint32_t w) {
   return __half22float2(h);
 }
 __device__ __forceinline__ float2 load_meta(const char* base, size_t i, bool m16) {
-  if (m16) return half2_bits_to_float2(__ldg(reinterpret_cast<const uint32_t*>(base) + i));
-  return __ldg(reinterpret_cast<const float2*>(base) + i);
+  if (m16) return half2_bits_to_float2(reinterpret_cast<const uint32_t*>(base)[i]);
+  return reinterpret_cast<const float2*>(base)[i];
 }
 
 // code = clamp(rint_even(fl32(d / scale)), 0, levels) computed without a
@@ -125,7 +125,10 @@ __device__ __forceinline__ float dequant1(uint32_t code, float scale, float zero
   return __fadd_rn(__fmul_rn((float)code, scale), zero);
 }
 
-__device__ __forceinline__ uint4 ldg16(const void* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
-__device__ __forceinline__ uint2 ldg8(const void* p) { return __ldg(reinterpret_cast<const uint2*>(p)); }
+// Vector loads of global memory.  Ordinary ones: the kernels start before the
+// ones they follow have finished (programmatic dependent launch), so what they
+// read is not constant over their lifetime, as the read-only path asks.
+__device__ __forceinline__ uint4 ldg16(const void* p) { return *reinterpret_cast<const uint4*>(p); }
+__device__ __forceinline__ uint2 ldg8(const void* p) { return *reinterpret_cast<const uint2*>(p); }
 
 }  // namespace hg

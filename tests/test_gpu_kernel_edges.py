@@ -214,3 +214,43 @@ def test_append_and_allocation_free_attention_back_to_back(base, group):
         for layer in range(3):
             ref = _row_reference(runner, layer, 1, *kept[layer], qs[step], news[:step + 1])
             assert_close(bits16(outs[step][layer, 1:2]), ref, "step %d layer %d" % (step, layer))
+
+
+@pytest.mark.parametrize("base,salient", [(wl.BASE_MINMAX, 0), (wl.BASE_KIVI, 0), (wl.BASE_AKVQ, 20)])
+def test_overlapping_launches_change_nothing(base, salient):
+    """Prefills over the same arena, reconstructions, appends at a position used before and decode calls with
+    nothing waiting in between (they overlap as programmatic dependent launches) give what the same calls give
+    with a wait after each."""
+    w = wl.custom("overlap", 2, 3, 8, 4, 10, 900, 30, base, 2, 1, decode_steps=2, seed=14, protected=[(0, 1), (1, 2)],
+                  salient_permille=salient)
+    prefills = [[wl.layer_kv(dataclasses.replace(w, seed=14 + i), l, "cuda") for l in range(2)] for i in range(3)]
+    news = [wl.step_new_kv(dataclasses.replace(w, seed=20 + i), 0, "cuda") for i in range(3)]
+    q = wl.step_query(w, 0, "cuda")
+
+    def calls(wait):
+        runner = CacheRunner(w)
+        got = []
+        for kv, (k_new, v_new) in zip(prefills, news):
+            for l in range(2):
+                hg.hg_quantize_kv(runner.cache, l, [kv[l][0]], [kv[l][1]])
+                wait()
+            for fused in (False, True):
+                hg.hg_cache_reset_appended(runner.cache)
+                out = torch.empty_like(q)
+                if fused:
+                    hg.hg_decode_step(runner.cache, 0, 2, q, v_new, k_new, out, SIGMA, runner.ws, runner.ws_bytes)
+                else:
+                    hg.hg_append_kv(runner.cache, 0, 2, k_new, v_new)
+                    wait()
+                    hg.hg_decode_attention_noalloc(runner.cache, 0, 2, q, out, SIGMA)
+                wait()
+                k_out = torch.empty(2, w.batch, w.kv_heads, w.seq_len + 1, 128, dtype=torch.bfloat16, device="cuda")
+                v_out = torch.empty_like(k_out)
+                hg.hg_dequantize_kv(runner.cache, 0, 2, k_out, v_out, False)
+                wait()
+                got += [out, k_out, v_out]
+        torch.cuda.synchronize()
+        return got
+
+    for i, (a, b) in enumerate(zip(calls(lambda: None), calls(torch.cuda.synchronize))):
+        assert torch.equal(a.view(torch.int16), b.view(torch.int16)), i
