@@ -126,6 +126,32 @@ __device__ __forceinline__ bool chunk_T(const uint64_t (&x2)[4], uint64_t mn2, u
   return __vcmpleu2(low, 0x00070007u) == 0u;
 }
 
+// 4-bit codes of a chunk's four channel pairs, packed in channel order, on the
+// fp32 pipe: t = RN(d r + 2^23) holds the rounded quotient f in its low bits, and
+// four of them become a 16-bit word by one packed FMA (f_i + 256 f_{i+2}) and one
+// integer multiply-add.  Returns true when no quotient is near a tie: e = d r - f
+// is within 2e-6 of the exact quotient's distance from f (1 / scale and the
+// reference division round by 2^-24 each, quotients below 16), so below 0.499995
+// the code is f.  (chunk_T and chunk_bits_T take four integer operations per
+// element, and the integer pipe bound these rows: InternVL2.5-8B-shaped prefill with
+// salient tokens, 4 layers one by one, 766 -> 729 us.)
+__device__ __forceinline__ bool chunk_codes4(const uint64_t (&x2)[4], uint64_t mn2, uint64_t r2, uint32_t& lo) {
+  const uint64_t m2 = f32x2(0x4B000000u, 0x4B000000u), c256 = f32x2(0xC3800000u, 0xC3800000u);  // 2^23, -256
+  uint64_t t[4], g[4];
+  float top = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint64_t d = f32x2_sub(x2[i], mn2);
+    t[i] = f32x2_fma(d, r2, m2);
+    g[i] = f32x2_sub(m2, t[i]);  // -f
+    const uint64_t e = f32x2_fma(d, r2, g[i]);
+    top = fmaxf(fmaxf(fabsf(__uint_as_float((uint32_t)e)), fabsf(__uint_as_float((uint32_t)(e >> 32)))), top);
+  }
+  const uint64_t u = f32x2_fma(g[1], c256, t[0]), v = f32x2_fma(g[3], c256, t[2]);
+  lo = prmt((uint32_t)u + 16u * (uint32_t)(u >> 32), (uint32_t)v + 16u * (uint32_t)(v >> 32), 0x5410);
+  return top < 0.499995f;
+}
+
 // Code e (0..31, token order) of one KIVI-style key group row into its packed
 // words: 2 / 4 bits at word e / (32 / bits), bit bits * (e mod 32 / bits); 3
 // bits: bits 0-1 at word e / 16, bit 2 e mod 16, and bit 2 into plane word 2 at
@@ -140,6 +166,63 @@ __device__ __forceinline__ void add_key_code(uint32_t (&wd)[BITS], int e, uint32
     constexpr int per = 32 / (BITS == 3 ? 2 : BITS);
     wd[e / per] |= c << (BITS * (e % per));
   }
+}
+
+// Min and max of BF16 values held as 16-bit words, by integer maxima that take
+// two new words per instruction: of values of both signs the largest is the
+// largest signed word, the smallest the largest unsigned one.  (Groups of one
+// sign, or with a NaN, which is the largest word of either kind, do not pass
+// the test of mixed_signs or of threshold_scale.)
+struct PairMinMax {
+  uint32_t s, u;
+};
+__device__ __forceinline__ void minmax2(PairMinMax& m, uint32_t a, uint32_t b) {
+  m.s = __vimax3_s16x2(m.s, a, b);
+  m.u = __vimax3_u16x2(m.u, a, b);
+}
+// Both maxima over chunks [k0, k0 + nk) of a row, over both halves (low half).
+__device__ __forceinline__ PairMinMax chunk_maxima(const uint4* r4, int k0, int nk) {
+  const uint4 f = r4[k0];
+  PairMinMax m = {f.x, f.x};
+#pragma unroll 4
+  for (int k = k0; k < k0 + nk; ++k) {
+    const uint4 v = r4[k];
+    minmax2(m, v.x, v.y);
+    minmax2(m, v.z, v.w);
+  }
+  return {__vmaxs2(m.s, __byte_perm(m.s, 0u, 0x1032)), __vmaxu2(m.u, __byte_perm(m.u, 0u, 0x1032))};
+}
+
+// Min and max (signed zeros folded to +0) of chunks [k0, k0 + nk) of a row.
+template <bool MAXIMA>
+__device__ __forceinline__ void row_minmax(const uint4* r4, int k0, int nk, float& mn, float& mx) {
+  if (MAXIMA && nk > 4) {  // (no gain over a 32-channel group)
+    const PairMinMax m = chunk_maxima(r4, k0, nk);
+    // values of both signs, all finite; else value by value
+    if (((m.u & ~m.s) & 0x8000u) && (m.s & 0x7f80u) != 0x7f80u && (m.u & 0x7f80u) != 0x7f80u) {
+      mn = __fadd_rn(__uint_as_float(m.u << 16), 0.0f);
+      mx = __fadd_rn(__uint_as_float(m.s << 16), 0.0f);
+      return;
+    }
+  }
+  __nv_bfloat162 mn2, mx2;
+  {
+    const uint4 v = r4[k0];
+    mn2 = mx2 = *reinterpret_cast<const __nv_bfloat162*>(&v.x);
+  }
+#pragma unroll 4
+  for (int k = k0; k < k0 + nk; ++k) {
+    const uint4 v = r4[k];
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&w[i]);
+      mn2 = __hmin2(mn2, h);
+      mx2 = __hmax2(mx2, h);
+    }
+  }
+  mn = __fadd_rn(fminf(__low2float(mn2), __high2float(mn2)), 0.0f);  // -0 -> +0
+  mx = __fadd_rn(fmaxf(__low2float(mx2), __high2float(mx2)), 0.0f);
 }
 
 // ---------------------------------------------------------------------------
@@ -165,18 +248,6 @@ __device__ __forceinline__ void add_key_code(uint32_t (&wd)[BITS], int e, uint32
 // candidates tried per threshold it measured no better than the rule of the
 // other widths.
 // ---------------------------------------------------------------------------
-// Min and max of BF16 values held as 16-bit words, by integer maxima that take
-// two new words per instruction: of values of both signs the largest is the
-// largest signed word, the smallest the largest unsigned one.  (Groups of one
-// sign, or with a NaN, which is the largest word of either kind, do not pass
-// the test of mixed_signs or of threshold_scale.)
-struct PairMinMax {
-  uint32_t s, u;
-};
-__device__ __forceinline__ void minmax2(PairMinMax& m, uint32_t a, uint32_t b) {
-  m.s = __vimax3_s16x2(m.s, a, b);
-  m.u = __vimax3_u16x2(m.u, a, b);
-}
 // Steps the comparisons serve: scale 2^-25 stays normal, 1 / scale finite.
 __device__ __forceinline__ bool threshold_scale(float scale) {
   return scale >= 7.8886090522101181e-31f && scale <= 8.5070591730234616e37f;  // 2^-100, 2^126
@@ -472,26 +543,8 @@ __device__ __forceinline__ void patch_chunk(int k, const uint32_t (&c)[8], uint3
 template <int BITS, bool M16>
 __device__ __forceinline__ void quantize_row_group_any(const uint4* r4, int k0, int nk, uint32_t* codes, char* meta,
                                                    size_t mi) {
-  __nv_bfloat162 mn2, mx2;
-  {
-    const uint4 v = r4[k0];
-    mn2 = mx2 = *reinterpret_cast<const __nv_bfloat162*>(&v.x);
-  }
-#pragma unroll 4
-  for (int k = k0; k < k0 + nk; ++k) {
-    const uint4 v = r4[k];
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&w[i]);
-      mn2 = __hmin2(mn2, h);
-      mx2 = __hmax2(mx2, h);
-    }
-  }
-  float mn = fminf(__low2float(mn2), __high2float(mn2));
-  float mx = fmaxf(__low2float(mx2), __high2float(mx2));
-  mn = __fadd_rn(mn, 0.0f);  // -0 -> +0
-  mx = __fadd_rn(mx, 0.0f);
+  float mn, mx;
+  row_minmax<BITS != 2>(r4, k0, nk, mn, mx);  // (2 bits: the groups that bf16_thresholds left)
   const float levels = (float)((1u << BITS) - 1u);
   float scale = __fdiv_rn(__fsub_rn(mx, mn), levels);
   const float mn_x = mn;  // the group's own minimum
@@ -528,9 +581,13 @@ __device__ __forceinline__ void quantize_row_group_any(const uint4* r4, int k0, 
         uint64_t x2[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) x2[i] = f32x2(w[i] << 16, w[i] & 0xffff0000u);  // channels 2i, 2i + 1
-        uint32_t a[8];
-        if (!chunk_T(x2, mnp, r2, c2, a)) ties |= 1u << (k - k0);  // about one chunk in 100
-        chunk_bits_T<BITS>(a, lo[kk], hb[kk]);
+        if constexpr (BITS == 4) {
+          if (!chunk_codes4(x2, mnp, r2, lo[kk])) ties |= 1u << (k - k0);
+        } else {
+          uint32_t a[8];
+          if (!chunk_T(x2, mnp, r2, c2, a)) ties |= 1u << (k - k0);  // about one chunk in 100
+          chunk_bits_T<BITS>(a, lo[kk], hb[kk]);
+        }
       } else {
         uint32_t c8[8];
         if (scale == 0.0f) {  // constant group (or a step below binary16 range): every code 0
@@ -775,9 +832,10 @@ __device__ __forceinline__ void quantize_row_rotated(const char* row_s, int hh, 
     for (int k = 0; k < NK; ++k) {
       const uint64_t x2[4] = {xp[4 * k], xp[4 * k + 1], xp[4 * k + 2], xp[4 * k + 3]};
       uint32_t a[8];
-      if (chunk_T(x2, mn2, r2, c2, a)) {
-        chunk_bits_T<BITS>(a, lo[k], hb[k]);
+      if (BITS == 4 ? chunk_codes4(x2, mn2, r2, lo[k]) : chunk_T(x2, mn2, r2, c2, a)) {
+        if (BITS != 4) chunk_bits_T<BITS>(a, lo[k], hb[k]);
       } else {
+        if (BITS == 4) chunk_T(x2, mn2, r2, c2, a);
         uint32_t c8[8];
         chunk_near_tie<BITS>(a, [&](int i) { return (i & 1) ? pair_hi(x2[i >> 1]) : pair_lo(x2[i >> 1]); }, mn,
                              scale, c8);
