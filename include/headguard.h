@@ -305,8 +305,9 @@ hg_status hg_decode_step(hg_cache *cache, int32_t layer_begin, int32_t layer_cou
  * synchronisation.  (This entry point has no counterpart in the paper.)
  *   Scratch   the split-K workspace is one static device array of 32 MiB
  *             inside this library; every GPU that loads the library holds it
- *             until the process exits.  A launch whose workspace
- *             (hg_decode_workspace_size) exceeds 32 MiB is rejected with
+ *             until the process exits.  A launch that cannot run in 32 MiB
+ *             (hg_decode_workspace_size may ask for more than the least a
+ *             launch takes, for a finer split) is rejected with
  *             HG_ERR_WORKSPACE_TOO_SMALL before anything is enqueued.
  *   Set-up    the first call on a device (with that device current) looks up
  *             the array's device address with cudaGetSymbolAddress; make that

@@ -318,7 +318,8 @@ DecodePlan plan_decode(const hg_cache* c, int begin, int count, DecodePlan* leas
   // pieces of half the mean run as two to three waves instead, costliest
   // first: one layer of 32 rows, 8 KV heads and 8,576 tokens 150 -> 90 us (96
   // and 91 us at 2/3 and 1/3 of the mean); 3,520 tokens of 4-bit rotated keys
-  // 84 -> 53 us (53, 58).  Chunks under 256 KB keep one wave: a CTA's start
+  // 84 -> 53 us (53, 58), all measured with CTA-wide tiles (the warps' own
+  // pipelines since take 70 and 44 us).  Chunks under 256 KB keep one wave: a CTA's start
   // and merge (about 8 us) outweigh the balance there (28 layers of 4 heads:
   // 15.3 us a step in one wave, 18.1 with pieces of 2/3).
   double worst = 0;

@@ -28,7 +28,7 @@ struct QuantizeParams {
   Dims d;
   char* arena;
   int n_layers;
-  int tile_origin;  // s mod 32: KIVI-style tile i covers [tile_origin - 32 + 64 i, +64) clipped to [0, T)
+  int tile_origin;  // s mod 32: KIVI-style tile i covers [tile_origin - 32 + 32 i, +32) clipped to [0, T)
   LayerTable lt;
   GeomTable gt;
   const uint16_t* k[kMaxLayersPerLaunch];

@@ -40,7 +40,8 @@ __device__ __forceinline__ void bf16x4_to_f32(uint2 w, float (&x)[4]) {
 // head), staged in shared memory with coalesced loads (272-byte row pitch, so
 // that a lane's 16-byte reads of its own row are conflict free); lane i owns
 // row i.  A coded vector is quantized by its lane alone -- min / max over
-// bf16x2 pairs (exact), then per element
+// bf16x2 pairs (exact), then at 2 bits three comparisons with the BF16 values
+// where the code changes (bf16_thresholds), else per element
 //   T = RN(d * r + 192), d = fl(x - min), r = RN(1 / scale):
 // T lies in [128, 256), so its low 16 mantissa bits hold d * r to 2^-16 and
 // bits 16.. hold floor(d * r + 0.5) once 0x8000 is added.  Within 2^-16 of
