@@ -709,8 +709,8 @@ __device__ __forceinline__ void quantize_row_kivi_v(const char* row_s, uint32_t*
 // own words of the packed row (lane 0 stores the metadata).  Half the pairs
 // per thread: twice the rows resident.  Bound by instruction issue: stage 64 as
 // one FMA by +-1, not a sum, a difference and a selection, InternVL2.5-8B-shaped
-// prefill with salient tokens, 4 layers one by one, 729 -> 692 us.  (At 96
-// registers, 20 warps per SM instead of 16, it spills: 697 us.)
+// prefill with salient tokens, 4 layers one by one, 729 -> 692 us (94 registers
+// instead of 102: 20 warps per SM, not 16).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float pair_lo(uint64_t x) { return __uint_as_float((uint32_t)x); }
 __device__ __forceinline__ float pair_hi(uint64_t x) { return __uint_as_float((uint32_t)(x >> 32)); }
