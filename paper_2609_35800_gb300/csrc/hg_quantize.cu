@@ -336,6 +336,7 @@ __device__ __forceinline__ void quantize_key_pair_any(const char* col, uint32_t*
   uint32_t wd0[BITS], wd1[BITS];  // the two channels' packed words, filled code by code
 #pragma unroll
   for (int i = 0; i < BITS; ++i) wd0[i] = wd1[i] = 0u;
+  uint32_t tie0 = 0u, tie1 = 0u;  // tokens whose code is near a tie
   if (fast) {
     const float r0 = __frcp_rn(sc[0]), r1 = __frcp_rn(sc[1]);
     const uint64_t mn2p = f32x2(__float_as_uint(mn[0]), __float_as_uint(mn[1]));
@@ -346,11 +347,10 @@ __device__ __forceinline__ void quantize_key_pair_any(const char* col, uint32_t*
     for (int e = 0; e < kKiviGroup; ++e) {
       const uint64_t t2 = f32x2_fma(f32x2_sub(f32x2(w[e] << 16, w[e] & 0xffff0000u), mn2p), r2, c2);
       const uint32_t a0 = (uint32_t)t2, a1 = (uint32_t)(t2 >> 32);
-      uint32_t k0 = (a0 >> 16) & L, k1 = (a1 >> 16) & L;
-      if (!(a0 & 0xfff8u)) k0 = exact_code(__fsub_rn(__uint_as_float(w[e] << 16), mn[0]), sc[0], levels);
-      if (!(a1 & 0xfff8u)) k1 = exact_code(__fsub_rn(__uint_as_float(w[e] & 0xffff0000u), mn[1]), sc[1], levels);
-      add_key_code<BITS>(wd0, e, k0);
-      add_key_code<BITS>(wd1, e, k1);
+      add_key_code<BITS>(wd0, e, (a0 >> 16) & L);
+      add_key_code<BITS>(wd1, e, (a1 >> 16) & L);
+      if (!(a0 & 0xfff8u)) tie0 |= 1u << e;
+      if (!(a1 & 0xfff8u)) tie1 |= 1u << e;
     }
   } else {
 #pragma unroll
@@ -380,6 +380,29 @@ __device__ __forceinline__ void quantize_key_pair_any(const char* col, uint32_t*
     } else {
       d4[0] = make_uint4(wd0[0], wd0[1 % BITS], wd0[2 % BITS], wd0[3 % BITS]);
       d4[1] = make_uint4(wd1[0], wd1[1 % BITS], wd1[2 % BITS], wd1[3 % BITS]);
+    }
+  }
+  // near ties by the exact rule, each code written over its stored bits (the
+  // positions of add_key_code); side by side in the warp's threads.  (As a branch
+  // at each element of the loop above: 14 layers of 14 rows, 16 heads and 856
+  // tokens at 4 bits one by one 495 -> 471 us, a 3-bit layer of 6 rows 7.5 -> 6.3
+  // us; at 2 bits the few groups that come here hold up their warps: LLaVA-NeXT-
+  // 7B-shaped, 4 layers one by one, 761 -> 730 us.)
+  while (tie0 | tie1) {
+    const bool j = tie0 == 0u;
+    const int e = __ffs(j ? tie1 : tie0) - 1;
+    if (j) tie1 &= tie1 - 1;
+    else tie0 &= tie0 - 1;
+    const float x = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(col + (size_t)e * kQPitch)[j] << 16);
+    const uint32_t c = exact_code(__fsub_rn(x, j ? mn[1] : mn[0]), j ? sc[1] : sc[0], levels);
+    uint32_t* dst = j ? dst1 : dst0;
+    constexpr int LB = BITS == 4 ? 4 : 2, per = 32 / LB;
+    constexpr uint32_t M = (1u << LB) - 1u;
+    const int sh = LB * (e % per);
+    dst[e / per] = (dst[e / per] & ~(M << sh)) | ((c & M) << sh);
+    if (BITS == 3) {
+      const int b = (e & 7) | (((e >> 4) & 1) << 3) | (((e >> 3) & 1) << 4);
+      dst[2] = (dst[2] & ~(1u << b)) | ((c >> 2) << b);
     }
   }
 }
@@ -502,28 +525,46 @@ __device__ __forceinline__ void chunk_near_tie(const uint32_t (&a)[8], X x, floa
     c8[i] = (a[i] & 0xfff8u) ? ((a[i] >> 16) & L) : exact_code(__fsub_rn(x(i), mn), scale, (float)L);
 }
 
-// Chunk k's codes written over its bits of a packed row that this thread has
-// already stored: word k (4 bits), or half k % 2 of word k / 2 (2 and 3 bits)
-// and, at 3 bits, byte ((k >> 1) & 1) | ((k & 1) << 1) of plane word 8 + k / 4
-// (the layout of store_group).  The other chunks' bits are read back.
+// Elements near a tie of chunk k of a packed row that this thread has already
+// stored, coded again by the exact rule, each written over its bits: word k (4
+// bits), or half k % 2 of word k / 2 (2 and 3 bits) and, at 3 bits, byte
+// ((k >> 1) & 1) | ((k & 1) << 1) of plane word 8 + k / 4 (the layout of
+// store_group).  The other elements' codes are read back and kept: they were
+// decided by the fast rule.  The loop runs over a thread's own elements near a
+// tie (mostly one), so the threads of a warp divide side by side; with the eight
+// elements in turn a warp went through nearly all eight for its threads'
+// different ones.  One layer of 862 tokens at 4 bits 5.2 -> 4.4 us; 17 layers of
+// 1,560 tokens one by one 100 -> 85 us; 3 bits, 2 layers of 6 rows and 7,415
+// tokens 55 -> 50 us.
 template <int BITS>
-__device__ __forceinline__ void patch_chunk(int k, const uint32_t (&c)[8], uint32_t* codes) {
-  uint32_t lo = 0u, hb = 0u;
+__device__ __forceinline__ void recode_near_ties(const uint4* r4, int k, uint64_t mn2, uint64_t r2, uint64_t c2, float mn,
+                                                 float scale, uint32_t* codes) {
+  const uint4 v = r4[k];
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  uint64_t x2[4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    lo |= (BITS == 4) ? (c[i] << (4 * i)) : ((c[i] & 3u) << (2 * i));
-    if (BITS == 3) hb |= ((c[i] >> 2) & 1u) << i;
+  for (int i = 0; i < 4; ++i) x2[i] = f32x2(w[i] << 16, w[i] & 0xffff0000u);
+  uint32_t a[8], el = 0u;  // bit i: T' low bits of element i in [0, 7]
+  chunk_T(x2, mn2, r2, c2, a);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (!(a[i] & 0xfff8u)) el |= 1u << i;
+  uint32_t* lw = codes + (BITS == 4 ? k : k >> 1);
+  uint32_t* hw = codes + 8 + (k >> 2);
+  const int ls = BITS == 4 ? 0 : 16 * (k & 1), hs = 8 * (((k >> 1) & 1) | ((k & 1) << 1));
+  uint32_t lo = *lw, hb = BITS == 3 ? *hw : 0u;
+  while (el) {
+    const int i = __ffs(el) - 1;
+    el &= el - 1;
+    const float x = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(r4 + k)[i] << 16);
+    const uint32_t c = exact_code(__fsub_rn(x, mn), scale, (float)((1u << BITS) - 1u));
+    constexpr int LB = BITS == 4 ? 4 : 2;
+    constexpr uint32_t M = (1u << LB) - 1u;
+    lo = (lo & ~(M << (ls + LB * i))) | ((c & M) << (ls + LB * i));
+    if (BITS == 3) hb = (hb & ~(1u << (hs + i))) | ((c >> 2) << (hs + i));
   }
-  if (BITS == 4) {
-    codes[k] = lo;
-    return;
-  }
-  const int sh = 16 * (k & 1);
-  codes[k >> 1] = (codes[k >> 1] & ~(0xffffu << sh)) | (lo << sh);
-  if (BITS == 3) {
-    const int pb = 8 * (((k >> 1) & 1) | ((k & 1) << 1));
-    codes[8 + (k >> 2)] = (codes[8 + (k >> 2)] & ~(0xffu << pb)) | (hb << pb);
-  }
+  *lw = lo;
+  if (BITS == 3) *hw = hb;
 }
 
 // One group of a BF16 row: chunks [k0, k0 + nk) (8 channels each) with their
@@ -535,10 +576,9 @@ __device__ __forceinline__ void patch_chunk(int k, const uint32_t (&c)[8], uint3
 // loop stays rolled so that the code stays small in the instruction cache
 // (eight chunks per step measured slower on the per-token rows).
 // A chunk with an element near a tie (fast rule) is emitted with its fast
-// codes and flagged; after the loop each thread codes its flagged chunks again,
-// the flagged elements by the exact rule, and writes each chunk's bits over
-// the stored ones (patch_chunk).  The threads of a warp do this side by side,
-// so a warp pays for the largest number of flagged chunks of one thread
+// codes and flagged; after the loop each thread codes the elements of its flagged
+// chunks that are near a tie again (recode_near_ties).  The threads of a warp do
+// this side by side, so a warp pays for the largest number of one thread
 // instead of running every thread's near ties one after another inside the
 // loop.
 template <int BITS, bool M16>
@@ -605,16 +645,7 @@ __device__ __forceinline__ void quantize_row_group_any(const uint4* r4, int k0, 
   while (ties) {
     const int k = k0 + (__ffs(ties) - 1);
     ties &= ties - 1;
-    const uint4 v = r4[k];
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    uint64_t x2[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) x2[i] = f32x2(w[i] << 16, w[i] & 0xffff0000u);
-    uint32_t a[8], c8[8];
-    chunk_T(x2, mnp, r2, c2, a);
-    chunk_near_tie<BITS>(a, [&](int i) { return __uint_as_float((i & 1) ? (w[i >> 1] & 0xffff0000u) : (w[i >> 1] << 16)); },
-                         mn, scale, c8);
-    patch_chunk<BITS>(k, c8, codes);
+    recode_near_ties<BITS>(r4, k, mnp, r2, c2, mn, scale, codes);
   }
 }
 

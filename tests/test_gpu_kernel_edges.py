@@ -193,6 +193,28 @@ def test_two_bit_codes_by_comparison(base, meta_bits):
     check_arena_layer(runner, 0, bits16(k), bits16(v), oracle_layer(runner, 0, bits16(k), bits16(v)))
 
 
+@pytest.mark.parametrize("meta_bits", [64, 32])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("base", [wl.BASE_MINMAX, wl.BASE_KIVI, wl.BASE_AKVQ])
+def test_every_code_on_a_tie(base, bits, meta_bits):
+    """Groups of half-integers from 0 to the top level (step 1): every element but the extremes is exactly on a
+    tie, at every position of a chunk and of a key group, and each is coded again alone.  Bit for bit."""
+    w = wl.custom("ties", 1, 2, 4, 2, 3, 96, 5, base, bits, 0, seed=14, protected=[], residual=0, meta_bits=meta_bits)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    top = (1 << bits) - 1
+    x = torch.randint(0, top, (2, 2, 2, w.seq_len, 128), generator=g, device="cuda") + 0.5
+    tok, ch = torch.arange(w.seq_len, device="cuda")[:, None] - 3, torch.arange(128, device="cuda")
+    x = torch.where((ch + tok) % 32 == 0, 0.0, x)        # one of each per 32 channels and per 32 tokens
+    x = torch.where((ch + tok) % 32 == 17, float(top), x)
+    x[..., 40:48] = torch.where(x[..., 40:48] % 1 == 0, x[..., 40:48], x[..., 40:48] + 0.125 * (tok % 2 == 0))
+    x = x.clamp(max=float(top)).bfloat16()
+    k, v = x[0].contiguous(), x[1].contiguous()
+    runner = CacheRunner(w)
+    hg.hg_quantize_kv(runner.cache, 0, [k], [v])
+    torch.cuda.synchronize()
+    check_arena_layer(runner, 0, bits16(k), bits16(v), oracle_layer(runner, 0, bits16(k), bits16(v)))
+
+
 @pytest.mark.parametrize("base,group", [(wl.BASE_MINMAX, 7), (wl.BASE_KIVI, 1), (wl.BASE_AKVQ, 12)])
 def test_append_and_allocation_free_attention_back_to_back(base, group):
     """Tokens appended and attended layer by layer with nothing waiting in between (append, counter clear and
