@@ -1164,7 +1164,7 @@ __global__ void __launch_bounds__(32) quantize_tiles_kernel(const __grid_constan
 //
 // One CTA per head for both read the keys with 8 KB in flight: 88 us for a
 // layer of 32 rows, 8 KV heads and 3,328 image tokens (191 MB of keys read, 28 us
-// at the measured copy rate); now 33 us and 12 us.
+// at the measured copy rate); now 33 us and 8 us.
 // ---------------------------------------------------------------------------
 constexpr int kNormThreads = 256, kNormRows = 8, kNormTokens = kNormThreads / 32 * kNormRows;
 constexpr int kSalThreads = 512;
@@ -1263,35 +1263,50 @@ __global__ void __launch_bounds__(kSalThreads) salient_select_kernel(const __gri
     const float* src = salient_scores(d, hd, p.arena + p.lt.base[li], b);
     for (int i = tid; i < nq; i += kSalThreads) score[i] = src[i];
   }
+  __shared__ uint32_t hist[256];
+  __shared__ uint32_t s_prefix, s_need, s_eq, s_diff;
+  if (tid == 0) {
+    s_eq = (uint32_t)nq;
+    s_diff = 0u;
+  }
   __syncthreads();
 
   // The ns largest scores, ties to the lower index -- the set that ns rounds
   // of arg-max (taken tokens dropping out) would pick -- by a radix select on
-  // the scores' bit patterns (non-negative floats order as their bits): four
-  // 8-bit digits from the top, each pass a histogram of the candidates that
-  // match the digits chosen so far and the digit where the count of larger
-  // keys reaches ns.  Then every key above the final threshold T is taken,
-  // and of the keys equal to T the first `need` by index.
+  // the scores' bit patterns (non-negative floats order as their bits): 8-bit
+  // digits from the highest bit in which two keys differ, each pass a histogram
+  // of the candidates that match the digits chosen so far and the digit where
+  // the count of larger keys reaches ns.  When all candidates with that digit are
+  // taken, no lower digit matters.  Then every key above the final threshold T is
+  // taken, and of the keys equal to T the first `need` by index.  A pass is
+  // three barriers, a histogram and a scan, about 2 us: usually two of them, where
+  // four fixed digits spent the first on a byte that two values share.  Spread
+  // digits make plain atomics the better histogram (one per distinct digit of a
+  // warp, found by a match: 2 us more).  A layer of 32 rows, 8 KV heads and 3,328
+  // image tokens 12 -> 8 us; 11 layers of 2 rows, 16 heads and 110 image tokens,
+  // prefill in all 133 -> 119 us; the same with one key far above the others, or
+  // all equal.
   static_assert(kSalThreads >= 256, "a thread per histogram bin");
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t s_prefix, s_need, s_eq;
-  uint32_t prefix = 0u, pmask = 0u, need = (uint32_t)d.ns;
+  uint32_t diff = 0u;
+  const uint32_t key0 = __float_as_uint(score[0]);
+  for (int i = tid; i < nq; i += kSalThreads) diff |= __float_as_uint(score[i]) ^ key0;
+  diff = __reduce_or_sync(kFull, diff);
+  if (lane == 0 && diff) atomicOr(&s_diff, diff);
+  __syncthreads();
+  int left_bits = 32 - __clz(s_diff);  // the low bits not decided yet
+  uint32_t pmask = left_bits == 32 ? 0u : ~0u << left_bits, prefix = key0 & pmask, need = (uint32_t)d.ns;
 #pragma unroll 1
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 24 - 8 * pass;
+  while (left_bits > 0 && s_eq != need) {
+    const int shift = max(left_bits - 8, 0);
+    const uint32_t dmask = (1u << (left_bits - shift)) - 1u;
     if (tid < 256) hist[tid] = 0u;
     __syncthreads();
     for (int i0 = warp * 32; i0 < nq; i0 += kSalThreads) {  // warp-uniform: lane i0 + lane
       const int i = i0 + lane;
       const uint32_t key = i < nq ? __float_as_uint(score[i]) : 0u;
       const bool cand = i < nq && (key & pmask) == prefix;
-      const uint32_t dg = (key >> shift) & 255u;
-      // one atomic per distinct digit of the warp's candidates
-      const uint32_t act = __ballot_sync(kFull, cand);
-      if (cand) {
-        const uint32_t same = __match_any_sync(act, dg);
-        if ((__ffs(same) - 1) == lane) atomicAdd(&hist[dg], (uint32_t)__popc(same));
-      }
+      const uint32_t dg = (key >> shift) & dmask;
+      if (cand) atomicAdd(&hist[dg], 1u);
     }
     __syncthreads();
     if (warp == 0) {
@@ -1327,7 +1342,8 @@ __global__ void __launch_bounds__(kSalThreads) salient_select_kernel(const __gri
     __syncthreads();
     prefix = s_prefix;
     need = s_need;
-    pmask |= 255u << shift;
+    pmask |= dmask << shift;
+    left_bits = shift;
   }
   // T = prefix: `need` of the s_eq keys equal to T are taken, by index
   const uint32_t T = prefix;

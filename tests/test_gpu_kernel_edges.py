@@ -160,6 +160,34 @@ def test_salient_selection_in_one_or_two_launches(image):
     _run_and_check(w)
 
 
+@pytest.mark.parametrize("image", [97, 700])
+@pytest.mark.parametrize("kind", ["one far above", "two sizes", "two values", "neighbours", "equal", "zero"])
+def test_salient_selection_of_norms_in_few_digits(kind, image):
+    """Keys whose squared norms differ in few bits, or in high and low ones at once (the selection starts at the
+    highest bit in which two differ and ends at a digit that is taken whole).  Bit for bit."""
+    w = wl.custom("digits", 1, 2, 4, 2, 5, image, 6, wl.BASE_AKVQ, 4, 0, seed=15, protected=[], residual=0,
+                  salient_permille=100)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    k = torch.randn(2, 2, w.seq_len, 128, generator=g, device="cuda")
+    if kind == "one far above":
+        k[:, :, 40] *= 1e8
+    elif kind == "two sizes":
+        k[:, :, ::3] *= 16.0
+    elif kind == "two values":
+        k = torch.where(torch.arange(w.seq_len, device="cuda")[:, None] % 7 == 0, 2.0, 1.0).expand_as(k)
+    elif kind == "neighbours":  # 128 + small steps: only low bits differ
+        k = torch.ones_like(k)
+        k[..., 0] = 1.0 + torch.randint(0, 6, k.shape[:3], generator=g, device="cuda") * 2.0 ** -7
+    else:
+        k = torch.full_like(k, 0.0 if kind == "zero" else -1.5)
+    k = k.bfloat16().contiguous()
+    v = torch.randn(2, 2, w.seq_len, 128, generator=g, device="cuda").bfloat16()
+    runner = CacheRunner(w)
+    hg.hg_quantize_kv(runner.cache, 0, [k], [v])
+    torch.cuda.synchronize()
+    check_arena_layer(runner, 0, bits16(k), bits16(v), oracle_layer(runner, 0, bits16(k), bits16(v)))
+
+
 @pytest.mark.parametrize("meta_bits", [64, 32])
 @pytest.mark.parametrize("base", [wl.BASE_MINMAX, wl.BASE_KIVI, wl.BASE_AKVQ])
 def test_two_bit_codes_by_comparison(base, meta_bits):
