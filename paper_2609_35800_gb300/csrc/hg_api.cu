@@ -307,7 +307,10 @@ DecodePlan plan_decode(const hg_cache* c, int begin, int count, DecodePlan* leas
   limit_splits(d, least);
   const double mean = mean_cost(d, thr, hc, wave);
   if (mean < kLatencyCost) {
-    limit_splits_by_kind(d, &p);
+    // KIVI-style codes of 3 to 8 queries: a chunk of coded tokens is by far the
+    // longest, so the splits go to them (doubled sizes leave the text one or two)
+    if (d.base == kKivi && d.G > 2 && d.G <= 8) limit_splits(d, &p);
+    else limit_splits_by_kind(d, &p);
     return p;
   }
   p = one_wave_plan(d, thr, hc, wave, mean);

@@ -1661,9 +1661,10 @@ __device__ __forceinline__ void locate_item(const DecodeParams& p, int x, int& l
 }
 
 // NT: 8-query column tiles of the MMAs.  QC: queries per KV head where
-// run_item_cols serves the KIVI-style items (1 or 2), else 0.
+// run_item_cols serves the KIVI-style items (1 or 2), else 0; -1: the same with
+// registers for three CTAs per SM instead of four.
 template <int BITS, int NT, int BASE, int MB, int QC>
-__global__ void __launch_bounds__(kThreads, NT == 1 ? 4 : 2)
+__global__ void __launch_bounds__(kThreads, NT == 1 ? (QC < 0 ? 3 : 4) : 2)
 decode_kernel(const __grid_constant__ DecodeParams p) {
   extern __shared__ __align__(1024) char smem_raw[];
   // swizzled TMA boxes need 1024-byte aligned shared addresses
@@ -1871,6 +1872,12 @@ cudaError_t launch_base(const DecodeParams& p, int grid_x, cudaStream_t s) {
       if constexpr (NT == 1) {
         if (p.d.G == 1) return launch_t<BITS, NT, kKivi, MB, 1>(p, grid_x, s);
         if (p.d.G == 2) return launch_t<BITS, NT, kKivi, MB, 2>(p, grid_x, s);
+        // Four CTAs per SM leave the converting path short of registers (50 to 100
+        // bytes of spills).  A launch of one wave or less is better off without
+        // them, if some of its CTAs have to wait (one layer, 8 KV heads: 2 rows of
+        // 2,900 tokens at 4 bits 23 -> 19 us; 4 rows of 8,200 at 2 bits 41 -> 33 us);
+        // more waves want the fourth CTA (10 rows of 3,400 tokens: 45 and 48 us).
+        if (p.total_items <= 4 * p.deal) return launch_t<BITS, NT, kKivi, MB, -1>(p, grid_x, s);
       }
       return launch_t<BITS, NT, kKivi, MB, 0>(p, grid_x, s);
     case kAkvq: return launch_t<BITS, NT, kAkvq, MB, 0>(p, grid_x, s);
