@@ -113,6 +113,16 @@ def test_kivi_few_queries_per_head(group, bits, meta_bits):
         _decode_against_oracle(w, [wl.layer_kv(w, 0, "cuda")], 2)
 
 
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("batch", [2, 24])
+def test_kivi_grouped_queries_in_one_wave_and_more(batch, bits):
+    """Four queries per KV head over KIVI-style codes in launches below and above four CTAs per SM (registers for
+    three and for four CTAs)."""
+    w = wl.custom("wave%d" % batch, 2, batch, 32, 8, 20, 150, 30, wl.BASE_KIVI, bits, 0, decode_steps=1, seed=16,
+                  protected=[(0, 1)])
+    _decode_against_oracle(w, [wl.layer_kv(w, layer, "cuda") for layer in range(2)], 1)
+
+
 @pytest.mark.parametrize("base,bits,group", [(wl.BASE_KIVI, 2, 1), (wl.BASE_KIVI, 3, 2), (wl.BASE_KIVI, 4, 1),
                                              (wl.BASE_MINMAX, 2, 4), (wl.BASE_MINMAX, 4, 12), (wl.BASE_AKVQ, 3, 7)])
 def test_decode_scales_over_many_binades(base, bits, group):
