@@ -974,15 +974,17 @@ __device__ __forceinline__ bool copy_tile_whole(const QuantizeParams& p, int li,
 // The per-token bases, one thread per vector: min-max rows (Sec. 1) and
 // AKVQ-style rows (Sec. 4: keys rotated first; values per token, unrotated).
 // Tiles of 32 tokens from token 0; a CTA (one warp) takes the K rows or the V
-// rows of a tile (PARTS 1: K only, 2: V only, 3: both, as two CTAs).  With
-// salient tokens (AKVQ-style, Sec. 4) a thread finds its token in the head's
-// map: a salient token's K and V rows go to the BF16 region at position
-// s + (its rank), every other image token to coded slot ti - (the salient
-// tokens before it).
-template <int BITS, bool M16, int BASE, int PARTS>
+// rows of a tile.  With salient tokens (AKVQ-style, Sec. 4) a thread finds its
+// token in the head's map: a salient token's K and V rows go to the BF16 region
+// at position s + (its rank), every other image token to coded slot ti - (the
+// salient tokens before it).
+template <int BITS, bool M16, int BASE>
 struct TokenTiles {
-  static constexpr int kNParts = PARTS == 3 ? 2 : 1;
-  static __device__ __forceinline__ int part(int i) { return PARTS == 3 ? i : (PARTS == 1 ? 0 : 1); }
+  static constexpr bool kKeysFirst = BASE == kAkvq;
+  // 96: 21 warps per SM where the rotated rows and the value rows of one kernel came
+  // to 99 (InternVL2.5-8B-shaped prefill with salient tokens, 4 layers one by one, 692 ->
+  // 659 us; at most two registers spilled); 80: what the rows take anyway.
+  static constexpr int kRegisters = BASE == kAkvq ? 96 : 80;
   static __device__ __forceinline__ TileSpan span(const QuantizeParams& p, int tx) {
     TileSpan sp;
     sp.t0 = sp.tlo = tx * kQTok;
@@ -1016,9 +1018,9 @@ struct TokenTiles {
     if (kv == 0) {
       if (coded && hd.cls == kQuantized && !sal) {
         uint32_t* crow = reinterpret_cast<uint32_t*>(Lb + hd.kq + b * hd.kq_bs) + (size_t)ci * W;
-        if (BASE == kAkvq)
+        if constexpr (SPLIT == 2)
           quantize_row_rotated<BITS, M16, SPLIT>(row_s, hh, pmask, crow, Lb + hd.kqm + b * hd.kqm_bs, ci);
-        else if constexpr (SPLIT == 1)
+        else if constexpr (BASE != kAkvq)
           quantize_row_token<BITS, M16>(row_s, crow, Lb + hd.kqm + b * hd.kqm_bs, ci);
         return;
       }
@@ -1037,14 +1039,16 @@ struct TokenTiles {
   static __device__ __forceinline__ void process(const QuantizeParams& p, int li, int b, int kv, const TileSpan& sp,
                                                  const StagedRows& rows, const HeadGeom& hd) {
     if (copy_tile_whole(p, li, b, kv, sp, rows, hd)) return;
-    if (BASE == kAkvq && PARTS == 1) {
-      // rotated key rows: two lanes per row, rows lane / 2 and 16 + lane / 2
-      // (both lanes of a pair take the same path, so the pair's shuffles meet)
-      const int hh = threadIdx.x & 1;
-      const unsigned pmask = 3u << (threadIdx.x & 30);
+    if constexpr (BASE == kAkvq) {
+      if (kv == 0) {
+        // rotated key rows: two lanes per row, rows lane / 2 and 16 + lane / 2
+        // (both lanes of a pair take the same path, so the pair's shuffles meet)
+        const int hh = threadIdx.x & 1;
+        const unsigned pmask = 3u << (threadIdx.x & 30);
 #pragma unroll 1
-      for (int r = threadIdx.x >> 1; r < sp.n; r += 16) row<2>(p, li, b, kv, sp, rows, hd, r, hh, pmask);
-      return;
+        for (int r = threadIdx.x >> 1; r < sp.n; r += 16) row<2>(p, li, b, 0, sp, rows, hd, r, hh, pmask);
+        return;
+      }
     }
     if ((int)threadIdx.x < sp.n) row<1>(p, li, b, kv, sp, rows, hd, threadIdx.x, 0, 0u);
   }
@@ -1061,10 +1065,10 @@ struct TokenTiles {
 // the BF16 residual window and a trailing partial group, protected heads,
 // keys of keys-only heads) is copied.
 // ---------------------------------------------------------------------------
-template <int BITS, bool M16, int PARTS>
+template <int BITS, bool M16>
 struct KiviTiles {
-  static constexpr int kNParts = PARTS == 3 ? 2 : 1;
-  static __device__ __forceinline__ int part(int i) { return PARTS == 3 ? i : (PARTS == 1 ? 0 : 1); }
+  static constexpr bool kKeysFirst = true;
+  static constexpr int kRegisters = 80;  // what the rows take anyway
   // tile x: [origin - 32 + 32 x, + 32) clipped to [0, T), origin = s mod 32
   static __device__ __forceinline__ TileSpan span(const QuantizeParams& p, int tx) {
     TileSpan sp;
@@ -1115,32 +1119,33 @@ struct KiviTiles {
   }
 };
 
-// The quantizer kernel: one CTA of one warp per (tile, part); grid x = tile
-// x part (part fastest), y = batch row x KV head, z = layer.  A warp
-// stages its 32 rows, waits for its own copies and codes them; no CTA-wide
-// barrier, so the warps of an SM (23 resident) run out of step and one
+// The quantizer kernel: one CTA of one warp per (tile, part); grid x = tile,
+// y = batch row x KV head, z = layer, and part: the lowest digit of x (min-max),
+// or (kKeysFirst) the highest of z, all keys of the launch before all values,
+// so that the warps of an SM share one of two unlike code paths at a time.  A
+// warp stages its 32 rows, waits for its own copies and codes them; no CTA-wide
+// barrier, so the warps of an SM (21 to 23 resident) run out of step and one
 // warp's loads overlap another's coding.
-// Programmatic dependent launches: a launch's CTAs may come to the SMs while the
-// kernels before it still run, and wait for them before their first load.
-// FOLLOWS: the launch right after another one of the same call that it does
-// not depend on.  The first lets the next one start only once its own wait is
-// over, so a following launch's CTAs run beside the first one's last ones and
-// wait at their end (the launch after both must find both done).  Per call the
-// gaps between launches were 2 us each and the last wave ran out alone:
-// Qwen2.5-VL-7B-shaped prefill 24.6 -> 22.2 us, LLaVA-NeXT-7B-shaped 4 layers one by
-// one 794 -> 762 us, with salient tokens (four launches a layer)
-// InternVL2.5-8B-shaped 809 -> 767 us.
-template <class TP, bool FOLLOWS>
-__global__ void __launch_bounds__(32) quantize_tiles_kernel(const __grid_constant__ QuantizeParams p) {
+// A programmatic dependent launch: its CTAs may come to the SMs while the
+// kernels before it still run, and wait for them before their first load (no
+// other grid's wait orders this one's reads).  Keys and values are one launch
+// because neither needs the other: LLaVA-NeXT-7B-shaped, 4 layers one by one, 712
+// us, against 740 with the values in a launch that waits for the keys'.
+template <class TP>
+__global__ void __maxnreg__(TP::kRegisters) quantize_tiles_kernel(const __grid_constant__ QuantizeParams p) {
   __shared__ __align__(16) StagedRows rows;
-  const int pi = blockIdx.x % TP::kNParts, tx = blockIdx.x / TP::kNParts;
-  const int li = blockIdx.z, b = blockIdx.y / p.d.H, h = blockIdx.y % p.d.H;
-  const int kv = TP::part(pi);
-  const TileSpan sp = TP::span(p, tx);
-  if (!FOLLOWS) {
-    grid_dependency_wait();
-    grid_launch_dependents();
+  int tx = blockIdx.x, li = blockIdx.z, kv;
+  if (TP::kKeysFirst) {
+    kv = li >= p.n_layers;
+    li -= kv ? p.n_layers : 0;
+  } else {
+    kv = tx & 1;
+    tx >>= 1;
   }
+  const int b = blockIdx.y / p.d.H, h = blockIdx.y % p.d.H;
+  const TileSpan sp = TP::span(p, tx);
+  grid_dependency_wait();
+  grid_launch_dependents();
   if (sp.n <= 0) return;
   stage_rows(p, li, b, h, kv, sp, rows);
   cp_async_commit();
@@ -1148,7 +1153,6 @@ __global__ void __launch_bounds__(32) quantize_tiles_kernel(const __grid_constan
   cp_async_wait<0>();
   __syncwarp();
   TP::process(p, li, b, kv, sp, rows, hd);
-  if (FOLLOWS) grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------
@@ -1805,34 +1809,22 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Launch of the quantizer kernel over every tile of the launch's layers.
-template <class TP, bool FOLLOWS = false>
+// Launch of the quantizer kernel over every tile of the launch's layers, keys and values.
+template <class TP>
 cudaError_t launch_tiles(const QuantizeParams& p, int tiles_x, cudaStream_t s) {
-  const dim3 grid((unsigned)(tiles_x * TP::kNParts), (unsigned)(p.d.B * p.d.H), (unsigned)p.n_layers);
-  return launch_dependent(quantize_tiles_kernel<TP, FOLLOWS>, grid, 32, 0, s, p);
+  const dim3 grid((unsigned)(tiles_x * (TP::kKeysFirst ? 1 : 2)), (unsigned)(p.d.B * p.d.H),
+                  (unsigned)(p.n_layers * (TP::kKeysFirst ? 2 : 1)));
+  return launch_dependent(quantize_tiles_kernel<TP>, grid, 32, 0, s, p);
 }
 
 template <int BITS, bool M16>
 cudaError_t launch_quantize_bits(const QuantizeParams& p, cudaStream_t s) {
   const Dims& d = p.d;
-  if (d.base == kKivi) {
-    const int tx = (d.T - p.tile_origin + kKiviGroup + kQTok - 1) / kQTok;
-    // keys and values in launches of their own: each kernel holds one of the
-    // two code paths, so the warps of an SM share less instruction cache
-    const cudaError_t e = launch_tiles<KiviTiles<BITS, M16, 1>>(p, tx, s);
-    if (e != cudaSuccess) return e;
-    return launch_tiles<KiviTiles<BITS, M16, 2>, true>(p, tx, s);
-  }
+  if (d.base == kKivi)
+    return launch_tiles<KiviTiles<BITS, M16>>(p, (d.T - p.tile_origin + kKiviGroup + kQTok - 1) / kQTok, s);
   const int tx = (d.T + kQTok - 1) / kQTok;
-  if (d.base == kAkvq) {
-    // keys and values in CTAs of their own: a rotated key row holds 64 fp32
-    // pairs in registers, a value row far fewer, and a kernel's threads all
-    // get the larger count -- split, twice as many key rows are resident
-    const cudaError_t e = launch_tiles<TokenTiles<BITS, M16, kAkvq, 1>>(p, tx, s);
-    if (e != cudaSuccess) return e;
-    return launch_tiles<TokenTiles<BITS, M16, kAkvq, 2>, true>(p, tx, s);
-  }
-  return launch_tiles<TokenTiles<BITS, M16, kMinMax, 3>>(p, tx, s);
+  if (d.base == kAkvq) return launch_tiles<TokenTiles<BITS, M16, kAkvq>>(p, tx, s);
+  return launch_tiles<TokenTiles<BITS, M16, kMinMax>>(p, tx, s);
 }
 
 cudaError_t launch_quantize(const QuantizeParams& p, cudaStream_t s) {
