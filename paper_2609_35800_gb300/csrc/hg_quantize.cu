@@ -12,6 +12,7 @@
 // BF16 copy path.  Codes, scales and zeros follow the group quantizer exactly
 // (round half to even of the IEEE quotient, no contraction).
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 
@@ -1836,19 +1837,31 @@ cudaError_t launch_quantize(const QuantizeParams& p, cudaStream_t s) {
 
 template <bool NORMS>
 cudaError_t launch_salient_select(const QuantizeParams& p, cudaStream_t s) {
-  const size_t smem = salient_smem_bytes(p.d);
-  if (smem > 48 * 1024) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(salient_select_kernel<NORMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   return launch_dependent(salient_select_kernel<NORMS>, dim3((unsigned)(p.d.B * p.d.H), (unsigned)p.n_layers, 1),
-                          kSalThreads, smem, s, p);
+                          kSalThreads, salient_smem_bytes(p.d), s, p);
+}
+
+// Lets the selection have the shared memory of the longest span, once per device:
+// the same value whatever the call's span, so host threads with different ones
+// cannot take it from each other.  (The default 48 KB also hold the kernel's own
+// arrays, so spans of less than that need it too.)
+cudaError_t allow_salient_smem() {
+  static std::atomic<bool> configured[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 0 && dev < 64 && configured[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  e = cudaFuncSetAttribute(salient_select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kMaxSalientSmem);
+  if (e == cudaSuccess && dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
+  return e;
 }
 
 cudaError_t launch_salient(const QuantizeParams& p, cudaStream_t s) {
   if (p.d.nq <= kSalOneLaunch) return launch_salient_select<true>(p, s);
-  const cudaError_t e = launch_dependent(
+  cudaError_t e = allow_salient_smem();  // before anything is enqueued
+  if (e != cudaSuccess) return e;
+  e = launch_dependent(
       salient_norm_kernel,
       dim3((p.d.nq + kNormTokens - 1) / kNormTokens, (unsigned)(p.d.B * p.d.H), (unsigned)p.n_layers), kNormThreads, 0, s, p);
   if (e != cudaSuccess) return e;

@@ -170,6 +170,15 @@ def test_salient_selection_in_one_or_two_launches(image):
     _run_and_check(w)
 
 
+@pytest.mark.parametrize("image", [11663, 11664, 11915, 11916])
+def test_salient_spans_around_the_default_shared_memory(image):
+    """Scores and bits of the span, with the selection's own arrays, around the 48 KB that a block may have
+    without asking for more."""
+    w = wl.custom("smem", 1, 1, 4, 2, 3, image, 9, wl.BASE_AKVQ, 4, 0, decode_steps=1, seed=9,
+                  protected=[(0, 1)], salient_permille=20)
+    _run_and_check(w)
+
+
 @pytest.mark.parametrize("image", [97, 700])
 @pytest.mark.parametrize("kind", ["one far above", "two sizes", "two values", "neighbours", "equal", "zero"])
 def test_salient_selection_of_norms_in_few_digits(kind, image):
