@@ -232,14 +232,17 @@ hg_status hg_append_kv(hg_cache *cache, int32_t layer_begin, int32_t layer_count
 
 /* Workspace bytes hg_decode_attention needs for a launch over layer_count
  * layers (any appended count up to max_new_tokens).  The workspace holds the
+ * split counters of the cache's largest launch (at most 64 layers) and the
  * split-K partials of the decode kernel (a GPU work decomposition; the paper
  * has no counterpart). */
 hg_status hg_decode_workspace_size(const hg_cache *cache, int32_t layer_count, size_t *bytes);
 
 /* Zero a workspace (cudaMemsetAsync; no counterpart in the paper).  Required
- * once before its first use; decode attention leaves it zeroed again on
- * completion.  Layout: a 512-byte header holding a status word at byte 0,
- * split counters, split partials.  workspace NULL: clear the status word of
+ * once before its first use with a cache; every launch over any layers of that
+ * cache (or of one with the same batch, KV heads and layers) leaves the split
+ * counters at zero again.  Before it serves a cache of other dimensions it has
+ * to be cleared again.  Layout: a 512-byte header holding a status word at byte
+ * 0, split counters, split partials (left as they are).  workspace NULL: clear the status word of
  * the scratch array hg_decode_attention_noalloc uses on the current device
  * (`bytes` is ignored). */
 hg_status hg_workspace_clear(void *workspace, size_t bytes, hg_stream_t stream);
@@ -279,7 +282,8 @@ hg_status hg_check_bounded_wait(void *word, uint32_t rounds, hg_stream_t stream)
  * token of that head (prefill text, image, appended), with
  * score = softmax_scale * <q, k>; softmax_scale <= 0 selects 1/sqrt(128).
  * workspace: device, >= hg_decode_workspace_size(layer_count) bytes, zeroed
- * once by hg_workspace_clear; one launch at a time may use it. */
+ * once by hg_workspace_clear; launches over different layer ranges may take
+ * turns on one that is large enough for each, one launch at a time. */
 hg_status hg_decode_attention(const hg_cache *cache, int32_t layer_begin, int32_t layer_count,
                               const void *q, void *out, float softmax_scale,
                               void *workspace, size_t workspace_bytes, hg_stream_t stream);
@@ -306,8 +310,8 @@ hg_status hg_decode_step(hg_cache *cache, int32_t layer_begin, int32_t layer_cou
  *   Scratch   the split-K workspace is one static device array of 32 MiB
  *             inside this library; every GPU that loads the library holds it
  *             until the process exits.  A launch that cannot run in 32 MiB
- *             (hg_decode_workspace_size may ask for more than the least a
- *             launch takes, for a finer split) is rejected with
+ *             (hg_decode_workspace_size may ask for more than the least that
+ *             takes, for a finer split) is rejected with
  *             HG_ERR_WORKSPACE_TOO_SMALL before anything is enqueued.
  *   Set-up    the first call on a device (with that device current) looks up
  *             the array's device address with cudaGetSymbolAddress; make that

@@ -35,7 +35,7 @@ struct hg_cache {
   size_t needed_bytes;
   // The arena as a BF16 tensor [arena_bytes / 256][128] for the decode
   // kernel's TMA loads; encoded by the first decode call.
-  mutable int least_layers = 0, least_sms = 0;  // decode_least_workspace's last answer
+  mutable int least_layers = 0, least_sms = 0;  // decode_least_scratch's last answer
   mutable size_t least_bytes = 0;
   mutable CUtensorMap arena_map;
   mutable bool arena_map_ready;
@@ -264,8 +264,17 @@ void limit_splits_by_kind(const Dims& d, DecodePlan* p) {
   p->cbP = std::max(p->cbP, at_most(d.T + d.S_new, most));
 }
 
-size_t plan_ws_bytes(const Dims& d, int count, const DecodePlan& p) {
-  return (size_t)ws_bytes(d, count, max_items_of(d, p));
+// What holds a launch's counters and partials: a caller's workspace, zeroed once,
+// or the allocation-free entry point's scratch, whose counters every call clears
+// (and which therefore holds those of the launch's own layers only).
+enum class WsKind { kWorkspace, kScratch };
+
+int counter_layers(const Dims& d, int count, WsKind kind) {
+  return kind == WsKind::kScratch ? count : ws_counter_layers(d);
+}
+
+size_t plan_ws_bytes(const Dims& d, int count, const DecodePlan& p, WsKind kind) {
+  return (size_t)ws_bytes(d, counter_layers(d, count, kind), count, max_items_of(d, p));
 }
 
 // Cost of a layer range per CTA of a full wave.
@@ -335,17 +344,18 @@ DecodePlan plan_decode(const hg_cache* c, int begin, int count, DecodePlan* leas
   return p;
 }
 
-// Least workspace a launch accepts / workspace of the plan it then runs with.
-size_t ws_least_for(const hg_cache* c, int begin, int count) {
+// Least scratch a launch accepts / workspace of the plan that it runs with.
+size_t scratch_least_for(const hg_cache* c, int begin, int count) {
   DecodePlan least;
   plan_decode(c, begin, count, &least);
-  return plan_ws_bytes(c->d, count, least);
+  return plan_ws_bytes(c->d, count, least, WsKind::kScratch);
 }
 
 size_t ws_size_for(const hg_cache* c, int begin, int count) {
   DecodePlan least;
   const DecodePlan p = plan_decode(c, begin, count, &least);
-  return std::max(plan_ws_bytes(c->d, count, least), plan_ws_bytes(c->d, count, p));
+  return std::max(plan_ws_bytes(c->d, count, least, WsKind::kWorkspace),
+                  plan_ws_bytes(c->d, count, p, WsKind::kWorkspace));
 }
 
 // A launch over more than kMaxLayersPerLaunch layers reuses the workspace for
@@ -684,10 +694,11 @@ struct Planned {
 // Decode attention over layers [layer_begin, +layer_count); with k_new / v_new
 // the step's new tokens (already counted in the cache's appended state) are
 // read from the inputs and stored into the arena by the same launch.
-// planned: what decode_checks worked out.
+// planned: what decode_checks worked out for the same kind of workspace.
 hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_count, const void* q,
                         const void* k_new, const void* v_new, void* out, float softmax_scale,
-                        void* ws, size_t ws_bytes_given, const Planned& planned, hg_stream_t stream) {
+                        void* ws, size_t ws_bytes_given, WsKind kind, const Planned& planned,
+                        hg_stream_t stream) {
   const Dims& d = c->d;
   const hg_status mst = arena_tensor_map(c);
   if (mst != HG_OK) return mst;
@@ -703,7 +714,7 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     p.n_layers = n;
     Planned pl = planned;
     if (done > 0) pl.plan = plan_decode(c, layer_begin + done, n, &pl.least);
-    p.plan = plan_ws_bytes(d, n, pl.plan) <= ws_bytes_given ? pl.plan : pl.least;
+    p.plan = plan_ws_bytes(d, n, pl.plan, kind) <= ws_bytes_given ? pl.plan : pl.least;
     p.max_items = max_items_of(d, p.plan);
     p.scale_log2 = scale * 1.4426950408889634f;
     p.q = static_cast<const uint16_t*>(q) + (size_t)done * layer_elems;
@@ -716,7 +727,7 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     p.arena_map = c->arena_map;
     p.status = reinterpret_cast<uint32_t*>(wsb);
     p.counters = reinterpret_cast<uint32_t*>(wsb + kWsHeaderBytes);
-    p.partials = reinterpret_cast<float*>(wsb + kWsHeaderBytes + ws_counter_bytes(d, n));
+    p.partials = reinterpret_cast<float*>(wsb + kWsHeaderBytes + ws_counter_bytes(d, counter_layers(d, n, kind)));
     fill_table(c, layer_begin + done, n, &p.lt);
     int most = 0, unprot = 0;
     for (int i = 0; i < n; ++i) {
@@ -738,7 +749,8 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
 }
 
 hg_status decode_checks(const hg_cache* c, int32_t layer_begin, int32_t layer_count, const void* q,
-                        void* out, float softmax_scale, void* ws, size_t ws_bytes_given, Planned* planned) {
+                        void* out, float softmax_scale, void* ws, size_t ws_bytes_given, WsKind kind,
+                        Planned* planned) {
   if (!range_ok(c, layer_begin, layer_count) || !q || !out || !ws) return HG_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(out) || !aligned16(ws)) return HG_ERR_ALIGNMENT;
   if (!(softmax_scale == softmax_scale)) return HG_ERR_INVALID_ARG;  // NaN
@@ -746,7 +758,7 @@ hg_status decode_checks(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     const int n = std::min(kMaxLayersPerLaunch, layer_count - done);
     Planned pl;
     pl.plan = plan_decode(c, layer_begin + done, n, &pl.least);
-    if (ws_bytes_given < plan_ws_bytes(c->d, n, pl.least)) return HG_ERR_WORKSPACE_TOO_SMALL;
+    if (ws_bytes_given < plan_ws_bytes(c->d, n, pl.least, kind)) return HG_ERR_WORKSPACE_TOO_SMALL;
     if (done == 0) *planned = pl;
   }
   return HG_OK;
@@ -760,17 +772,19 @@ hg_status hg_decode_attention(const hg_cache* c, int32_t layer_begin, int32_t la
                               const void* q, void* out, float softmax_scale, void* ws,
                               size_t ws_bytes_given, hg_stream_t stream) {
   Planned planned;
-  const hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given, &planned);
+  const hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given,
+                                     WsKind::kWorkspace, &planned);
   if (st != HG_OK) return st;
   return decode_launch(c, layer_begin, layer_count, q, nullptr, nullptr, out, softmax_scale, ws,
-                       ws_bytes_given, planned, stream);
+                       ws_bytes_given, WsKind::kWorkspace, planned, stream);
 }
 
 hg_status hg_decode_step(hg_cache* c, int32_t layer_begin, int32_t layer_count, const void* q,
                          const void* k_new, const void* v_new, void* out, float softmax_scale,
                          void* ws, size_t ws_bytes_given, hg_stream_t stream) {
   Planned planned;
-  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given, &planned);
+  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, ws, ws_bytes_given,
+                               WsKind::kWorkspace, &planned);
   if (st != HG_OK) return st;
   if (!k_new || !v_new) return HG_ERR_INVALID_ARG;
   if (!aligned16(k_new) || !aligned16(v_new)) return HG_ERR_ALIGNMENT;
@@ -778,7 +792,7 @@ hg_status hg_decode_step(hg_cache* c, int32_t layer_begin, int32_t layer_count, 
     if (c->appended[layer_begin + i] >= c->d.S_new) return HG_ERR_CAPACITY;
   for (int i = 0; i < layer_count; ++i) c->appended[layer_begin + i] += 1;
   st = decode_launch(c, layer_begin, layer_count, q, k_new, v_new, out, softmax_scale, ws,
-                     ws_bytes_given, planned, stream);
+                     ws_bytes_given, WsKind::kWorkspace, planned, stream);
   if (st != HG_OK)
     for (int i = 0; i < layer_count; ++i) c->appended[layer_begin + i] -= 1;
   return st;
@@ -788,13 +802,13 @@ hg_status hg_decode_step(hg_cache* c, int32_t layer_begin, int32_t layer_count, 
 
 namespace hg {
 
-hg_status decode_least_workspace(const hg_cache* c, int32_t layer_count, size_t* bytes) {
+hg_status decode_least_scratch(const hg_cache* c, int32_t layer_count, size_t* bytes) {
   // a plan per placement of the range: kept for the count asked last
   if (c && c->least_layers == layer_count && c->least_sms == sm_count()) {
     *bytes = c->least_bytes;
     return HG_OK;
   }
-  const hg_status st = workspace_bound(c, layer_count, bytes, ws_least_for);
+  const hg_status st = workspace_bound(c, layer_count, bytes, scratch_least_for);
   if (st == HG_OK) {
     c->least_layers = layer_count;
     c->least_sms = sm_count();
@@ -807,18 +821,21 @@ hg_status decode_attention_on_scratch(const hg_cache* c, int32_t layer_begin, in
                                       const void* q, void* out, float softmax_scale, void* scratch,
                                       size_t scratch_bytes, hg_stream_t stream) {
   Planned planned;
-  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, scratch, scratch_bytes, &planned);
+  hg_status st = decode_checks(c, layer_begin, layer_count, q, out, softmax_scale, scratch, scratch_bytes,
+                               WsKind::kScratch, &planned);
   if (st != HG_OK) return st;
   st = arena_tensor_map(c);
   if (st != HG_OK) return st;
   // launches over more than kMaxLayersPerLaunch layers reuse the counters of
-  // the first group, and every launch leaves them at zero again
+  // the first group, which every launch of a full group leaves at zero again (the
+  // last group has fewer layers, counters and all, and its partials may lie on
+  // the others': nothing of this call counts there any more)
   const size_t counters = ws_counter_bytes(c->d, std::min<int>(layer_count, kMaxLayersPerLaunch));
   st = cuda_status(launch_clear(static_cast<char*>(scratch) + kWsHeaderBytes, counters,
                                 reinterpret_cast<cudaStream_t>(stream)));
   if (st != HG_OK) return st;
   return decode_launch(c, layer_begin, layer_count, q, nullptr, nullptr, out, softmax_scale, scratch,
-                       scratch_bytes, planned, stream);
+                       scratch_bytes, WsKind::kScratch, planned, stream);
 }
 
 }  // namespace hg

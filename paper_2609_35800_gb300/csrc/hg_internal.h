@@ -142,9 +142,10 @@ int decode_max_splits(int G);
 hg_status decode_attention_on_scratch(const hg_cache* cache, int32_t layer_begin, int32_t layer_count,
                                       const void* q, void* out, float softmax_scale, void* scratch,
                                       size_t scratch_bytes, hg_stream_t stream);
-// Least workspace that every launch over layer_count layers accepts
-// (hg_decode_workspace_size may ask for more, for a finer work plan).
-hg_status decode_least_workspace(const hg_cache* cache, int32_t layer_count, size_t* bytes);
+// Least scratch that every launch over layer_count layers accepts
+// (hg_decode_workspace_size may ask for more: a finer work plan, and the counters
+// of the cache's largest launch).
+hg_status decode_least_scratch(const hg_cache* cache, int32_t layer_count, size_t* bytes);
 // Device address of the allocation-free entry point's scratch array on the
 // current device (its first 512 bytes are a workspace header with the status
 // word at byte 0).

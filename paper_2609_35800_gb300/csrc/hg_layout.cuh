@@ -299,16 +299,20 @@ HG_HD int nth_bit(uint64_t m, int n) {
 }
 
 // Decode workspace: a 512-byte header (status word at byte 0), a counter per
-// (layer, row, head), then partial results
-// [layer][row][head][split][G][kD + 4] floats (m, l, two pad, o[kD]).
+// (layer, row, head) of `counter_layers` layers, then partial results
+// [layer][row][head][split][G][kD + 4] floats (m, l, two pad, o[kD]).  A launch
+// counts on zeroed counters and leaves them at zero, so no launch may keep
+// partials where another one counts: in a caller's workspace the counters are
+// those of the cache's largest launch, whatever the launch (ws_counter_layers).
 constexpr uint64_t kWsHeaderBytes = 512;
 constexpr uint32_t kStatusWaitTimeout = 1u;  // a wait for a tile's data ran out
-HG_HD uint64_t ws_counter_bytes(const Dims& d, int n_layers) {
-  return align_up((uint64_t)n_layers * d.B * d.H * 4);
+HG_HD int ws_counter_layers(const Dims& d) { return d.L < kMaxLayersPerLaunch ? d.L : kMaxLayersPerLaunch; }
+HG_HD uint64_t ws_counter_bytes(const Dims& d, int counter_layers) {
+  return align_up((uint64_t)counter_layers * d.B * d.H * 4);
 }
 HG_HD uint64_t ws_partial_floats_per_split(const Dims& d) { return (uint64_t)d.G * (kD + 4); }
-HG_HD uint64_t ws_bytes(const Dims& d, int n_layers, int max_items) {
-  return kWsHeaderBytes + ws_counter_bytes(d, n_layers) +
+HG_HD uint64_t ws_bytes(const Dims& d, int counter_layers, int n_layers, int max_items) {
+  return kWsHeaderBytes + ws_counter_bytes(d, counter_layers) +
          align_up((uint64_t)n_layers * d.B * d.H * max_items * ws_partial_floats_per_split(d) * 4);
 }
 

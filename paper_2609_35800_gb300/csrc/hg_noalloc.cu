@@ -72,7 +72,7 @@ extern "C" hg_status hg_decode_attention_noalloc(const hg_cache* cache, int32_t 
   if (!aligned16(q) || !aligned16(out)) return HG_ERR_ALIGNMENT;
   if (!(softmax_scale == softmax_scale)) return HG_ERR_INVALID_ARG;
   size_t need = 0;
-  hg_status st = hg::decode_least_workspace(cache, layer_count, &need);
+  hg_status st = hg::decode_least_scratch(cache, layer_count, &need);
   if (st != HG_OK) return st;
   if (need > kScratchBytes) return HG_ERR_WORKSPACE_TOO_SMALL;
   void* scratch = nullptr;

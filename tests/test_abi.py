@@ -283,6 +283,19 @@ def test_workspace_size_grows_with_layers(lib):
     assert 0 < one < allw
 
 
+def test_workspace_counters_do_not_depend_on_the_launch(lib):
+    """A one-layer call's workspace has room for the split counters of the whole cache (up to 64 layers, the most
+    of one launch) before its partials: the sizes of two caches that differ in layers only differ by those."""
+    def one_layer(layers):
+        cache, _, _ = _fake_cache(wl.custom("ws", layers, 8, 8, 8, 20, 96, 20, wl.BASE_MINMAX, 2, 0, decode_steps=4,
+                                            protected=[]))
+        return hg.hg_decode_workspace_size(cache, 1)
+
+    counters = lambda layers: (layers * 8 * 8 * 4 + 255) // 256 * 256
+    for layers in (2, 33, 64, 80):
+        assert one_layer(layers) - one_layer(1) == counters(min(layers, 64)) - counters(1), layers
+
+
 def test_status_strings(lib):
     for s in range(8):
         assert isinstance(hg.hg_status_string(s), str) and hg.hg_status_string(s)

@@ -79,6 +79,46 @@ def test_decode_layers_with_different_appended_counts(base, keys_only, prefix):
             assert_close(bits16(out[layer, row:row + 1]), ref, "layer %d row %d" % (layer, row))
 
 
+def test_more_layers_than_one_launch_holds():
+    """70 layers in one call: launches of 64 and of 6 layers on one workspace, step after step."""
+    w = wl.custom("deep", 70, 1, 8, 8, 8, 72, 8, wl.BASE_MINMAX, 2, 0, decode_steps=3, seed=19, protected=[(1, 0), (66, 3)])
+    runner = CacheRunner(w)
+    kept = runner.quantize_all(keep=True)
+    news = []
+    for step in range(3):
+        k_new, v_new = wl.step_new_kv(w, step, "cuda")
+        q = wl.step_query(w, step, "cuda")
+        out = torch.full_like(q, float("nan"))
+        runner.decode_step(step, q=q, k_new=k_new, v_new=v_new, out=out)
+        news.append((k_new, v_new))
+        for layer in (0, 1, 15, 16, 40, 63, 64, 66, 69):
+            ref = _row_reference(runner, layer, 0, *kept[layer], q, news)
+            assert_close(bits16(out[layer, :1]), ref, "step %d layer %d" % (step, layer))
+
+
+@pytest.mark.parametrize("base,group", [(wl.BASE_MINMAX, 4), (wl.BASE_KIVI, 1)])
+def test_layer_ranges_take_turns_on_one_workspace(base, group):
+    """One layer, all layers, two layers, all layers on a workspace that was cleared once: the counters of the
+    larger launches (2 KB) lie beyond those of a layer (384 bytes)."""
+    w = wl.custom("turns", 6, 6, 16 * group, 16, 10, 96, 40, base, 2, 0, decode_steps=1, seed=21,
+                  protected=[(0, 1), (4, 5)])
+    runner = CacheRunner(w)
+    kept = runner.quantize_all(keep=True)
+    k_new, v_new = wl.step_new_kv(w, 0, "cuda")
+    hg.hg_append_kv(runner.cache, 0, w.layers, k_new, v_new)
+    q = wl.step_query(w, 0, "cuda")
+    refs = {}
+    for begin, count in ((0, 1), (0, 6), (3, 2), (0, 6), (5, 1), (1, 5), (0, 6)):
+        out = torch.full_like(q[begin:begin + count], float("nan"))
+        hg.hg_decode_attention(runner.cache, begin, count, q[begin:begin + count], out, SIGMA, runner.ws, runner.ws_bytes)
+        for layer in range(begin, begin + count):
+            for row in (0, 5):
+                if (layer, row) not in refs:
+                    refs[layer, row] = _row_reference(runner, layer, row, *kept[layer], q, [(k_new, v_new)])
+                assert_close(bits16(out[layer - begin, row:row + 1]), refs[layer, row],
+                             "layers %d+%d layer %d row %d" % (begin, count, layer, row))
+
+
 def _decode_against_oracle(w, kept, steps, q_scale=1.0, v_max=1.0):
     """Append `steps` tokens in fused steps on a cache quantized from `kept`; the last step's outputs, every row.
     The tolerance is the suite's (2e-3 + 1e-2 |r| for values of order one) with its absolute part in units of
