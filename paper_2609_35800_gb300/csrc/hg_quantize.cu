@@ -128,13 +128,22 @@ __device__ __forceinline__ bool chunk_T(const uint64_t (&x2)[4], uint64_t mn2, u
   return __vcmpleu2(low, 0x00070007u) == 0u;
 }
 
+// max(|a|, |b|, |c|); NaN if one of them is.
+__device__ __forceinline__ float abs_max3(float a, float b, float c) {
+  float d;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // 4-bit codes of a chunk's four channel pairs, packed in channel order, on the
 // fp32 pipe: t = RN(d r + 2^23) holds the rounded quotient f in its low bits, and
 // four of them become a 16-bit word by one packed FMA (f_i + 256 f_{i+2}) and one
 // integer multiply-add.  Returns true when no quotient is near a tie: e = d r - f
 // is within 2e-6 of the exact quotient's distance from f (1 / scale and the
 // reference division round by 2^-24 each, quotients below 16), so below 0.499995
-// the code is f.  (chunk_T and chunk_bits_T take four integer operations per
+// the code is f.  A NaN (an element's, or infinity times a step of infinity) spoils
+// the word's other codes too: `top` keeps it, and the chunk counts as near a tie.
+// (chunk_T and chunk_bits_T take four integer operations per
 // element, and the integer pipe bound these rows: InternVL2.5-8B-shaped prefill with
 // salient tokens, 4 layers one by one, 766 -> 729 us.)
 __device__ __forceinline__ bool chunk_codes4(const uint64_t (&x2)[4], uint64_t mn2, uint64_t r2, uint32_t& lo) {
@@ -147,7 +156,7 @@ __device__ __forceinline__ bool chunk_codes4(const uint64_t (&x2)[4], uint64_t m
     t[i] = f32x2_fma(d, r2, m2);
     g[i] = f32x2_sub(m2, t[i]);  // -f
     const uint64_t e = f32x2_fma(d, r2, g[i]);
-    top = fmaxf(fmaxf(fabsf(__uint_as_float((uint32_t)e)), fabsf(__uint_as_float((uint32_t)(e >> 32)))), top);
+    top = abs_max3(__uint_as_float((uint32_t)e), __uint_as_float((uint32_t)(e >> 32)), top);
   }
   const uint64_t u = f32x2_fma(g[1], c256, t[0]), v = f32x2_fma(g[3], c256, t[2]);
   lo = prmt((uint32_t)u + 16u * (uint32_t)(u >> 32), (uint32_t)v + 16u * (uint32_t)(v >> 32), 0x5410);
@@ -530,8 +539,9 @@ __device__ __forceinline__ void chunk_near_tie(const uint32_t (&a)[8], X x, floa
 // stored, coded again by the exact rule, each written over its bits: word k (4
 // bits), or half k % 2 of word k / 2 (2 and 3 bits) and, at 3 bits, byte
 // ((k >> 1) & 1) | ((k & 1) << 1) of plane word 8 + k / 4 (the layout of
-// store_group).  The other elements' codes are read back and kept: they were
-// decided by the fast rule.  The loop runs over a thread's own elements near a
+// store_group).  The other elements' codes, which the fast rule decided, are read
+// back and kept, or (4 bits, where a NaN would have spoiled them) taken from T'
+// again.  The loop runs over a thread's own elements near a
 // tie (mostly one), so the threads of a warp divide side by side; with the eight
 // elements in turn a warp went through nearly all eight for its threads'
 // different ones.  One layer of 862 tokens at 4 bits 5.2 -> 4.4 us; 17 layers of
@@ -553,7 +563,13 @@ __device__ __forceinline__ void recode_near_ties(const uint4* r4, int k, uint64_
   uint32_t* lw = codes + (BITS == 4 ? k : k >> 1);
   uint32_t* hw = codes + 8 + (k >> 2);
   const int ls = BITS == 4 ? 0 : 16 * (k & 1), hs = 8 * (((k >> 1) & 1) | ((k & 1) << 1));
-  uint32_t lo = *lw, hb = BITS == 3 ? *hw : 0u;
+  uint32_t lo, hb;
+  if (BITS == 4) {
+    chunk_bits_T<4>(a, lo, hb);
+  } else {
+    lo = *lw;
+    hb = BITS == 3 ? *hw : 0u;
+  }
   while (el) {
     const int i = __ffs(el) - 1;
     el &= el - 1;

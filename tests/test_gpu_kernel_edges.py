@@ -302,6 +302,55 @@ def test_every_code_on_a_tie(base, bits, meta_bits):
     check_arena_layer(runner, 0, bits16(k), bits16(v), oracle_layer(runner, 0, bits16(k), bits16(v)))
 
 
+@pytest.mark.parametrize("meta_bits", [64, 32])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("base", [wl.BASE_MINMAX, wl.BASE_KIVI, wl.BASE_AKVQ])
+def test_non_finite_elements_keep_to_themselves(base, bits, meta_bits):
+    """A NaN or an infinity (at every position of a chunk, one per row and key group): the metadata and the
+    codes of the group's other elements are the oracle's.  (The element's own code has no defined value; rotated
+    keys have none to compare, since the rotation spreads it over the row.)"""
+    w = wl.custom("nonfinite", 1, 1, 4, 2, 0, 128, 0, base, bits, 0, seed=18, protected=[], residual=0,
+                  meta_bits=meta_bits)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    x = torch.randn(2, 1, 2, 128, 128, generator=g, device="cuda")
+    special = torch.zeros(128, 128, dtype=torch.bool, device="cuda")
+    tok = torch.arange(128, device="cuda")
+    # token t: channel (t * 9 + 1) % 128, never a group's first element (which starts the oracle's extremes)
+    ch = (tok * 9 + 1) % 128
+    keep = (ch % 32 != 0) & (tok % 32 != 0)
+    special[tok[keep], ch[keep]] = True
+    value = torch.where(tok % 2 == 0, float("nan"), float("inf"))
+    x = torch.where(special, value[:, None], x).bfloat16()
+    k, v = x[0].contiguous(), x[1].contiguous()
+    if base == wl.BASE_AKVQ:
+        k = torch.randn(k.shape, generator=g, device="cuda").bfloat16()
+    runner = CacheRunner(w)
+    hg.hg_quantize_kv(runner.cache, 0, [k], [v])
+    torch.cuda.synchronize()
+    o = oracle_layer(runner, 0, bits16(k), bits16(v))
+    arena = runner.arena.cpu().numpy()
+    other = ~special.cpu().numpy()
+    for h in range(2):
+        r = hg.hg_cache_head_regions(runner.cache, 0, h)
+        for off, moff, words, meta, name in ((r.kq, r.kqm, o["k_words"][0, h], o["k_meta"][0, h], "k"),
+                                             (r.vq, r.vqm, o["v_words"][0, h], o["v_meta"][0, h], "v")):
+            got = arena[off:off + words.nbytes].view(np.uint32)
+            key_groups = name == "k" and base == wl.BASE_KIVI
+            n = 32 if key_groups else 128  # codes of one packed run
+
+            def codes(a):
+                c = np.stack([oracle.unpack(row, n, bits) for row in a.reshape(-1, n * bits // 32)])
+                return c.reshape(4, 128, 32).transpose(0, 2, 1).reshape(128, 128) if key_groups else c
+
+            differ = codes(got) != codes(words)
+            if name == "v" or base != wl.BASE_AKVQ:
+                differ &= other
+            assert not differ.any(), (name, h, np.argwhere(differ)[:4])
+            m = arena[moff:moff + meta.size * (2 if meta_bits == 32 else 4)]
+            want = meta.astype(np.float16) if meta_bits == 32 else meta
+            assert np.array_equal(m.view(want.dtype), want), (name, h, "metadata")
+
+
 @pytest.mark.parametrize("base,group", [(wl.BASE_MINMAX, 7), (wl.BASE_KIVI, 1), (wl.BASE_AKVQ, 12)])
 def test_append_and_allocation_free_attention_back_to_back(base, group):
     """Tokens appended and attended layer by layer with nothing waiting in between (append, counter clear and
