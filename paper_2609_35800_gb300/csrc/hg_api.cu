@@ -540,6 +540,7 @@ hg_status hg_quantize_kv(hg_cache* c, int32_t layer_begin, int32_t layer_count,
     p.tile_origin = d.s % 32;
     fill_table(c, layer_begin + done, n, &p.lt);
     p.gt.gc = c->gc;
+    p.neg_zero2 = kNegZero2;
     for (int i = 0; i < n; ++i) {
       p.gt.off[i] = c->layer_off[layer_begin + done + i];
       p.k[i] = static_cast<const uint16_t*>(k[done + i]);
@@ -575,7 +576,7 @@ hg_status hg_dequantize_kv(const hg_cache* c, int32_t layer_begin, int32_t layer
     fill_table(c, layer_begin + done, n, &p.lt);
     p.appended = appended;
     p.out_fp32 = out_fp32 ? 1 : 0;
-    p.neg_zero2 = 0x8000000080000000ull;
+    p.neg_zero2 = kNegZero2;
     p.k_out = static_cast<char*>(k_out) + (size_t)done * layer_bytes;
     p.v_out = static_cast<char*>(v_out) + (size_t)done * layer_bytes;
     const hg_status st = cuda_status(launch_dequantize(p, sm_count(), reinterpret_cast<cudaStream_t>(stream)));

@@ -31,9 +31,12 @@ struct QuantizeParams {
   int tile_origin;  // s mod 32: KIVI-style tile i covers [tile_origin - 32 + 32 i, +32) clipped to [0, T)
   LayerTable lt;
   GeomTable gt;
+  uint64_t neg_zero2;  // two fp32 -0 (see f32x2_product)
   const uint16_t* k[kMaxLayersPerLaunch];
   const uint16_t* v[kMaxLayersPerLaunch];
 };
+
+constexpr uint64_t kNegZero2 = 0x8000000080000000ull;  // two fp32 -0
 
 struct DequantParams {
   Dims d;
@@ -44,7 +47,7 @@ struct DequantParams {
   int out_fp32;
   void* k_out;   // [n_layers][B][H][T + appended][128]
   void* v_out;
-  uint64_t neg_zero2;  // two fp32 -0 (see scale_add)
+  uint64_t neg_zero2;  // two fp32 -0 (see f32x2_product)
 };
 
 struct AppendParams {

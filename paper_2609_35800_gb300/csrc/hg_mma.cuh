@@ -30,8 +30,8 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
 }
 
 // Packed pairs of binary32 values (Blackwell's paired fp32 pipe): each half is
-// one IEEE operation rounded to nearest even, exactly as the scalar form.
-// Element 0 is the low 32 bits.
+// one IEEE operation rounded to nearest even, as the scalar form.  Element 0 is
+// the low 32 bits.
 __device__ __forceinline__ uint64_t f32x2(uint32_t lo, uint32_t hi) {
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
@@ -47,16 +47,16 @@ __device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
-__device__ __forceinline__ uint64_t f32x2_mul(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
 __device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+// The rounded product a b, whatever is done with it: an FMA with nz = (-0, -0), the
+// same value.  mul.rn.f32x2 and an addition that takes its result may become one
+// FMA, which does not round the product (seen with this compiler), so nz is a
+// launch parameter that it cannot see through.
+__device__ __forceinline__ uint64_t f32x2_product(uint64_t a, uint64_t b, uint64_t nz) { return f32x2_fma(a, b, nz); }
 
 // Programmatic dependent launch (PTX griddepcontrol): let the next grid on the
 // stream be scheduled once every CTA of this one has issued this (or exited),

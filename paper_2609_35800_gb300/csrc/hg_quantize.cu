@@ -769,8 +769,8 @@ __device__ __forceinline__ uint64_t shfl_xor_pair(unsigned mask, uint64_t x, int
 }
 
 template <int BITS, bool M16, int SPLIT>
-__device__ __forceinline__ void quantize_row_rotated(const char* row_s, int hh, unsigned pmask, uint32_t* codes,
-                                                     char* meta, size_t mi) {
+__device__ __forceinline__ void quantize_row_rotated(const char* row_s, int hh, unsigned pmask, uint64_t nz,
+                                                     uint32_t* codes, char* meta, size_t mi) {
   constexpr int NP = 64 / SPLIT;  // pairs per thread
   constexpr int NK = 16 / SPLIT;  // chunks per thread
   const uint32_t* r32 = reinterpret_cast<const uint32_t*>(row_s) + NP * hh;
@@ -805,7 +805,7 @@ __device__ __forceinline__ void quantize_row_rotated(const char* row_s, int hh, 
     const uint32_t cb = __float_as_uint(hadamard_c());
     const uint64_t c2 = f32x2(cb, cb);
 #pragma unroll
-    for (int m = 0; m < NP; ++m) xp[m] = f32x2_mul(xp[m], c2);
+    for (int m = 0; m < NP; ++m) xp[m] = f32x2_product(xp[m], c2, nz);
   }
   // min / max of the rotated vector (exact; signed zeros folded to +0)
   float mn = fminf(pair_lo(xp[0]), pair_hi(xp[0])), mx = fmaxf(pair_lo(xp[0]), pair_hi(xp[0]));
@@ -1036,7 +1036,8 @@ struct TokenTiles {
       if (coded && hd.cls == kQuantized && !sal) {
         uint32_t* crow = reinterpret_cast<uint32_t*>(Lb + hd.kq + b * hd.kq_bs) + (size_t)ci * W;
         if constexpr (SPLIT == 2)
-          quantize_row_rotated<BITS, M16, SPLIT>(row_s, hh, pmask, crow, Lb + hd.kqm + b * hd.kqm_bs, ci);
+          quantize_row_rotated<BITS, M16, SPLIT>(row_s, hh, pmask, p.neg_zero2, crow, Lb + hd.kqm + b * hd.kqm_bs,
+                                                 ci);
         else if constexpr (BASE != kAkvq)
           quantize_row_token<BITS, M16>(row_s, crow, Lb + hd.kqm + b * hd.kqm_bs, ci);
         return;
@@ -1480,11 +1481,9 @@ __device__ __forceinline__ Codes8 load_codes8(const char* row, int c) {
 __device__ __forceinline__ uint32_t int_magic(uint32_t c) { return c | 0x4B000000u; }
 __device__ __forceinline__ uint64_t magic_pair() { return f32x2(0x4B000000u, 0x4B000000u); }
 
-// fl(fl(x s) + z) of two elements.  The product is an FMA with nz = (-0, -0),
-// the same value: the compiler contracts a packed multiply and add, explicitly
-// rounded or not, into one FMA, so nz is a launch parameter it cannot see through.
+// fl(fl(x s) + z) of two elements.
 __device__ __forceinline__ uint64_t scale_add(uint64_t x, uint64_t s, uint64_t z, uint64_t nz) {
-  return f32x2_add(f32x2_fma(x, s, nz), z);
+  return f32x2_add(f32x2_product(x, s, nz), z);
 }
 
 // fl(fl(code * scale) + zero) of eight codes.

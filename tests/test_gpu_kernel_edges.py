@@ -351,6 +351,26 @@ def test_non_finite_elements_keep_to_themselves(base, bits, meta_bits):
             assert np.array_equal(m.view(want.dtype), want), (name, h, "metadata")
 
 
+@pytest.mark.parametrize("meta_bits", [64, 32])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_rotated_keys_with_one_channel_far_above_the_rest(bits, meta_bits):
+    """Channel 0 up to a million times the others: every rotated value of a row is far from zero against the
+    row's range, so the group minimum's subtraction shows whether the rotated values were rounded first.  Bit for
+    bit."""
+    w = wl.custom("onechannel", 1, 2, 4, 2, 3, 600, 5, wl.BASE_AKVQ, bits, 0, seed=17, protected=[], residual=0,
+                  meta_bits=meta_bits)
+    g = torch.Generator(device="cuda").manual_seed(8)
+    k = torch.randn(2, 2, w.seq_len, 128, generator=g, device="cuda")
+    v = torch.randn(2, 2, w.seq_len, 128, generator=g, device="cuda").bfloat16()
+    k[..., 0] = torch.exp2(torch.rand(k.shape[:3], generator=g, device="cuda") * 14 + 6)
+    k[:, 1, :, 0] *= -1
+    k = k.bfloat16().contiguous()
+    runner = CacheRunner(w)
+    hg.hg_quantize_kv(runner.cache, 0, [k], [v])
+    torch.cuda.synchronize()
+    check_arena_layer(runner, 0, bits16(k), bits16(v), oracle_layer(runner, 0, bits16(k), bits16(v)))
+
+
 @pytest.mark.parametrize("base,group", [(wl.BASE_MINMAX, 7), (wl.BASE_KIVI, 1), (wl.BASE_AKVQ, 12)])
 def test_append_and_allocation_free_attention_back_to_back(base, group):
     """Tokens appended and attended layer by layer with nothing waiting in between (append, counter clear and
