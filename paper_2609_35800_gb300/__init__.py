@@ -172,8 +172,11 @@ def _stream(stream):
     """cudaStream_t handle: a torch.cuda.Stream, an int, or None (current torch stream)."""
     if stream is None:
         import torch
-        if torch.cuda.is_initialized():  # the handle alone, without a Stream object around it
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        if torch.cuda.is_initialized():
+            try:  # the handle alone, without a Stream object around it; not part of torch's public interface
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:
+                pass
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream

@@ -119,3 +119,17 @@ def test_generated_inputs_pass_the_extent_checks(name):
     _raises(lambda: hg.hg_dequantize_kv(c, 0, 1, k32, k32, True), cuda)
     _raises(lambda: hg.hg_dequantize_kv(c, 0, 1, k, v, False), cuda)
     _raises(lambda: hg.hg_workspace_clear(ws), cuda)
+
+
+@pytest.mark.parametrize("absent", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_torch_internals(monkeypatch, absent):
+    """Where torch does not have its raw-stream functions, the public interface gives the current stream."""
+    class Stream:
+        cuda_stream = 1234
+
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.setattr(torch._C, name, lambda *a: 0, raising=False)
+    monkeypatch.delattr(torch._C, absent)
+    assert hg._stream(None) == 1234
