@@ -259,7 +259,7 @@ def hg_quantize_kv(cache, layer_begin, k_list, v_list, stream=None):
     ptrs = []
     for x in (*k_list, *v_list):
         if x is None or isinstance(x, int):
-            ptrs.append(x or 0)
+            ptrs.append((x or 0) & 0xffffffffffffffff)  # any integer, as ctypes takes one for a pointer
         elif x.is_cuda and x.is_contiguous() and x.nbytes >= need:
             ptrs.append(x.data_ptr())
         else:

@@ -133,3 +133,15 @@ def test_current_stream_without_torch_internals(monkeypatch, absent):
         monkeypatch.setattr(torch._C, name, lambda *a: 0, raising=False)
     monkeypatch.delattr(torch._C, absent)
     assert hg._stream(None) == 1234
+
+
+@pytest.mark.parametrize("address", [-8, (1 << 64) + 8])
+def test_integer_addresses_reach_the_library(cache, address):
+    """Integers that are no 64-bit address are cut to one, as for every other entry point, and the library's
+    alignment check refuses these."""
+    with pytest.raises(hg.HGError) as e:
+        hg.hg_quantize_kv(cache, 0, [address], [1 << 40], stream=0)
+    assert e.value.status == 2
+    with pytest.raises(hg.HGError) as e:
+        hg.hg_append_kv(cache, 0, 1, address, 1 << 40, stream=0)
+    assert e.value.status == 2
