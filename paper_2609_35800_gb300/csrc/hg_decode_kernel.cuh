@@ -317,31 +317,38 @@ __device__ __forceinline__ bool wait_tile(uint32_t bar, uint32_t parity, volatil
 }
 
 // A warp's pipeline over its token range [wb, we): fill i uses slot i % SLOTS
-// and phase i / SLOTS of that slot's mbarrier; fills are consumed in order.
-template <int BITS, int NT, int KM, int VM, int MB, bool COLS>
+// and phase i / SLOTS of that slot's mbarrier; fills are consumed in order.  The
+// CTA's chunk is divided in units of GRAN tokens.
+template <int BITS, int NT, int KM, int VM, int MB, bool COLS, int GRAN>
 struct WarpPipe {
   using TL = Tile<BITS, KM, VM, MB, COLS>;
   static constexpr int SLOTS = TL::slots, FPT = TL::SPLIT ? 2 : 1;  // fills per tile
+  // A tile of KIVI-style keys is a whole group, of which only one half may be the
+  // warp's: tiles then start at multiples of ALIGN.
+  static constexpr int ALIGN = KM == K_KIVI && GRAN < kKiviGroup ? kKiviGroup : 1;
   const Seg& sg;
   const DecodeParams& p;
-  int wb, we, n_tiles, n_fills, issued;
+  int wb, we;  // the warp's tokens; wb of its first tile
+  int skip;    // tokens of the first tile that are another warp's
+  int n_tiles, n_fills, issued;
   int fs, fp;  // slot and phase parity of the next fill to consume
   char* buf;
   uint32_t buf0, bars;
   volatile int* abort;
 
-  // The warp's quarter of the chunk [tb, te), in whole units of GRAN tokens.
+  // The warp's quarter of the chunk [tb, te).
   // Only the first tile goes in flight now: with every CTA of the launch
   // starting at once, first tiles alone make a burst the memory system serves
   // quickly, so compute starts early; the other slots are filled once the
   // first tile has landed.  (Filling them all at once measured the same, also
   // in launches of a few dozen CTAs.)
-  __device__ __forceinline__ WarpPipe(char* smem, int warp, const Seg& s, const DecodeParams& dp, int tb, int te,
-                                      int gran)
+  __device__ __forceinline__ WarpPipe(char* smem, int warp, const Seg& s, const DecodeParams& dp, int tb, int te)
       : sg(s), p(dp), fs(0), fp(0) {
-    const int span = (max(te - tb, 0) + kWarps * gran - 1) / (kWarps * gran) * gran;
+    const int span = (max(te - tb, 0) + kWarps * GRAN - 1) / (kWarps * GRAN) * GRAN;
     wb = min(tb + warp * span, te);
     we = min(wb + span, te);
+    skip = wb < we ? wb % ALIGN : 0;
+    wb -= skip;
     n_tiles = (max(we - wb, 0) + TL::tokens - 1) / TL::tokens;
     n_fills = n_tiles * FPT;
     buf = smem + kStageOff + warp * kWarpBuf;
@@ -353,7 +360,8 @@ struct WarpPipe {
       for (int i = 0; i < issued; ++i) issue(i, i);
   }
   __device__ __forceinline__ void issue(int slot, int i) {
-    issue_fill<BITS, KM, VM, MB, COLS>(buf0 + slot * TL::slot_bytes, bars + 8 * slot, sg, i, wb, we, &p.arena_map);
+    issue_fill<BITS, KM, VM, MB, COLS>(buf0 + slot * TL::slot_bytes, bars + 8 * slot, sg, i, wb,
+                                       (we + ALIGN - 1) / ALIGN * ALIGN, &p.arena_map);
   }
   __device__ __forceinline__ int tile_tokens(int it) const { return min(TL::tokens, we - wb - it * TL::tokens); }
   __device__ __forceinline__ const char* slot() const { return buf + fs * TL::slot_bytes; }
@@ -641,13 +649,14 @@ __device__ __forceinline__ void vscale_update(WarpState<NT, NZ>& ws, float smax)
 }
 
 // ---------------------------------------------------------------------------
-// One tile of a warp: kst / vst its K and V in shared memory.  between() runs
+// One tile of a warp: kst / vst its K and V in shared memory, of which the tokens
+// [skip, nvalid) are the warp's (skip: KIVI-style keys, 0 or 16).  between() runs
 // after the last read of kst by a SPLIT tile (one slice) and returns false
 // when the values did not arrive; the tile's probabilities are then dropped.
 // ---------------------------------------------------------------------------
 template <int BITS, int NT, int KM, int VM, bool ROT, int MB, class F>
 __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws, const char* kst, const char* vst,
-                                             int nvalid, const uint32_t (&qb)[NT][8][2],
+                                             int skip, int nvalid, const uint32_t (&qb)[NT][8][2],
                                              const uint32_t (&ql)[NT][8][2], const float* q_s,
                                              const float (&kq)[NT][2], const float (&s0)[NT][2],
                                              float scale_log2, int lane, F&& between) {
@@ -801,6 +810,7 @@ __device__ __forceinline__ void compute_tile(WarpState<NT, NZOf<VM>::value>& ws,
     for (int s = 0; s < SPU; ++s) {
       const int tok0 = (u * SPU + s) * 16;
       if (tok0 >= nvalid) break;
+      if (SPU > 1 && tok0 < skip) continue;
       float ks[NT][4];  // KIVI-style: this slice's scores against the scaled queries
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt)
@@ -1146,7 +1156,7 @@ __device__ __forceinline__ void stage_queries(float* q_s, float* qn, const uint4
   }
 }
 
-template <int BITS, int NT, int KM, int VM, bool ROT, int MB>
+template <int BITS, int NT, int KM, int VM, bool ROT, int MB, int GRAN = 16>
 __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int te, const DecodeParams& p,
                                          const uint4 (&qv)[QPieces<NT>::n], int G, float* parts) {
   using TL = Tile<BITS, KM, VM, MB>;
@@ -1159,7 +1169,7 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
   float* q_s = reinterpret_cast<float*>(smem + SmemLayout<NT>::q);
   const float scale_log2 = p.scale_log2;
 
-  WarpPipe<BITS, NT, KM, VM, MB, false> pipe(smem, warp, sg, p, tb, te, (KM == K_KIVI) ? kKiviGroup : 16);
+  WarpPipe<BITS, NT, KM, VM, MB, false, GRAN> pipe(smem, warp, sg, p, tb, te);
 
   // Queries of this KV head's group (fp32, rows >= G zero), rotated for
   // AKVQ-style coded keys.
@@ -1227,8 +1237,8 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
     const char* kst = pipe.slot();
     const char* vst = TL::SPLIT ? pipe.next_slot() : kst;
     bool ok = true;
-    compute_tile<BITS, NT, KM, VM, ROT, MB>(ws, kst, vst, pipe.tile_tokens(it), qb, ql, q_s, kq, s0, scale_log2, lane,
-                                            [&]() {
+    compute_tile<BITS, NT, KM, VM, ROT, MB>(ws, kst, vst, it == 0 ? pipe.skip : 0, pipe.tile_tokens(it), qb, ql, q_s, kq,
+                                            s0, scale_log2, lane, [&]() {
                                               pipe.refill();
                                               return ok = pipe.landed();
                                             });
@@ -1490,7 +1500,7 @@ __device__ __forceinline__ void run_item_cols(char* smem, const Seg& sg, int tb,
   // scores and probabilities of the warp's tile, [2][64], behind the QC query rows
   static_assert((2 * kQRow + kWarps * 128) * 4 <= 8 * kQRow * 4, "the query rows above the first two hold the scores");
   float* ps = q_s + 2 * kQRow + warp * 128;
-  WarpPipe<BITS, 1, KM, V_KIVI, MB, true> pipe(smem, warp, sg, p, tb, te, (KM == K_KIVI) ? kKiviGroup : 16);
+  WarpPipe<BITS, 1, KM, V_KIVI, MB, true, KM == K_KIVI ? kKiviGroup : 16> pipe(smem, warp, sg, p, tb, te);
 
   float* qn = reinterpret_cast<float*>(smem + SmemLayout<1>::qn);
   stage_queries<1, KM == K_BF16 ? -1 : 15>(q_s, qn, qv, tid);
@@ -1660,6 +1670,17 @@ __device__ __forceinline__ void locate_item(const DecodeParams& p, int x, int& l
   h = all ? n : nth_bit(prot ? mask : ~mask, n);
 }
 
+// Tokens in which the warps of a CTA divide a chunk of KIVI-style codes (run_item).
+// Half groups keep the four warps' shares within 16 tokens of each other; the two
+// warps that share a group both scale its queries.  In whole groups a chunk of 160
+// tokens was 64, 64, 32 and none.  One layer or a few in one call: 9 rows of 5 KV
+// heads, G = 12, 2,112 tokens at 4 bits 52.0 -> 49.7 us; 10 rows of 8, G = 8, 1,024
+// tokens at 3 bits 58.7 -> 55.7 us; small launches up to 15% (11.8 -> 10.1 us), no
+// change to -2% where the shares were even.  3-bit codes with four CTAs per SM, which
+// are short of registers, stay with whole groups (44.5 us, 48.6 in halves).
+template <int BITS, int NT, int QC>
+__host__ __device__ constexpr int kivi_unit() { return BITS == 3 && NT == 1 && QC == 0 ? kKiviGroup : 16; }
+
 // NT: 8-query column tiles of the MMAs.  QC: queries per KV head where
 // run_item_cols serves the KIVI-style items (1 or 2), else 0; -1: the same with
 // registers for three CTAs per SM instead of four.
@@ -1771,7 +1792,7 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
     if constexpr (QC > 0)
       run_item_cols<BITS, QC, K_KIVI, MB>(smem, sg, tb, te, p, qv, parts);
     else if constexpr (BASE == kKivi)
-      run_item<BITS, NT, K_KIVI, V_KIVI, false, MB>(smem, sg, tb, te, p, qv, G, parts);
+      run_item<BITS, NT, K_KIVI, V_KIVI, false, MB, kivi_unit<BITS, NT, QC>()>(smem, sg, tb, te, p, qv, G, parts);
     else if constexpr (BASE == kAkvq)
       run_item<BITS, NT, K_TOKEN, V_TOKEN, true, MB>(smem, sg, tb, te, p, qv, G, parts);
     else

@@ -163,6 +163,18 @@ def test_kivi_grouped_queries_in_one_wave_and_more(batch, bits):
     _decode_against_oracle(w, [wl.layer_kv(w, layer, "cuda") for layer in range(2)], 1)
 
 
+@pytest.mark.parametrize("meta_bits", [64, 32])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("group", [3, 8, 12])
+def test_kivi_groups_shared_by_two_warps(group, bits, meta_bits):
+    """Three and more queries per KV head over KIVI-style codes: spans whose quarter ends in the middle of a
+    32-token group (one to seven groups, and several chunks), so that its halves are two warps'."""
+    for image in (32, 64, 96, 160, 224, 1120):
+        w = wl.custom("halves%d" % image, 1, 2, 2 * group, 2, 7, image, 5, wl.BASE_KIVI, bits, 0, decode_steps=1, seed=23,
+                      protected=[(0, 1)], residual=0, meta_bits=meta_bits)
+        _decode_against_oracle(w, [wl.layer_kv(w, 0, "cuda")], 1)
+
+
 @pytest.mark.parametrize("base,bits,group", [(wl.BASE_KIVI, 2, 1), (wl.BASE_KIVI, 3, 2), (wl.BASE_KIVI, 4, 1),
                                              (wl.BASE_MINMAX, 2, 4), (wl.BASE_MINMAX, 4, 12), (wl.BASE_AKVQ, 3, 7)])
 def test_decode_scales_over_many_binades(base, bits, group):
