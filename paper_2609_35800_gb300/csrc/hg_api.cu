@@ -742,8 +742,7 @@ hg_status decode_launch(const hg_cache* c, int32_t layer_begin, int32_t layer_co
     // fewer tokens may get an empty last chunk, which merges as nothing
     p.counts = counts_of(d, most, p.plan);
     p.total_items = fill_runs(d, {unprot, n * d.H - unprot}, &p);
-    const int total = p.total_items;
-    const hg_status st = cuda_status(launch_decode(p, total, reinterpret_cast<cudaStream_t>(stream)));
+    const hg_status st = cuda_status(launch_decode(p, reinterpret_cast<cudaStream_t>(stream)));
     if (st != HG_OK) return st;
   }
   return HG_OK;

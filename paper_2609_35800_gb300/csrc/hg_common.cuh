@@ -12,8 +12,6 @@
 
 namespace hg {
 
-__device__ __forceinline__ float bf16_to_f32(uint32_t h16) { return __uint_as_float(h16 << 16); }
-
 // Two BF16 packed in a 32-bit word -> two floats (low half first).
 __device__ __forceinline__ void bf16x2_to_f32(uint32_t w, float& lo, float& hi) {
   lo = __uint_as_float(w << 16);
@@ -118,11 +116,6 @@ __device__ __forceinline__ uint32_t code_of(float d, float scale, float r, float
   }
   rq = fminf(fmaxf(rq, 0.0f), levels);
   return (uint32_t)rq;
-}
-
-// Reconstruction fl32(fl32(code * scale) + zero).
-__device__ __forceinline__ float dequant1(uint32_t code, float scale, float zero) {
-  return __fadd_rn(__fmul_rn((float)code, scale), zero);
 }
 
 // Vector loads of global memory.  Ordinary ones: the kernels start before the

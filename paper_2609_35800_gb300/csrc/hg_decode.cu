@@ -37,8 +37,8 @@ cudaError_t launch_wait_probe(uint32_t* result, uint32_t rounds, cudaStream_t s)
   return cudaGetLastError();
 }
 
-cudaError_t launch_decode(const DecodeParams& p, int grid_x, cudaStream_t s) {
-  return p.d.meta16 ? launch_decode_m16(p, grid_x, s) : launch_decode_mb<8>(p, grid_x, s);
+cudaError_t launch_decode(const DecodeParams& p, cudaStream_t s) {
+  return p.d.meta16 ? launch_decode_m16(p, s) : launch_decode_mb<8>(p, s);
 }
 
 }  // namespace hg

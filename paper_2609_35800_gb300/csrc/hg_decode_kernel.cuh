@@ -98,19 +98,12 @@ struct NZOf {
 };
 
 struct Seg {
-  const char* k;   // BF16 key rows (K_BF16)
-  const char* v;   // BF16 value rows (V_BF16)
   int k_row0;      // arena tensor-map row of key token 0 (K_BF16)
   int v_row0;      // arena tensor-map row of value token 0 (V_BF16)
   const char* kc;  // key codes
   const char* km;  // key metadata
   const char* vc;  // value codes
   const char* vm;  // value metadata
-  // Fused append: BF16 row new_pos of this segment is stored from these
-  // input rows into the arena before its tile is loaded (new_pos < 0: none).
-  int new_pos;
-  const char* k_new;
-  const char* v_new;
 };
 
 // Mask of a code pair at bits [0, b) and [16, 16 + b).
@@ -1744,27 +1737,20 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
   // tiles are consumed (the same row layout as the split partials)
   float* parts = reinterpret_cast<float*>(smem + kStageOff);
   Seg sg;
-  sg.k = sg.v = sg.kc = sg.km = sg.vc = sg.vm = nullptr;
-  sg.new_pos = -1;
-  sg.k_new = sg.v_new = nullptr;
+  sg.kc = sg.km = sg.vc = sg.vm = nullptr;
   sg.k_row0 = sg.v_row0 = 0;
   if (!coded) {
-    sg.k = Lb + hd.kb + b * hd.kb_bs;
-    sg.v = Lb + hd.vb + b * hd.kb_bs;
     sg.k_row0 = (int)((p.lt.base[li] + hd.kb + b * hd.kb_bs) >> 8);
     sg.v_row0 = (int)((p.lt.base[li] + hd.vb + b * hd.kb_bs) >> 8);
     const int pos = hd.bf16_prefill + p.appended[li] - 1;  // the step's new token
     if (p.k_new && pos >= tb && pos < te) {
       const size_t row = (((size_t)li * d.B + b) * d.H + h) * kD;
-      sg.new_pos = pos;
-      sg.k_new = reinterpret_cast<const char*>(p.k_new + row);
-      sg.v_new = reinterpret_cast<const char*>(p.v_new + row);
       // this CTA alone owns the position in this launch: store it in the
       // arena, ordered before the TMA reads of its tile
       if (threadIdx.x < 32) {
         const int c = threadIdx.x & 15;
-        const char* src = (threadIdx.x < 16) ? sg.k_new : sg.v_new;
-        char* dst = const_cast<char*>((threadIdx.x < 16) ? sg.k : sg.v) + (size_t)pos * 256;
+        const char* src = reinterpret_cast<const char*>(((threadIdx.x < 16) ? p.k_new : p.v_new) + row);
+        char* dst = const_cast<char*>(Lb) + ((threadIdx.x < 16) ? hd.kb : hd.vb) + b * hd.kb_bs + (size_t)pos * 256;
         *reinterpret_cast<uint4*>(dst + c * 16) = ldg16(src + c * 16);
         fence_proxy_async_global();
       }
@@ -1773,7 +1759,6 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
     run_item<BITS, NT, K_BF16, V_BF16, false, MB>(smem, sg, tb, te, p, qv, G, parts);
   } else if (hd.cls == kKeysOnly) {
     __syncthreads();  // barriers initialised
-    sg.k = Lb + hd.kimg + b * hd.kimg_bs;
     sg.k_row0 = (int)((p.lt.base[li] + hd.kimg + b * hd.kimg_bs) >> 8);
     sg.vc = Lb + hd.vq + b * hd.vq_bs;
     sg.vm = Lb + hd.vqm + b * hd.vqm_bs;
@@ -1853,7 +1838,7 @@ decode_kernel(const __grid_constant__ DecodeParams p) {
 }
 
 template <int BITS, int NT, int BASE, int MB, int QC>
-cudaError_t launch_t(const DecodeParams& p, int grid_x, cudaStream_t s) {
+cudaError_t launch_t(const DecodeParams& p, cudaStream_t s) {
   // set once per device; host threads that race here both set the same
   // attributes, and the flags themselves are atomic
   static std::atomic<bool> configured[64];
@@ -1870,7 +1855,6 @@ cudaError_t launch_t(const DecodeParams& p, int grid_x, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev].store(true, std::memory_order_release);
   }
-  (void)grid_x;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)p.total_items, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -1887,33 +1871,33 @@ cudaError_t launch_t(const DecodeParams& p, int grid_x, cudaStream_t s) {
 }
 
 template <int BITS, int NT, int MB>
-cudaError_t launch_base(const DecodeParams& p, int grid_x, cudaStream_t s) {
+cudaError_t launch_base(const DecodeParams& p, cudaStream_t s) {
   switch (p.d.base) {
     case kKivi:
       if constexpr (NT == 1) {
-        if (p.d.G == 1) return launch_t<BITS, NT, kKivi, MB, 1>(p, grid_x, s);
-        if (p.d.G == 2) return launch_t<BITS, NT, kKivi, MB, 2>(p, grid_x, s);
+        if (p.d.G == 1) return launch_t<BITS, NT, kKivi, MB, 1>(p, s);
+        if (p.d.G == 2) return launch_t<BITS, NT, kKivi, MB, 2>(p, s);
         // Four CTAs per SM leave the converting path short of registers (50 to 100
         // bytes of spills).  A launch of one wave or less is better off without
         // them, if some of its CTAs have to wait (one layer, 8 KV heads: 2 rows of
         // 2,900 tokens at 4 bits 23 -> 19 us; 4 rows of 8,200 at 2 bits 41 -> 33 us);
         // more waves want the fourth CTA (10 rows of 3,400 tokens: 45 and 48 us).
-        if (p.total_items <= 4 * p.deal) return launch_t<BITS, NT, kKivi, MB, -1>(p, grid_x, s);
+        if (p.total_items <= 4 * p.deal) return launch_t<BITS, NT, kKivi, MB, -1>(p, s);
       }
-      return launch_t<BITS, NT, kKivi, MB, 0>(p, grid_x, s);
-    case kAkvq: return launch_t<BITS, NT, kAkvq, MB, 0>(p, grid_x, s);
-    default: return launch_t<BITS, NT, kMinMax, MB, 0>(p, grid_x, s);
+      return launch_t<BITS, NT, kKivi, MB, 0>(p, s);
+    case kAkvq: return launch_t<BITS, NT, kAkvq, MB, 0>(p, s);
+    default: return launch_t<BITS, NT, kMinMax, MB, 0>(p, s);
   }
 }
 
 // Every kernel shape for one metadata width (MB bytes per {scale, zero} pair).
 template <int MB>
-cudaError_t launch_decode_mb(const DecodeParams& p, int grid_x, cudaStream_t s) {
+cudaError_t launch_decode_mb(const DecodeParams& p, cudaStream_t s) {
   if (p.d.bits == 2)
-    return p.d.G <= 8 ? launch_base<2, 1, MB>(p, grid_x, s) : launch_base<2, 2, MB>(p, grid_x, s);
+    return p.d.G <= 8 ? launch_base<2, 1, MB>(p, s) : launch_base<2, 2, MB>(p, s);
   if (p.d.bits == 3)
-    return p.d.G <= 8 ? launch_base<3, 1, MB>(p, grid_x, s) : launch_base<3, 2, MB>(p, grid_x, s);
-  return p.d.G <= 8 ? launch_base<4, 1, MB>(p, grid_x, s) : launch_base<4, 2, MB>(p, grid_x, s);
+    return p.d.G <= 8 ? launch_base<3, 1, MB>(p, s) : launch_base<3, 2, MB>(p, s);
+  return p.d.G <= 8 ? launch_base<4, 1, MB>(p, s) : launch_base<4, 2, MB>(p, s);
 }
 
 }  // namespace

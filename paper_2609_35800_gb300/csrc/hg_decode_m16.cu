@@ -4,8 +4,8 @@
 
 namespace hg {
 
-cudaError_t launch_decode_m16(const DecodeParams& p, int grid_x, cudaStream_t s) {
-  return launch_decode_mb<4>(p, grid_x, s);
+cudaError_t launch_decode_m16(const DecodeParams& p, cudaStream_t s) {
+  return launch_decode_mb<4>(p, s);
 }
 
 }  // namespace hg

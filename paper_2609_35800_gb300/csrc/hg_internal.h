@@ -131,10 +131,10 @@ cudaError_t launch_append(const AppendParams& p, cudaStream_t s);
 // Zero `bytes` (a multiple of 16, 16-byte aligned) in stream order, as a
 // programmatic dependent launch (a memset between two would serialise them).
 cudaError_t launch_clear(void* words, size_t bytes, cudaStream_t s);
-cudaError_t launch_decode(const DecodeParams& p, int grid_x, cudaStream_t s);
+cudaError_t launch_decode(const DecodeParams& p, cudaStream_t s);
 cudaError_t launch_wait_probe(uint32_t* result, uint32_t rounds, cudaStream_t s);
 // The decode kernels for binary16 metadata pairs (called by launch_decode).
-cudaError_t launch_decode_m16(const DecodeParams& p, int grid_x, cudaStream_t s);
+cudaError_t launch_decode_m16(const DecodeParams& p, cudaStream_t s);
 // Most splits of one head the decode kernel's merge can take.
 int decode_max_splits(int G);
 
