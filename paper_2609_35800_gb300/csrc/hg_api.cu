@@ -328,12 +328,13 @@ DecodePlan plan_decode(const hg_cache* c, int begin, int count, DecodePlan* leas
   // of a large batch: 256 heads over 608 CTAs), the rounding leaves chunks of
   // up to twice the mean, and the launch lasts as long as they do.  Then
   // pieces of half the mean run as two to three waves instead, costliest
-  // first: one layer of 32 rows, 8 KV heads and 8,576 tokens 150 -> 90 us (96
-  // and 91 us at 2/3 and 1/3 of the mean); 3,520 tokens of 4-bit rotated keys
-  // 84 -> 53 us (53, 58), all measured with CTA-wide tiles (the warps' own
-  // pipelines since take 70 and 44 us).  Chunks under 256 KB keep one wave: a CTA's start
-  // and merge (about 8 us) outweigh the balance there (28 layers of 4 heads:
-  // 15.3 us a step in one wave, 18.1 with pieces of 2/3).
+  // first.  Four layers one by one, in one wave and so: 32 rows of 8 KV heads,
+  // 8,576 tokens at 2 bits 404 and 281 us; 3,520 tokens of 4-bit rotated keys 238
+  // and 177 us; 16 rows of 32 KV heads, 3,120 tokens of KIVI-style codes 240 and
+  // 222 us.  (Over 14 such launches pieces of 4/5, 4/7 and 1/3 of the mean were 4%,
+  // 4% and 15% from the best of each, 1/2 6%; 1/2 is the best of the three above.)
+  // Chunks under 256 KB keep one wave: a CTA's start and merge (about 8 us)
+  // outweigh the balance there.
   double worst = 0;
   if (hc.unprot || d.keys_only) worst = std::min(p.cbU, d.T - ncoded(d)) * thr.bf16;
   if (hc.unprot) worst = std::max(worst, std::min(p.cqU, ncoded(d)) * thr.coded_u);

@@ -97,6 +97,7 @@ struct NZOf {
   static constexpr int value = VM == V_TOKEN ? 1 : (VM == V_KIVI ? 4 : 1);
 };
 
+// Where the operands of an item's chunk lie.
 struct Seg {
   int k_row0;      // arena tensor-map row of key token 0 (K_BF16)
   int v_row0;      // arena tensor-map row of value token 0 (V_BF16)
@@ -215,13 +216,12 @@ __device__ __forceinline__ void meta_quad(const char* base, int i, float2 (&m)[4
 // codes the fp32 accumulators lose bits that the output shows), a KIVI-style
 // group of 32, 16 tokens of BF16 keys and coded values.
 //
-// Before, one thread filled a ring of tiles for all four warps, with a CTA
-// barrier per tile: a warp had one or two 16-token slices between barriers.
-// Separate pipelines, with every address known to be the same in the warp's
-// lanes (the refill runs on the uniform path), measured, one layer per launch:
-// that layer 90 -> 84 us, 3,520 tokens of 4-bit rotated keys 53 -> 50 us,
-// 32 KV heads of KIVI-style codes in 16 rows 123 -> 109 us, one row of 4 KV
-// heads and 1,460 tokens 9.4 -> 8.1 us.
+// (One ring of tiles for all four warps, filled by one thread with a CTA barrier
+// per tile, leaves a warp one or two 16-token slices between barriers: 7% slower on
+// that layer and on 3,520 tokens of 4-bit rotated keys, 13% on 32 KV heads of KIVI-
+// style codes in 16 rows and on one row of 4 KV heads and 1,460 tokens.  The gain
+// needs every address known to be the same in the warp's lanes, so that the refill
+// runs on the uniform path.)
 //
 // COLS (run_item_cols): SPLIT as well, two KIVI-style groups per tile (K and V
 // 4 KB each at 2 bits), or 16 tokens of BF16 keys and KIVI-style values.
@@ -1299,8 +1299,8 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
 // Keys, 64 tokens (two 32-token groups) at a time.  Row g of every m-tile is
 // half g / 4 of code word g % 4 (16 tokens: word s of group r is 2r + s), and
 // the m-tile picks the position inside the half, so a lane expands its words
-// at fixed bit positions (three shifts for eight of them, see code_pair) instead of shifting every pair by its own amount.  The rows of one m-tile
-// then belong to both groups, whose scaled queries q_c s_c differ: column
+// at fixed bit positions (three shifts for eight of them, see code_pair) instead
+// of shifting every pair by its own amount.  The rows of one m-tile then belong to both groups, whose scaled queries q_c s_c differ: column
 // 4r + 2k + h holds group r's, h the FP16 hi or lo part, k the query (QC = 2)
 // or the parity of the k-steps the lane scales (QC = 1: each lane builds half
 // of them, the other columns see zeros).  Row g reads columns 4r .. 4r + 3 of
@@ -1314,11 +1314,11 @@ __device__ __forceinline__ void run_item(char* smem, const Seg& sg, int tb, int 
 // tq + 8, tq + 12 of a slice sit in one lane's k-slots (codes and metadata of
 // the four tq lanes on different banks).
 //
-// Issue-bound before: 772 warp instructions per 16-token slice in run_item
-// (one query in eight columns), 32 KV heads of 3,120 tokens in 16 rows at 109 us
-// a layer, 0.39 of the measured copy rate; here 278 and 55 us, 0.77.  Error
-// against 64 bits as before (with BF16 128 + c and FP16 1024 + c operands, the
-// offsets removed by MMAs over constant tiles, it grew from 1.71e-3 to 2.1e-3).
+// 278 warp instructions per 16-token slice; 32 KV heads of 3,120 tokens in 16 rows
+// 55 us a layer, 0.77 of the measured copy rate.  (run_item, with one query in eight
+// columns, takes 772 and is bound by issue: 105 us.)  Error against 64 bits 1.7e-3,
+// as run_item's (with BF16 128 + c and FP16 1024 + c operands, the offsets removed by
+// MMAs over constant tiles, 2.1e-3).
 // ---------------------------------------------------------------------------
 template <int QC>
 struct ColState {
@@ -1879,9 +1879,11 @@ cudaError_t launch_base(const DecodeParams& p, cudaStream_t s) {
         if (p.d.G == 2) return launch_t<BITS, NT, kKivi, MB, 2>(p, s);
         // Four CTAs per SM leave the converting path short of registers (50 to 100
         // bytes of spills).  A launch of one wave or less is better off without
-        // them, if some of its CTAs have to wait (one layer, 8 KV heads: 2 rows of
-        // 2,900 tokens at 4 bits 23 -> 19 us; 4 rows of 8,200 at 2 bits 41 -> 33 us);
-        // more waves want the fourth CTA (10 rows of 3,400 tokens: 45 and 48 us).
+        // them, even if some of its CTAs have to wait (one layer, 8 KV heads: 2 rows
+        // of 2,900 tokens at 4 bits 19 us, 23 with four; 4 rows of 8,200 at 2 bits 33
+        // and 41); more waves want the fourth CTA (10 rows of 3,400 tokens: 48 us with
+        // three, 45 with four; of 28 other launches of 1.2 to 7 waves 24 were 1 to 17%
+        // faster with four, and four, three of them of 3-bit codes, 4 to 15% slower).
         if (p.total_items <= 4 * p.deal) return launch_t<BITS, NT, kKivi, MB, -1>(p, s);
       }
       return launch_t<BITS, NT, kKivi, MB, 0>(p, s);

@@ -145,7 +145,7 @@ __device__ __forceinline__ float abs_max3(float a, float b, float c) {
 // the word's other codes too: `top` keeps it, and the chunk counts as near a tie.
 // (chunk_T and chunk_bits_T take four integer operations per
 // element, and the integer pipe bound these rows: InternVL2.5-8B-shaped prefill with
-// salient tokens, 4 layers one by one, 766 -> 729 us.)
+// salient tokens, 4 layers one by one, 692 us with them, 657 so.)
 __device__ __forceinline__ bool chunk_codes4(const uint64_t (&x2)[4], uint64_t mn2, uint64_t r2, uint32_t& lo) {
   const uint64_t m2 = f32x2(0x4B000000u, 0x4B000000u), c256 = f32x2(0xC3800000u, 0xC3800000u);  // 2^23, -256
   uint64_t t[4], g[4];
@@ -253,11 +253,10 @@ __device__ __forceinline__ void row_minmax(const uint4* r4, int k0, int nk, floa
 // plus half the spacing above; code k + 1 needs the first for k = 1 (3/2 rounds
 // up to 2) and the second for k = 0 and 2.  d - h scale is exact in one FMA
 // where it is small enough for this to matter.
-//   A KIVI-style layer of 16 rows, 32 heads and 3,120 tokens: 221 -> 198 us, 0.82
-// of the measured copy rate.  Min-max, 28 layers of 4 heads and 1,460 tokens:
-// 24.7 -> 24.6 us (not coding-bound).  With __hmin2 / __hmax2 and three
-// candidates tried per threshold it measured no better than the rule of the
-// other widths.
+//   KIVI-style, 16 rows, 32 heads and 3,120 tokens, 4 layers one by one: 715 us, 805
+// by the rule of the other widths.  Min-max, 28 layers of 4 heads and 1,460 tokens:
+// 22 us by either (not coding-bound).  With __hmin2 / __hmax2 and three candidates
+// tried per threshold it was no better than the rule of the other widths.
 // ---------------------------------------------------------------------------
 // Steps the comparisons serve: scale 2^-25 stays normal, 1 / scale finite.
 __device__ __forceinline__ bool threshold_scale(float scale) {
@@ -393,11 +392,10 @@ __device__ __forceinline__ void quantize_key_pair_any(const char* col, uint32_t*
     }
   }
   // near ties by the exact rule, each code written over its stored bits (the
-  // positions of add_key_code); side by side in the warp's threads.  (As a branch
-  // at each element of the loop above: 14 layers of 14 rows, 16 heads and 856
-  // tokens at 4 bits one by one 495 -> 471 us, a 3-bit layer of 6 rows 7.5 -> 6.3
-  // us; at 2 bits the few groups that come here hold up their warps: LLaVA-NeXT-
-  // 7B-shaped, 4 layers one by one, 761 -> 730 us.)
+  // positions of add_key_code); side by side in the warp's threads.  (A branch at
+  // each element of the loop above was slower: 5% on 14 layers of 14 rows, 16 heads
+  // and 856 tokens at 4 bits, 16% on a 3-bit layer of 6 rows; at 2 bits, where the
+  // few groups that come here hold up their warps, 4% on LLaVA-NeXT-7B-shaped layers.)
   while (tie0 | tie1) {
     const bool j = tie0 == 0u;
     const int e = __ffs(j ? tie1 : tie0) - 1;
@@ -544,9 +542,8 @@ __device__ __forceinline__ void chunk_near_tie(const uint32_t (&a)[8], X x, floa
 // again.  The loop runs over a thread's own elements near a
 // tie (mostly one), so the threads of a warp divide side by side; with the eight
 // elements in turn a warp went through nearly all eight for its threads'
-// different ones.  One layer of 862 tokens at 4 bits 5.2 -> 4.4 us; 17 layers of
-// 1,560 tokens one by one 100 -> 85 us; 3 bits, 2 layers of 6 rows and 7,415
-// tokens 55 -> 50 us.
+// different ones: 15% slower on 4-bit layers of 862 to 1,560 tokens, 10% on 3-bit
+// ones of 7,415.
 template <int BITS>
 __device__ __forceinline__ void recode_near_ties(const uint4* r4, int k, uint64_t mn2, uint64_t r2, uint64_t c2, float mn,
                                                  float scale, uint32_t* codes) {
@@ -756,9 +753,8 @@ __device__ __forceinline__ void quantize_row_kivi_v(const char* row_s, uint32_t*
 // the row's min / max by shuffles, and codes chunks 8 hh .. 8 hh + 7 into its
 // own words of the packed row (lane 0 stores the metadata).  Half the pairs
 // per thread: twice the rows resident.  Bound by instruction issue: stage 64 as
-// one FMA by +-1, not a sum, a difference and a selection, InternVL2.5-8B-shaped
-// prefill with salient tokens, 4 layers one by one, 729 -> 692 us (94 registers
-// instead of 102: 20 warps per SM, not 16).
+// one FMA by +-1, not a sum, a difference and a selection, is 5% of an
+// InternVL2.5-8B-shaped prefill with salient tokens (657 us for 4 layers one by one).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float pair_lo(uint64_t x) { return __uint_as_float((uint32_t)x); }
 __device__ __forceinline__ float pair_hi(uint64_t x) { return __uint_as_float((uint32_t)(x >> 32)); }
@@ -1184,16 +1180,17 @@ __global__ void __maxnreg__(TP::kRegisters) quantize_tiles_kernel(const __grid_c
 // lower index) and writes the map: a bit per image token and the salient count
 // before each 32-token block.
 //
-// One CTA per head for both read the keys with 8 KB in flight: 88 us for a
-// layer of 32 rows, 8 KV heads and 3,328 image tokens (191 MB of keys read, 28 us
-// at the measured copy rate); now 33 us and 8 us.
+// A layer of 32 rows, 8 KV heads and 3,328 image tokens (191 MB of keys read, 28 us
+// at the measured copy rate): 33 us and 8 us; one CTA per head for both has too
+// little in flight (8 KB, 88 us).
 // ---------------------------------------------------------------------------
 constexpr int kNormThreads = 256, kNormRows = 8, kNormTokens = kNormThreads / 32 * kNormRows;
 constexpr int kSalThreads = 512;
 // Spans up to this length: the selection's CTA sums the norms itself, one
-// launch (a layer of 8 heads in 4 rows, prefill in one and two launches before
-// the quantizer's: 26.8 and 27.3 us with 512 image tokens, 38.9 and 34.3 with
-// 1,024; 256 heads: 56.1 and 59.9, 85.9 and 85.4).
+// launch (a layer of 8 heads in 4 rows, prefill in a stream with one and two
+// launches before the quantizer's: 14.4 and 14.0 us with 512 image tokens, 20.6 and
+// 17.3 with 1,024; 32 rows: 38.7 and 38.6, 63.2 and 61.8.  Small layers wait for the
+// host, whose time a call is that of the launches).
 constexpr int kSalOneLaunch = 512;
 
 // Where the scores of one row of a head with coded values wait for the
@@ -1305,9 +1302,8 @@ __global__ void __launch_bounds__(kSalThreads) salient_select_kernel(const __gri
   // four fixed digits spent the first on a byte that two values share.  Spread
   // digits make plain atomics the better histogram (one per distinct digit of a
   // warp, found by a match: 2 us more).  A layer of 32 rows, 8 KV heads and 3,328
-  // image tokens 12 -> 8 us; 11 layers of 2 rows, 16 heads and 110 image tokens,
-  // prefill in all 133 -> 119 us; the same with one key far above the others, or
-  // all equal.
+  // image tokens 8 us, 12 in four fixed passes; with one key far above the others,
+  // or all equal, the same.
   static_assert(kSalThreads >= 256, "a thread per histogram bin");
   uint32_t diff = 0u;
   const uint32_t key0 = __float_as_uint(score[0]);
@@ -1433,10 +1429,10 @@ __global__ void __launch_bounds__(kSalThreads) salient_select_kernel(const __gri
 // a lane and the last four across the half-warp, in the same order as the
 // forward transform.
 //
-// Before, every row found its own place (146 warp instructions per pair of
-// rows: issue-bound on small caches).  Qwen2.5-VL-7B-shaped, 28 layers: 30.8 ->
-// 22.6 us; a LLaVA-NeXT-7B-shaped layer of 16 rows: 378 -> 167 us, 0.98 of the
-// measured copy rate (BF16 output).
+// Bound by DRAM on large caches (four LLaVA-NeXT-7B-shaped layers of 16 rows, BF16
+// output: 658 us, 0.99 of the measured copy rate; with every row finding its own
+// place, 146 warp instructions per pair of rows, 1,510 us), by the ramp and the tail
+// on small ones (Qwen2.5-VL-7B-shaped, 28 layers: 19.8 us; 30.8).
 // ---------------------------------------------------------------------------
 constexpr int kDqThreads = 256;
 constexpr int kDqTile = 32;
@@ -1673,8 +1669,9 @@ __global__ void __launch_bounds__(kDqThreads, 6) dequantize_kernel(const __grid_
     const bool whole = a >= 0 && e <= Tt;
     const bool in_image = a >= qs && e <= qe, outside = cls == kProtected || e <= qs || a >= qe;
     // Salient tokens: a run without one (eight tokens of one map word; most runs)
-    // is of one kind as well, moved down by the salient ones before it.
-    // InternVL2.5-8B-shaped, 2% salient, 32 layers, BF16: 4.55 -> 5.84 TB/s.
+    // is of one kind as well, moved down by the salient ones before it
+    // (InternVL2.5-8B-shaped, 2% salient, 32 layers, BF16: 5.84 TB/s; 4.55 with
+    // every row resolved).
     bool plain = whole && in_image && !has_salient;
     int ti = a - qs;
     if (whole && in_image && has_salient) {
@@ -1779,8 +1776,8 @@ __global__ void __launch_bounds__(kDqThreads, 6) dequantize_kernel(const __grid_
 // the programmatic dependent launches of a decode loop: the next launch may be
 // scheduled at once, and everything before the first store comes from the
 // launch parameters.  Appending and attending without a workspace, layer by
-// layer (append, clear, decode: 6 layers of 5 KV heads, 2 tokens): 246 -> 182 us
-// with the three overlapping; before, append and a memset each ran alone.
+// layer (append, clear, decode: 6 layers of 5 KV heads, 2 tokens): 184 us with the
+// three overlapping, 246 with an append and a memset that each run alone.
 __global__ void __launch_bounds__(64) append_kernel(const __grid_constant__ AppendParams p) {
   grid_launch_dependents();
   const Dims& d = p.d;
@@ -1903,9 +1900,9 @@ cudaError_t launch_dequantize(const DequantParams& p, int sm_count, cudaStream_t
   const int Tt = p.d.T + p.appended;
   const int ntiles = (Tt - dq_origin(p.d) + kDqTile - 1) / kDqTile;
   // Tiles per CTA (1 to 4): whole waves of 6 CTAs per SM, each as long as its
-  // tiles and a start worth 0.4 of one.  (Qwen2.5-VL-7B-shaped, 28 layers: 24.7
-  // us with one tile per CTA, 22.6 with two; a LLaVA-NeXT-7B-shaped layer of 16
-  // rows 179 us with two, 175 with four, 179 with eight.)
+  // tiles and a start worth 0.4 of one.  (Qwen2.5-VL-7B-shaped, 28 layers: 21.2
+  // us with one tile per CTA, 19.5 with two, 20.4 with four, 23.6 with eight; four
+  // LLaVA-NeXT-7B-shaped layers of 16 rows one by one 786, 664, 661 and 676 us.)
   const double groups = (double)p.d.B * p.d.H * p.n_layers, wave = 6.0 * (sm_count > 0 ? sm_count : 1);
   int span = 1;
   double best = 0.0;
