@@ -994,9 +994,9 @@ __device__ __forceinline__ bool copy_tile_whole(const QuantizeParams& p, int li,
 template <int BITS, bool M16, int BASE>
 struct TokenTiles {
   static constexpr bool kKeysFirst = BASE == kAkvq;
-  // 96: 21 warps per SM where the rotated rows and the value rows of one kernel came
-  // to 99 (InternVL2.5-8B-shaped prefill with salient tokens, 4 layers one by one, 692 ->
-  // 659 us; at most two registers spilled); 80: what the rows take anyway.
+  // 96: 20 warps per SM, where the rotated rows and the value rows of one kernel come
+  // to 99 and 16 (InternVL2.5-8B-shaped prefill with salient tokens, 4 layers one by
+  // one, 657 and 692 us; at most two registers spilled); 80: what the rows take anyway.
   static constexpr int kRegisters = BASE == kAkvq ? 96 : 80;
   static __device__ __forceinline__ TileSpan span(const QuantizeParams& p, int tx) {
     TileSpan sp;
@@ -1138,7 +1138,7 @@ struct KiviTiles {
 // or (kKeysFirst) the highest of z, all keys of the launch before all values,
 // so that the warps of an SM share one of two unlike code paths at a time.  A
 // warp stages its 32 rows, waits for its own copies and codes them; no CTA-wide
-// barrier, so the warps of an SM (21 to 23 resident) run out of step and one
+// barrier, so the warps of an SM (20 to 23 resident) run out of step and one
 // warp's loads overlap another's coding.
 // A programmatic dependent launch: its CTAs may come to the SMs while the
 // kernels before it still run, and wait for them before their first load (no

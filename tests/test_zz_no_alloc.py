@@ -5,12 +5,13 @@ memory (plugin interfaces that pass only inputs and outputs, a device pool
 owned by another framework, loops that cannot take cudaMalloc's implicit
 synchronisation): it runs decode attention with the library's own static
 scratch array instead of a caller-provided workspace.  Both entry points run
-the same kernel with the same work plan and a fixed merge order, so their
-outputs must be bit-identical -- on consecutive calls (each sees the scratch
+the same kernel with a fixed merge order and, where the finer work plan fits the
+scratch as in every case here, the same work plan, so their outputs must be
+bit-identical -- on consecutive calls (each sees the scratch
 the previous one left), after a call over a different layer range (other
 counters, other partial slots), on a non-default stream, and at a full
-benchmark shape.  A launch whose workspace exceeds the 32 MiB scratch is
-refused before anything is enqueued.  The file is named to be collected last.
+benchmark shape.  A launch that cannot run in the 32 MiB scratch is refused
+before anything is enqueued.  The file is named to be collected last.
 """
 import numpy as np
 import pytest
@@ -94,8 +95,8 @@ def test_noalloc_full_shape_one_layer_side_stream():
 
 
 def test_noalloc_refuses_a_workspace_beyond_the_scratch():
-    """The InternVL2.5-8B-shaped cache over all 32 layers needs just over 32 MiB
-    of workspace; the call is refused and `out` is left as it was."""
+    """The InternVL2.5-8B-shaped cache over all 32 layers needs more than 32 MiB in
+    the coarsest plan too; the call is refused and `out` is left as it was."""
     w = wl.WORKLOADS["internvl25_8b"]
     runner = CacheRunner(w, ws_layers=1)
     need = hg.hg_decode_workspace_size(runner.cache, w.layers)
