@@ -143,7 +143,7 @@ def attention_reference(runner, o, q_bits, appended_k, appended_v, sigma):
 def assert_close(got_bf16_bits, ref, where=""):
     g = f32_from_bits(got_bf16_bits).astype(np.float64)
     err = np.abs(g - ref)
-    bad = err > ATOL + RTOL * np.abs(ref)
+    bad = ~(err <= ATOL + RTOL * np.abs(ref))  # a NaN is outside
     if bad.any():
         i = np.argwhere(bad)[0]
         raise AssertionError("%s: %d / %d outside tolerance; first at %s got %r ref %r "
