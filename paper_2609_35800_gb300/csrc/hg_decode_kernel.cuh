@@ -1367,6 +1367,11 @@ __device__ __forceinline__ void cols_softmax(ColState<QC>& ws, const float (&x)[
   __syncwarp();
 }
 
+// The query rows of run_item_cols are staged with their largest element at 1 at
+// most, so that no sum over them overflows where the scores would not; times a
+// channel scale over kb it is brought to 2^kColsTop, near the top of FP16's range.
+constexpr int kColsTop = 15;
+
 // Raw scores of a 64-token tile of KIVI-style keys: kst its codes and metadata,
 // x[q][i] the scores of tokens 2 lane + i, in units of the staged query rows
 // and without the softmax scale.
@@ -1391,7 +1396,7 @@ __device__ __forceinline__ void cols_scores(const char* kst, const char* kmeta, 
     if (!two_groups && lane >= 16) top = 0.f;  // stale metadata of an absent second group
     if (__any_sync(kFull, top > kb)) kb = pow2_ceil(fminf(warp_max(top), kScaleTop));
   }
-  const float inv = pow2_inv(kb);
+  const float inv = pow2_inv(kb) * (float)(1 << kColsTop);
 #pragma unroll
   for (int i = 0; i < NB; ++i) {
     const int c0 = 16 * (QC == 1 ? 2 * i + sel : i) + 4 * tq;
@@ -1457,9 +1462,9 @@ __device__ __forceinline__ void cols_scores(const char* kst, const char* kmeta, 
     float v[8];
 #pragma unroll
     for (int mt = 0; mt < 4; ++mt) {
-      const float unit = kb * kCodeUnit;
-      v[mt] = (acc[mt][0] + acc[mt][1]) * (code_unit<BITS>(mt) * unit);
-      v[4 + mt] = (acc[mt][2] + acc[mt][3]) * (code_unit<BITS>(BITS == 4 ? mt : mt + 4) * unit);
+      constexpr float unit = kCodeUnit / (float)(1 << kColsTop);
+      v[mt] = (acc[mt][0] + acc[mt][1]) * (code_unit<BITS>(mt) * unit) * kb;
+      v[4 + mt] = (acc[mt][2] + acc[mt][3]) * (code_unit<BITS>(BITS == 4 ? mt : mt + 4) * unit) * kb;
     }
     float4* dst = reinterpret_cast<float4*>(ps + 64 * (tq & 1) + 16 * (g & 3) + 8 * (g >> 2));
     dst[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -1496,7 +1501,7 @@ __device__ __forceinline__ void run_item_cols(char* smem, const Seg& sg, int tb,
   WarpPipe<BITS, 1, KM, V_KIVI, MB, true, KM == K_KIVI ? kKiviGroup : 16> pipe(smem, warp, sg, p, tb, te);
 
   float* qn = reinterpret_cast<float*>(smem + SmemLayout<1>::qn);
-  stage_queries<1, KM == K_BF16 ? -1 : 15>(q_s, qn, qv, tid);
+  stage_queries<1, KM == K_BF16 ? -1 : 0>(q_s, qn, qv, tid);
   __syncthreads();
   float unit[QC];  // of the scores: the staged rows' and the softmax scale
 #pragma unroll

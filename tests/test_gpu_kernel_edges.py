@@ -193,6 +193,27 @@ def test_decode_scales_over_many_binades(base, bits, group):
         _decode_against_oracle(w, [(k, v)], 1, q_scale, float(v.abs().max()))
 
 
+@pytest.mark.parametrize("base,bits,group", [(wl.BASE_KIVI, 2, 1), (wl.BASE_KIVI, 3, 2), (wl.BASE_KIVI, 4, 1),
+                                             (wl.BASE_KIVI, 2, 4), (wl.BASE_MINMAX, 2, 4), (wl.BASE_MINMAX, 3, 12),
+                                             (wl.BASE_AKVQ, 4, 7)])
+@pytest.mark.parametrize("power", [-112, -80, 80, 112])
+def test_keys_near_the_ends_of_the_range(power, base, bits, group):
+    """Keys of 2^power, with a softmax scale that brings the scores back to order one: no intermediate of the
+    scores may overflow, or lose bits as a subnormal, where the scores themselves do not."""
+    w = wl.custom("range", 1, 1, 2 * group, 2, 8, 200, 40, base, bits, 0, decode_steps=1, seed=25, protected=[])
+    k, v = wl.layer_kv(w, 0, "cuda")
+    k = (k.float() * 2.0 ** power).bfloat16()
+    sigma = SIGMA * 2.0 ** -power
+    runner = CacheRunner(w)
+    hg.hg_quantize_kv(runner.cache, 0, [k], [v])
+    q = wl.step_query(w, 0, "cuda")
+    out = torch.empty_like(q)
+    hg.hg_decode_attention(runner.cache, 0, 1, q, out, sigma, runner.ws, runner.ws_bytes)
+    o = oracle_layer(runner, 0, bits16(k), bits16(v))
+    ref = oracle.attention_layer(bits16(q[0]), o["k_att"], o["v_deq"].astype(np.float64), sigma)
+    assert_close(bits16(out[0]), ref, "2^%d" % power)
+
+
 @pytest.mark.parametrize("meta_bits", [64, 32])
 @pytest.mark.parametrize("base,bits,salient", [(wl.BASE_MINMAX, 3, 0), (wl.BASE_KIVI, 2, 0), (wl.BASE_KIVI, 3, 0),
                                                (wl.BASE_KIVI, 4, 0), (wl.BASE_AKVQ, 2, 0), (wl.BASE_AKVQ, 4, 30)])
